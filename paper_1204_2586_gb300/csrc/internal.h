@@ -341,6 +341,11 @@ void build_sell_natural(DevPool &pool, const DCSR &A, DSell &S, bool want32, cud
 void build_sell_split(DevPool &pool, const DSplit &sp, int64_t n, bool upper, DSell &S, bool want32,
                       cudaStream_t s);
 
+// colour.cu: stable counting sort of the rows 0..n-1 by key (0..nkeys-1): perm[place] = row,
+// off[key] = first place of a key
+void key_sort(int64_t n, const int32_t *key, int64_t nkeys, int32_t *perm, std::vector<int64_t> &off,
+              cudaStream_t s);
+
 // small device utilities (util.cu)
 void to32(const double *x, float *y, int64_t n, cudaStream_t s);
 void exclusive_scan(int64_t *d, int64_t n, cudaStream_t s);  // in place, d[n] = total

@@ -1,7 +1,4 @@
 // setup.cu -- device-side construction of the auxiliary-space preconditioner:
-//   * Jones-Plassmann colouring of a matrix graph and the colour split used by the
-//     multicolour Gauss-Seidel smoothers (the paper's hybrid GS of Sec. 6.1 replaced by
-//     a GS that parallelises over colours);
 //   * the P1 algebraic multigrid hierarchy on A_H (Step 1 of Algorithm 2.1 solved by one
 //     AMG cycle, Remark 2.1): strength of connection (Sec. 6.2), PMIS coarsening and
 //     extended+i interpolation (cited in Sec. 1 and 6.1), Galerkin products P^T A P
@@ -27,119 +24,6 @@ unsigned blocks_for(int64_t n, int per) {
     return (unsigned)std::max<int64_t>(1, b);
 }
 
-
-// ---------------------------------------------------------------------------------
-// Jones-Plassmann colouring: priority (hash, -index); each round the local maxima among
-// uncoloured vertices take the smallest colour unused by already coloured neighbours.
-// ---------------------------------------------------------------------------------
-__global__ void k_jp_pick(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                          uint64_t stream, const int32_t *__restrict__ colour, uint8_t *__restrict__ pick) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (colour[i] >= 0) {
-        pick[i] = 0;
-        return;
-    }
-    // largest-degree-first priority (degree, hash, -index); the degree counts the
-    // off-diagonal entries of the row (rows are sorted, so the diagonal appears once)
-    const uint64_t hi = splitmix64(stream, (uint64_t)i);
-    const int64_t lo_i = ptr[i], hi_i = ptr[i + 1];
-    int64_t di = hi_i - lo_i;
-    for (int64_t e = lo_i; e < hi_i; ++e) di -= (col[e] == i);
-    uint8_t best = 1;
-    for (int64_t e = lo_i; e < hi_i; ++e) {
-        int32_t j = col[e];
-        if (j == i || colour[j] >= 0) continue;
-        int64_t dj = ptr[j + 1] - ptr[j];
-        for (int64_t f = ptr[j]; f < ptr[j + 1]; ++f) dj -= (col[f] == j);
-        bool i_wins;
-        if (di != dj) i_wins = di > dj;
-        else {
-            uint64_t hj = splitmix64(stream, (uint64_t)j);
-            i_wins = (hi != hj) ? (hi > hj) : (i < j);
-        }
-        if (!i_wins) {
-            best = 0;
-            break;
-        }
-    }
-    pick[i] = best;
-}
-
-__global__ void k_jp_assign(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                            int32_t *__restrict__ colour, const uint8_t *__restrict__ pick,
-                            unsigned long long *__restrict__ ncoloured, int *__restrict__ maxcol) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || !pick[i]) return;
-    int base = 0, c = -1;
-    while (c < 0) {
-        unsigned long long used = 0ull;
-        for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-            int32_t j = col[e];
-            if (j == i || pick[j]) continue;
-            int cj = colour[j] - base;
-            if (cj >= 0 && cj < 64) used |= 1ull << cj;
-        }
-        if (~used != 0ull) c = base + __ffsll((long long)~used) - 1;
-        else base += 64;
-    }
-    colour[i] = c;
-    atomicAdd(ncoloured, 1ull);
-    atomicMax(maxcol, c + 1);
-}
-
-// ---------------------------------------------------------------------------------
-// Colour split
-// ---------------------------------------------------------------------------------
-__global__ void k_split_count(int64_t n, const int32_t *__restrict__ perm, const int64_t *__restrict__ ptr,
-                              const int32_t *__restrict__ col, const int32_t *__restrict__ colour,
-                              int64_t *__restrict__ lcnt, int64_t *__restrict__ ucnt) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    int32_t i = perm[p];
-    int ci = colour[i];
-    int64_t l = 0, u = 0;
-    for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-        int32_t j = col[e];
-        if (j == i) continue;
-        if (colour[j] < ci) ++l;
-        else ++u;  // a proper colouring leaves no equal colours off the diagonal
-    }
-    lcnt[p] = l;
-    ucnt[p] = u;
-}
-
-__global__ void k_split_fill(int64_t n, const int32_t *__restrict__ perm, const int64_t *__restrict__ ptr,
-                             const int32_t *__restrict__ col, const double *__restrict__ val,
-                             const int32_t *__restrict__ colour, const int64_t *__restrict__ lptr,
-                             const int64_t *__restrict__ uptr, int32_t *__restrict__ lcol,
-                             double *__restrict__ lval, int32_t *__restrict__ ucol, double *__restrict__ uval,
-                             double *__restrict__ diag, double *__restrict__ dinv, int *__restrict__ bad) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    int32_t i = perm[p];
-    int ci = colour[i];
-    int64_t lo = lptr[p], uo = uptr[p];
-    double d = 0.0;
-    for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-        int32_t j = col[e];
-        if (j == i) {
-            d = val[e];
-            continue;
-        }
-        if (colour[j] == ci) atomicExch(bad, 2);
-        if (colour[j] < ci) {
-            lcol[lo] = j;
-            lval[lo++] = val[e];
-        } else {
-            ucol[uo] = j;
-            uval[uo++] = val[e];
-        }
-    }
-    if (d == 0.0) atomicExch(bad, 1);
-    diag[p] = d;
-    dinv[p] = d != 0.0 ? 1.0 / d : 0.0;
-}
 
 __global__ void k_l1norm(int64_t n, const int64_t *__restrict__ ptr, const double *__restrict__ val,
                          double *__restrict__ l1) {
@@ -242,22 +126,73 @@ __global__ void k_extpi_ub(int64_t n, const int64_t *__restrict__ ptr, const int
     ub[i] = s;
 }
 
-__device__ void sort_unique_i32(int32_t *a, int64_t &m) {
-    // insertion sort (rows are short), then drop duplicates
-    for (int64_t x = 1; x < m; ++x) {
-        int32_t v = a[x];
-        int64_t y = x - 1;
-        while (y >= 0 && a[y] > v) {
-            a[y + 1] = a[y];
-            --y;
-        }
-        a[y + 1] = v;
+// ---------------------------------------------------------------------------------
+// Sorted set of column indices, one block of NT threads per row: candidates go into an
+// open-addressing table of CAP slots in shared memory (at most half full), the distinct
+// ones are then gathered and sorted there (bitonic) and written out in ascending order.
+// A row with more distinct columns than that leaves cnt[row] = -1 and is taken by the
+// next larger table, at last by a heap sort in global memory (union_rows). One thread
+// per row with a heap sort of all candidates took 71 ms of a 312 ms setup at P3 24^3
+// (few threads, each with long chains of dependent global accesses); the table form
+// takes 0.35 ms.
+// ---------------------------------------------------------------------------------
+template <int NT, int CAP>
+struct ColSet {
+    static constexpr int kMost = CAP / 2;  // the other half leaves room for NT late inserts
+    static_assert(CAP / 2 >= NT, "table too small for the block");
+    int32_t *tab;   // [CAP]
+    int32_t *list;  // [CAP]
+    int *num;       // distinct entries; > kMost: overflow
+
+    __device__ void clear() {
+        for (int q = threadIdx.x; q < CAP; q += NT) tab[q] = -1;
+        if (threadIdx.x == 0) *num = 0;
+        __syncthreads();
     }
-    int64_t u = 0;
-    for (int64_t x = 0; x < m; ++x)
-        if (x == 0 || a[x] != a[x - 1]) a[u++] = a[x];
-    m = u;
-}
+    __device__ bool full() const { return *(volatile int *)num > kMost; }
+    __device__ void insert(int32_t v) {
+        if (full()) return;  // at most NT - 1 inserts are under way past this check
+        unsigned h = ((unsigned)v * 2654435761u) & (CAP - 1);
+        for (;;) {
+            const int32_t old = atomicCAS(&tab[h], -1, v);
+            if (old == v) return;
+            if (old == -1) {
+                atomicAdd(num, 1);
+                return;
+            }
+            h = (h + 1) & (CAP - 1);
+        }
+    }
+    // sorts the set into out[0..m); returns m, or -1 after an overflow (block-uniform)
+    __device__ int sorted(int32_t *out) {
+        __syncthreads();
+        const int m = *num;
+        if (m > kMost) return -1;
+        int p2 = 1;
+        while (p2 < m) p2 <<= 1;
+        __syncthreads();
+        if (threadIdx.x == 0) *num = 0;
+        for (int q = threadIdx.x; q < p2; q += NT) list[q] = INT32_MAX;
+        __syncthreads();
+        for (int q = threadIdx.x; q < CAP; q += NT)
+            if (tab[q] != -1) list[atomicAdd(num, 1)] = tab[q];
+        __syncthreads();
+        for (int k = 2; k <= p2; k <<= 1)
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int t = threadIdx.x; t < p2 / 2; t += NT) {
+                    const int x = ((t & ~(j - 1)) << 1) | (t & (j - 1)), y = x | j;
+                    const int32_t u = list[x], v = list[y];
+                    if ((u > v) == ((x & k) == 0)) {
+                        list[x] = v;
+                        list[y] = u;
+                    }
+                }
+                __syncthreads();
+            }
+        for (int q = threadIdx.x; q < m; q += NT) out[q] = list[q];
+        return m;
+    }
+};
 
 // 1 when k has a strong C point that is also a strong C point of i
 __device__ bool shares_strong_c(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
@@ -271,162 +206,76 @@ __device__ bool shares_strong_c(const int64_t *__restrict__ ptr, const int32_t *
     return false;
 }
 
-__global__ void k_extpi_hat(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                            const uint8_t *__restrict__ strong, const int8_t *__restrict__ cf,
-                            const int64_t *__restrict__ ub_off, int32_t *__restrict__ scratch,
-                            int64_t *__restrict__ cnt, int cc) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (cf[i] == 1) {
-        cnt[i] = 1;
-        return;
-    }
-    int32_t *h = scratch + ub_off[i];
-    int64_t m = 0;
-    for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-        if (!strong[e]) continue;
-        int32_t k = col[e];
-        if (cf[k] == 1) h[m++] = k;
-        else if (!cc || !shares_strong_c(ptr, col, strong, cf, i, k))
-            for (int64_t f = ptr[k]; f < ptr[k + 1]; ++f)
-                if (strong[f] && cf[col[f]] == 1) h[m++] = col[f];
-    }
-    sort_unique_i32(h, m);
-    cnt[i] = m;
-}
-
-__device__ __forceinline__ double abar(double akl, double akk) {
-    if (akk > 0.0) return akl < 0.0 ? akl : 0.0;
-    if (akk < 0.0) return akl > 0.0 ? akl : 0.0;
-    return akl;
-}
-
-__device__ __forceinline__ int64_t find_sorted(const int32_t *h, int64_t m, int32_t v) {
-    int64_t lo = 0, hi = m;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        if (h[mid] < v) lo = mid + 1;
-        else hi = mid;
-    }
-    return (lo < m && h[lo] == v) ? lo : -1;
-}
-
-__global__ void k_extpi_fill(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                             const double *__restrict__ val, const uint8_t *__restrict__ strong,
-                             const int8_t *__restrict__ cf, const int64_t *__restrict__ cidx,
-                             const int64_t *__restrict__ ub_off, const int32_t *__restrict__ scratch,
-                             const int64_t *__restrict__ pptr, int32_t *__restrict__ pcol,
-                             double *__restrict__ pval) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t o = pptr[i];
-    if (cf[i] == 1) {
-        pcol[o] = (int32_t)cidx[i];
-        pval[o] = 1.0;
-        return;
-    }
-    const int64_t m = pptr[i + 1] - o;
-    if (m == 0) return;
-    const int32_t *h = scratch + ub_off[i];
-    double *w = pval + o;
-    for (int64_t q = 0; q < m; ++q) {
-        w[q] = 0.0;
-        pcol[o + q] = (int32_t)cidx[h[q]];
-    }
-    double aii = 0.0;
-    for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e)
-        if (col[e] == i) aii = val[e];
-    double diag = aii;
-    for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-        int32_t j = col[e];
-        if (j == i) continue;
-        int64_t q = find_sorted(h, m, j);
-        if (q >= 0) w[q] = val[e];
-        else if (!strong[e]) diag = __dadd_rn(diag, val[e]);
-    }
-    for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-        if (!strong[e]) continue;
-        int32_t k = col[e];
-        if (cf[k] != -1) continue;
-        const double aik = val[e];
-        double akk = 0.0;
-        for (int64_t f = ptr[k]; f < ptr[k + 1]; ++f)
-            if (col[f] == k) akk = val[f];
-        double d = 0.0;
-        for (int64_t f = ptr[k]; f < ptr[k + 1]; ++f) {
-            int32_t l = col[f];
-            if (l == k) continue;
-            if (l == i || find_sorted(h, m, l) >= 0) d = __dadd_rn(d, abar(val[f], akk));
-        }
-        if (d == 0.0) {
-            diag = __dadd_rn(diag, aik);
-            continue;
-        }
-        for (int64_t f = ptr[k]; f < ptr[k + 1]; ++f) {
-            int32_t l = col[f];
-            if (l == k) continue;
-            double t = __ddiv_rn(__dmul_rn(aik, abar(val[f], akk)), d);
-            if (l == i) diag = __dadd_rn(diag, t);
-            else {
-                int64_t q = find_sorted(h, m, l);
-                if (q >= 0) w[q] = __dadd_rn(w[q], t);
+// The columns that a row of the product or of the interpolation may hold, as seen by one
+// lane group: visit(i, part, nparts, f) calls f(column) for the candidates of row i that
+// fall to lane `part` of `nparts`. ub is the row's number of candidates with repeats.
+struct HatCands {  // interpolatory set of F row i: strong C neighbours, and those of strong F neighbours
+    const int64_t *__restrict__ ptr;
+    const int32_t *__restrict__ col;
+    const uint8_t *__restrict__ strong;
+    const int8_t *__restrict__ cf;
+    int cc;
+    // C rows interpolate from themselves alone
+    __device__ bool single(int64_t i) const { return cf[i] == 1; }
+    template <class F>
+    __device__ void visit(int64_t i, int part, int nparts, F f) const {
+        for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
+            if (!strong[e]) continue;
+            const int32_t k = col[e];
+            if (cf[k] == 1) {
+                if (part == 0) f(k);
+            } else if (!cc || !shares_strong_c(ptr, col, strong, cf, i, k)) {
+                for (int64_t q = ptr[k] + part; q < ptr[k + 1]; q += nparts)
+                    if (strong[q] && cf[col[q]] == 1) f(col[q]);
             }
         }
     }
-    for (int64_t q = 0; q < m; ++q) w[q] = __ddiv_rn(-w[q], diag);
-}
+};
 
-// ---------------------------------------------------------------------------------
-// Transpose (R = P^T): count, scan, scatter, then sort every row of R by column.
-// ---------------------------------------------------------------------------------
-__global__ void k_count_cols(int64_t nnz, const int32_t *__restrict__ col, unsigned long long *__restrict__ cnt) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < nnz) atomicAdd(&cnt[col[e]], 1ull);
-}
-
-__global__ void k_transpose_scatter(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                                    const double *__restrict__ val, unsigned long long *__restrict__ fill,
-                                    int32_t *__restrict__ tcol, double *__restrict__ tval) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-        unsigned long long q = atomicAdd(&fill[col[e]], 1ull);
-        tcol[q] = (int32_t)i;
-        tval[q] = val[e];
-    }
-}
-
-__global__ void k_sort_rows(int64_t n, const int64_t *__restrict__ ptr, int32_t *__restrict__ col,
-                            double *__restrict__ val) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t lo = ptr[i], hi = ptr[i + 1];
-    for (int64_t x = lo + 1; x < hi; ++x) {
-        int32_t c = col[x];
-        double v = val[x];
-        int64_t y = x - 1;
-        while (y >= lo && col[y] > c) {
-            col[y + 1] = col[y];
-            val[y + 1] = val[y];
-            --y;
+struct GemmCands {  // columns of row i of A B
+    const int64_t *__restrict__ aptr;
+    const int32_t *__restrict__ acol;
+    const int64_t *__restrict__ bptr;
+    const int32_t *__restrict__ bcol;
+    __device__ bool single(int64_t) const { return false; }
+    template <class F>
+    __device__ void visit(int64_t i, int part, int nparts, F f) const {
+        // eight lanes per row of B (fewer than 32 entries are usual), several rows at once
+        const int w = nparts < 8 ? nparts : 8;
+        for (int64_t e = aptr[i] + part / w; e < aptr[i + 1]; e += nparts / w) {
+            const int32_t k = acol[e];
+            for (int64_t q = bptr[k] + part % w; q < bptr[k + 1]; q += w) f(bcol[q]);
         }
-        col[y + 1] = c;
-        val[y + 1] = v;
     }
-}
+};
 
-// ---------------------------------------------------------------------------------
-// SpGEMM C = A B, one thread per row: the candidate columns are collected in a private
-// scratch slice, heap-sorted and de-duplicated (symbolic phase); the numeric phase adds
-// the products in the order of A's row then B's row (a fixed order per entry).
-// ---------------------------------------------------------------------------------
-__global__ void k_gemm_ub(int64_t n, const int64_t *__restrict__ aptr, const int32_t *__restrict__ acol,
-                          const int64_t *__restrict__ bptr, int64_t *__restrict__ ub) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t s = 0;
-    for (int64_t e = aptr[i]; e < aptr[i + 1]; ++e) s += bptr[acol[e] + 1] - bptr[acol[e]];
-    ub[i] = s;
+// rows[0..*nrows) (or all rows 0..n-1 when rows is null): the sorted set of row i goes to
+// scratch[ub_off[i]..], its size to cnt[i]; rows that overflow are listed in over[0..*nover)
+template <int NT, int CAP, class C>
+__global__ void __launch_bounds__(NT) k_union_rows(int64_t n, const int32_t *__restrict__ rows,
+                                                   const unsigned *__restrict__ nrows, C cands,
+                                                   const int64_t *__restrict__ ub_off,
+                                                   int32_t *__restrict__ scratch, int64_t *__restrict__ cnt,
+                                                   int32_t *__restrict__ over, unsigned *__restrict__ nover) {
+    extern __shared__ int32_t smem[];  // table, list
+    __shared__ int num;
+    ColSet<NT, CAP> set{smem, smem + CAP, &num};
+    const int64_t total = rows ? (int64_t)*nrows : n;
+    for (int64_t q = blockIdx.x; q < total; q += gridDim.x) {
+        const int64_t i = rows ? rows[q] : q;
+        if (cands.single(i)) {
+            if (threadIdx.x == 0) cnt[i] = 1;
+            continue;
+        }
+        __syncthreads();
+        set.clear();
+        cands.visit(i, threadIdx.x, NT, [&](int32_t v) { set.insert(v); });
+        const int m = set.sorted(scratch + ub_off[i]);
+        if (threadIdx.x == 0) {
+            cnt[i] = m;
+            if (m < 0) over[atomicAdd(nover, 1u)] = (int32_t)i;
+        }
+    }
 }
 
 __device__ void heap_sort_i32(int32_t *a, int64_t m) {
@@ -450,228 +299,329 @@ __device__ void heap_sort_i32(int32_t *a, int64_t m) {
     }
 }
 
-__global__ void k_gemm_symbolic(int64_t n, const int64_t *__restrict__ aptr, const int32_t *__restrict__ acol,
-                                const int64_t *__restrict__ bptr, const int32_t *__restrict__ bcol,
-                                const int64_t *__restrict__ ub_off, int32_t *__restrict__ scratch,
-                                int64_t *__restrict__ cnt) {
+// the rows that no table holds (thousands of distinct columns): one thread per row
+template <class C>
+__global__ void k_union_heap(const int32_t *__restrict__ rows, const unsigned *__restrict__ nrows, C cands,
+                             const int64_t *__restrict__ ub_off, int32_t *__restrict__ scratch,
+                             int64_t *__restrict__ cnt) {
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)*nrows;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = rows[q];
+        int32_t *h = scratch + ub_off[i];
+        int64_t m = 0;
+        cands.visit(i, 0, 1, [&](int32_t v) { h[m++] = v; });
+        heap_sort_i32(h, m);
+        int64_t u = 0;
+        for (int64_t x = 0; x < m; ++x)
+            if (x == 0 || h[x] != h[x - 1]) h[u++] = h[x];
+        cnt[i] = u;
+    }
+}
+
+__device__ __forceinline__ double abar(double akl, double akk) {
+    if (akk > 0.0) return akl < 0.0 ? akl : 0.0;
+    if (akk < 0.0) return akl > 0.0 ? akl : 0.0;
+    return akl;
+}
+
+__device__ __forceinline__ int64_t find_sorted(const int32_t *h, int64_t m, int32_t v) {
+    int64_t lo = 0, hi = m;
+    while (lo < hi) {
+        int64_t mid = (lo + hi) >> 1;
+        if (h[mid] < v) lo = mid + 1;
+        else hi = mid;
+    }
+    return (lo < m && h[lo] == v) ? lo : -1;
+}
+
+// adds the lanes' values v (where has) to acc in lane order, one after another: the sum
+// is that of a loop over the entries, which the oracle runs too
+__device__ __forceinline__ double ordered_add(double acc, bool has, double v) {
+    for (unsigned m = __ballot_sync(0xffffffffu, has); m; m &= m - 1)
+        acc = __dadd_rn(acc, __shfl_sync(0xffffffffu, v, __ffs(m) - 1));
+    return acc;
+}
+
+// One warp per row; the lanes share the entries of the row being read, and every sum runs
+// in the order of those entries (ordered_add; a weight w[q] gets its terms in the order
+// of the strong F neighbours). Thread per row was bound by its chains of dependent
+// accesses: 43 of 312 ms of the setup at P3 24^3, against 0.7 ms here.
+__global__ void k_extpi_fill(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
+                             const double *__restrict__ val, const uint8_t *__restrict__ strong,
+                             const int8_t *__restrict__ cf, const int64_t *__restrict__ cidx,
+                             const int64_t *__restrict__ ub_off, const int32_t *__restrict__ scratch,
+                             const int64_t *__restrict__ pptr, int32_t *__restrict__ pcol, double *pval) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (i >= n) return;  // a whole warp, as every branch below
+    const int64_t o = pptr[i];
+    if (cf[i] == 1) {
+        if (lane == 0) {
+            pcol[o] = (int32_t)cidx[i];
+            pval[o] = 1.0;
+        }
+        return;
+    }
+    const int64_t m = pptr[i + 1] - o;
+    if (m == 0) return;
+    const int32_t *h = scratch + ub_off[i];
+    double *w = pval + o;
+    for (int64_t q = lane; q < m; q += 32) {
+        w[q] = 0.0;
+        pcol[o + q] = (int32_t)cidx[h[q]];
+    }
+    __syncwarp();
+    const int64_t lo = ptr[i], hi = ptr[i + 1];
+    const int64_t di = lower_bound_col(col, lo, hi, (int32_t)i);
+    double diag = di < hi && col[di] == (int32_t)i ? val[di] : 0.0;
+    for (int64_t e0 = lo; e0 < hi; e0 += 32) {
+        const int64_t e = e0 + lane;
+        const bool off = e < hi && col[e] != i;
+        const double v = off ? val[e] : 0.0;
+        const int64_t q = off ? find_sorted(h, m, col[e]) : -1;
+        if (q >= 0) w[q] = v;
+        diag = ordered_add(diag, off && q < 0 && !strong[e], v);
+    }
+    __syncwarp();
+    for (int64_t e = lo; e < hi; ++e) {
+        if (!strong[e]) continue;
+        const int32_t k = col[e];
+        if (cf[k] != -1) continue;
+        const double aik = val[e];
+        const int64_t klo = ptr[k], khi = ptr[k + 1];
+        const int64_t dk = lower_bound_col(col, klo, khi, k);
+        const double akk = dk < khi && col[dk] == k ? val[dk] : 0.0;
+        double d = 0.0;
+        for (int64_t f0 = klo; f0 < khi; f0 += 32) {
+            const int64_t f = f0 + lane;
+            const int32_t l = f < khi ? col[f] : k;
+            const bool in = l != k && (l == i || find_sorted(h, m, l) >= 0);
+            d = ordered_add(d, in, in ? abar(val[f], akk) : 0.0);
+        }
+        if (d == 0.0) {
+            diag = __dadd_rn(diag, aik);
+            continue;
+        }
+        for (int64_t f0 = klo; f0 < khi; f0 += 32) {
+            const int64_t f = f0 + lane;
+            const int32_t l = f < khi ? col[f] : k;
+            const int64_t q = l != k && l != i ? find_sorted(h, m, l) : -1;
+            const bool in = l != k && (l == i || q >= 0);
+            const double t = in ? __ddiv_rn(__dmul_rn(aik, abar(val[f], akk)), d) : 0.0;
+            if (q >= 0) w[q] = __dadd_rn(w[q], t);
+            diag = ordered_add(diag, in && l == i, t);
+        }
+        __syncwarp();  // w is read by other lanes for the next neighbour
+    }
+    for (int64_t q = lane; q < m; q += 32) w[q] = __ddiv_rn(-w[q], diag);
+}
+
+// ---------------------------------------------------------------------------------
+// Transpose (R = P^T): count, scan, scatter, then sort every row of R by column.
+// ---------------------------------------------------------------------------------
+__global__ void k_count_cols(int64_t nnz, const int32_t *__restrict__ col, unsigned long long *__restrict__ cnt) {
+    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < nnz) atomicAdd(&cnt[col[e]], 1ull);
+}
+
+__global__ void k_transpose_scatter(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
+                                    const double *__restrict__ val, unsigned long long *__restrict__ fill,
+                                    int32_t *__restrict__ tcol, double *__restrict__ tval) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    int32_t *h = scratch + ub_off[i];
-    int64_t m = 0;
-    for (int64_t e = aptr[i]; e < aptr[i + 1]; ++e) {
-        int32_t k = acol[e];
-        for (int64_t f = bptr[k]; f < bptr[k + 1]; ++f) h[m++] = bcol[f];
+    for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
+        unsigned long long q = atomicAdd(&fill[col[e]], 1ull);
+        tcol[q] = (int32_t)i;
+        tval[q] = val[e];
     }
-    heap_sort_i32(h, m);
-    int64_t u = 0;
-    for (int64_t x = 0; x < m; ++x)
-        if (x == 0 || h[x] != h[x - 1]) h[u++] = h[x];
-    cnt[i] = u;
+}
+
+// one warp per row: an entry's place is the number of smaller columns in its row (the
+// columns of a row are distinct)
+__global__ void k_sort_rows(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ icol,
+                            const double *__restrict__ ival, int32_t *__restrict__ col, double *__restrict__ val) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (i >= n) return;
+    const int64_t lo = ptr[i], hi = ptr[i + 1];
+    for (int64_t x = lo + lane; x < hi; x += 32) {
+        const int32_t c = icol[x];
+        int64_t at = lo;
+        for (int64_t y = lo; y < hi; ++y) at += icol[y] < c;
+        col[at] = c;
+        val[at] = ival[x];
+    }
+}
+
+// ---------------------------------------------------------------------------------
+// SpGEMM C = A B: the sorted columns of every row (union_rows), then one warp per row
+// adds the products in the order of A's row and then B's row (the lanes take the entries
+// of one row of B, which are distinct columns): a fixed order per entry.
+// ---------------------------------------------------------------------------------
+__global__ void k_gemm_ub(int64_t n, const int64_t *__restrict__ aptr, const int32_t *__restrict__ acol,
+                          const int64_t *__restrict__ bptr, int64_t *__restrict__ ub) {
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    int64_t s = 0;
+    for (int64_t e = aptr[i]; e < aptr[i + 1]; ++e) s += bptr[acol[e] + 1] - bptr[acol[e]];
+    ub[i] = s;
 }
 
 __global__ void k_gemm_numeric(int64_t n, const int64_t *__restrict__ aptr, const int32_t *__restrict__ acol,
                                const double *__restrict__ aval, const int64_t *__restrict__ bptr,
                                const int32_t *__restrict__ bcol, const double *__restrict__ bval,
                                const int64_t *__restrict__ ub_off, const int32_t *__restrict__ scratch,
-                               const int64_t *__restrict__ cptr, int32_t *__restrict__ ccol,
-                               double *__restrict__ cval) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                               const int64_t *__restrict__ cptr, int32_t *__restrict__ ccol, double *cval) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (i >= n) return;
-    const int64_t lo = cptr[i], hi = cptr[i + 1];
+    const int64_t lo = cptr[i], m = cptr[i + 1] - lo;
     const int32_t *h = scratch + ub_off[i];
-    for (int64_t q = lo; q < hi; ++q) {
-        ccol[q] = h[q - lo];
-        cval[q] = 0.0;
+    for (int64_t q = lane; q < m; q += 32) {
+        ccol[lo + q] = h[q];
+        cval[lo + q] = 0.0;
     }
+    __syncwarp();
     for (int64_t e = aptr[i]; e < aptr[i + 1]; ++e) {
-        int32_t k = acol[e];
-        double a = aval[e];
-        for (int64_t f = bptr[k]; f < bptr[k + 1]; ++f) {
-            int64_t q = lower_bound_col(ccol, lo, hi, bcol[f]);
-            if (q < hi) cval[q] = __dadd_rn(cval[q], __dmul_rn(a, bval[f]));
+        const int32_t k = acol[e];
+        const double a = aval[e];
+        for (int64_t f = bptr[k] + lane; f < bptr[k + 1]; f += 32) {
+            const int64_t q = find_sorted(h, m, bcol[f]);
+            if (q >= 0) cval[lo + q] = __dadd_rn(cval[lo + q], __dmul_rn(a, bval[f]));
         }
+        __syncwarp();  // the next row of B may reach the same entries from other lanes
     }
 }
 
 // ---------------------------------------------------------------------------------
-// Coarsest level: dense Cholesky factor and explicit inverse (one block).
+// Coarsest level: explicit inverse of a dense SPD matrix by in-place block Gauss-Jordan
+// elimination, kGj rows at a time and without pivoting (every pivot of a positive definite
+// matrix is the square of a Cholesky pivot; one that is not positive reports the matrix).
+// For the pivot block K:  D = A_KK^{-1},  R = D A_K*,  A_i* -= A_iK R  for i outside K
+// (columns K start from 0 there), A_K* = R with D in its columns K. The n^3 FMAs need many
+// SMs (2 FP64 FMAs per clock per SM): one block's Cholesky factor and triangular solves
+// took 0.61 ms for 73 rows and grew with their cube; three small launches per pivot block
+// take 0.29 ms with the allocations around them (0.23 ms for 62 rows).
 // ---------------------------------------------------------------------------------
+constexpr int kGj = 32;
+
 __global__ void k_csr_to_dense(int64_t n, const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
                                const double *__restrict__ val, double *__restrict__ D) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    for (int64_t j = 0; j < n; ++j) D[i * n + j] = 0.0;
     for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) D[i * n + col[e]] = val[e];
 }
 
-__global__ void k_cholesky_inverse(int64_t n, double *__restrict__ L, double *__restrict__ Ainv,
-                                   int *__restrict__ bad) {
-    __shared__ double piv;
-    // right-looking is not needed: column j uses the finished columns q < j
-    for (int64_t j = 0; j < n; ++j) {
-        if (threadIdx.x == 0) {
-            double s = L[j * n + j];
-            for (int64_t q = 0; q < j; ++q) s -= L[j * n + q] * L[j * n + q];
-            if (!(s > 0.0)) {
-                atomicExch(bad, 1);
-                s = 1.0;
+// D = inverse of the pivot block at k0 (32 x 32 threads; rows past n are the identity)
+__global__ void __launch_bounds__(kGj *kGj) k_gj_pivot(int64_t n, int64_t k0, const double *__restrict__ A,
+                                                       double *__restrict__ D, int *__restrict__ bad) {
+    __shared__ double a[kGj][kGj + 1];
+    const int i = threadIdx.y, j = threadIdx.x;
+    const bool in = k0 + i < n && k0 + j < n;
+    a[i][j] = in ? A[(k0 + i) * n + k0 + j] : (i == j ? 1.0 : 0.0);
+    __syncthreads();
+    for (int p = 0; p < kGj; ++p) {
+        const double aip = a[i][p];
+        __syncthreads();
+        if (i == p) {  // one warp: the pivot row
+            double piv = aip;
+            if (!(piv > 0.0)) {
+                if (j == 0) atomicExch(bad, 1);
+                piv = 1.0;
             }
-            piv = sqrt(s);
-            L[j * n + j] = piv;
+            const double inv = 1.0 / piv;
+            a[p][j] = j == p ? inv : a[p][j] * inv;
         }
         __syncthreads();
-        for (int64_t i = j + 1 + threadIdx.x; i < n; i += blockDim.x) {
-            double t = L[i * n + j];
-            for (int64_t q = 0; q < j; ++q) t -= L[i * n + q] * L[j * n + q];
-            L[i * n + j] = t / piv;
-        }
+        if (i != p) a[i][j] = (j == p ? 0.0 : a[i][j]) - aip * a[p][j];
         __syncthreads();
     }
-    // column c of A^{-1}: solve L y = e_c, then L^T x = y (x stored in Ainv column c)
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
-        for (int64_t i = 0; i < n; ++i) {
-            double s = (i == c) ? 1.0 : 0.0;
-            for (int64_t q = c; q < i; ++q) s -= L[i * n + q] * Ainv[q * n + c];
-            Ainv[i * n + c] = (i < c) ? 0.0 : s / L[i * n + i];
+    D[i * kGj + j] = a[i][j];
+}
+
+// R = D A_K* (its columns K hold D) and C = A_*K, one thread per column (row)
+__global__ void k_gj_panels(int64_t n, int64_t k0, const double *__restrict__ A, const double *__restrict__ D,
+                            double *__restrict__ R, double *__restrict__ C) {
+    __shared__ double d[kGj * kGj];
+    for (int q = threadIdx.x; q < kGj * kGj; q += blockDim.x) d[q] = D[q];
+    __syncthreads();
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    double v[kGj];
+#pragma unroll
+    for (int q = 0; q < kGj; ++q) v[q] = k0 + q < n ? A[(k0 + q) * n + j] : 0.0;
+    const int64_t own = j - k0;
+    for (int q = 0; q < kGj; ++q) {
+        double t = 0.0;
+#pragma unroll
+        for (int u = 0; u < kGj; ++u) t += d[q * kGj + u] * v[u];
+        R[(int64_t)q * n + j] = own >= 0 && own < kGj ? d[q * kGj + own] : t;
+    }
+    for (int q = 0; q < kGj; ++q) C[j * kGj + q] = k0 + q < n ? A[j * n + k0 + q] : 0.0;
+}
+
+__global__ void k_gj_update(int64_t n, int64_t k0, const double *__restrict__ R, const double *__restrict__ C,
+                            double *__restrict__ A) {
+    __shared__ double r[kGj][kGj], c[kGj][kGj + 1];
+    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+    const int64_t j = (int64_t)blockIdx.x * kGj + tx, i0 = (int64_t)blockIdx.y * kGj;
+    for (int q = ty; q < kGj; q += 8) {
+        r[q][tx] = j < n ? R[(int64_t)q * n + j] : 0.0;
+        c[q][tx] = i0 + q < n ? C[(i0 + q) * kGj + tx] : 0.0;
+    }
+    __syncthreads();
+    if (j >= n) return;
+    const bool jk = j >= k0 && j < k0 + kGj;
+    for (int q = ty; q < kGj; q += 8) {
+        const int64_t i = i0 + q;
+        if (i >= n) break;
+        if (i >= k0 && i < k0 + kGj) {
+            A[i * n + j] = r[i - k0][tx];
+            continue;
         }
-        for (int64_t i = n - 1; i >= 0; --i) {
-            double s = Ainv[i * n + c];
-            for (int64_t q = i + 1; q < n; ++q) s -= L[q * n + i] * Ainv[q * n + c];
-            Ainv[i * n + c] = s / L[i * n + i];
-        }
+        double t = jk ? 0.0 : A[i * n + j];
+#pragma unroll
+        for (int u = 0; u < kGj; ++u) t -= c[q][u] * r[u][tx];
+        A[i * n + j] = t;
     }
 }
 
 // ---------------------------------------------------------------------------------
 // host drivers
 // ---------------------------------------------------------------------------------
-int jp_colour(int64_t n, const int64_t *ptr, const int32_t *col, uint64_t stream, int32_t *colour,
-              DevPool &tmp, cudaStream_t s) {
-    uint8_t *pick = tmp.get<uint8_t>(n);
-    unsigned long long *cnt = tmp.get<unsigned long long>(1);
-    int *maxc = tmp.get<int>(1);
-    PK_CUDA(cudaMemsetAsync(colour, 0xff, sizeof(int32_t) * n, s));
-    PK_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
-    PK_CUDA(cudaMemsetAsync(maxc, 0, sizeof(int), s));
-    unsigned long long done = 0;
-    int rounds = 0;
-    while ((int64_t)done < n) {
-        for (int r = 0; r < 4; ++r) {
-            k_jp_pick<<<blocks_for(n, 256), 256, 0, s>>>(n, ptr, col, stream, colour, pick);
-            PK_LAUNCH();
-            k_jp_assign<<<blocks_for(n, 256), 256, 0, s>>>(n, ptr, col, colour, pick, cnt, maxc);
-            PK_LAUNCH();
-        }
-        PK_CUDA(cudaMemcpyAsync(&done, cnt, sizeof(done), cudaMemcpyDeviceToHost, s));
-        PK_CUDA(cudaStreamSynchronize(s));
-        rounds += 4;
-        if (rounds > 4 * (n + 8)) fail(PKASP_ECUDA, "colouring did not terminate");
-    }
-    int h = 0;
-    PK_CUDA(cudaMemcpyAsync(&h, maxc, sizeof(int), cudaMemcpyDeviceToHost, s));
+}  // namespace
+
+namespace {
+
+// the sorted candidate columns of every row: a block of one warp and a 1024-slot table per
+// row (28 blocks of 8 KB per SM), then 256 threads and 16384 slots for the rows that
+// overflow it, then the heap sort
+template <class C>
+void union_rows(int64_t n, const C &cands, const int64_t *ub_off, int32_t *scratch, int64_t *cnt, DevPool &tmp,
+                cudaStream_t s) {
+    if (n <= 0) return;
+    int32_t *over = tmp.get<int32_t>(2 * n);
+    unsigned *nover = tmp.get<unsigned>(2);
+    PK_CUDA(cudaMemsetAsync(nover, 0, sizeof(unsigned) * 2, s));
+    constexpr int cap1 = 1024, cap2 = 16384;
+    k_union_rows<32, cap1, C><<<(unsigned)std::min<int64_t>(n, 152 * 28), 32, 2 * cap1 * sizeof(int32_t), s>>>(
+        n, nullptr, nullptr, cands, ub_off, scratch, cnt, over, nover);
+    PK_LAUNCH();
+    unsigned left[2];
+    PK_CUDA(cudaMemcpyAsync(left, nover, sizeof(left), cudaMemcpyDeviceToHost, s));
     PK_CUDA(cudaStreamSynchronize(s));
-    return h;
+    if (left[0] == 0) return;
+    auto big = k_union_rows<256, cap2, C>;
+    const size_t sm2 = 2 * cap2 * sizeof(int32_t);
+    PK_CUDA(cudaFuncSetAttribute(big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2));
+    big<<<(unsigned)std::min<unsigned>(left[0], 152), 256, sm2, s>>>(n, over, nover, cands, ub_off, scratch, cnt,
+                                                                    over + n, nover + 1);
+    PK_LAUNCH();
+    k_union_heap<C><<<152, 128, 0, s>>>(over + n, nover + 1, cands, ub_off, scratch, cnt);
+    PK_LAUNCH();
 }
 
 }  // namespace
-
-// Colour split of A for the multicolour Gauss-Seidel sweeps.
-void build_split(DevPool &pool, const DCSR &A, uint64_t stream, bool want32, DSplit &sp, cudaStream_t s) {
-    DevPool tmp;
-    try {
-        const int64_t n = A.n;
-        sp.colour = pool.get<int32_t>(n > 0 ? n : 1);
-        sp.ncol = n > 0 ? jp_colour(n, A.ptr, A.col, stream, sp.colour, tmp, s) : 0;
-        // stable counting sort of the rows by colour (host: n small integers)
-        std::vector<int32_t> hc(n);
-        PK_CUDA(cudaMemcpyAsync(hc.data(), sp.colour, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, s));
-        PK_CUDA(cudaStreamSynchronize(s));
-        sp.off.assign(sp.ncol + 1, 0);
-        for (int32_t c : hc) sp.off[c + 1]++;
-        for (int c = 0; c < sp.ncol; ++c) sp.off[c + 1] += sp.off[c];
-        std::vector<int64_t> fill(sp.off.begin(), sp.off.end() - 1);
-        std::vector<int32_t> perm(n);
-        for (int64_t i = 0; i < n; ++i) perm[fill[hc[i]]++] = (int32_t)i;
-        sp.perm = pool.get<int32_t>(n > 0 ? n : 1);
-        PK_CUDA(cudaMemcpyAsync(sp.perm, perm.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, s));
-        sp.lptr = pool.get<int64_t>(n + 1);
-        sp.uptr = pool.get<int64_t>(n + 1);
-        if (n > 0) {
-            k_split_count<<<blocks_for(n, 256), 256, 0, s>>>(n, sp.perm, A.ptr, A.col, sp.colour, sp.lptr, sp.uptr);
-            PK_LAUNCH();
-        }
-        exclusive_scan(sp.lptr, n, s);
-        exclusive_scan(sp.uptr, n, s);
-        sp.nnz_l = read_i64(sp.lptr + n, s);
-        sp.nnz_u = read_i64(sp.uptr + n, s);
-        {
-            // longest lower/upper part of each colour: it fixes the lanes per row of that
-            // colour's phase (one batch of loads per lane covers the whole row)
-            std::vector<int64_t> hl(n + 1), hu(n + 1);
-            PK_CUDA(cudaMemcpyAsync(hl.data(), sp.lptr, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s));
-            PK_CUDA(cudaMemcpyAsync(hu.data(), sp.uptr, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s));
-            PK_CUDA(cudaStreamSynchronize(s));
-            sp.lmax.assign(sp.ncol, 0);
-            sp.umax.assign(sp.ncol, 0);
-            sp.l90.assign(sp.ncol, 0);
-            sp.u90.assign(sp.ncol, 0);
-            std::vector<int> ll, ul;
-            for (int c = 0; c < sp.ncol; ++c) {
-                ll.clear();
-                ul.clear();
-                for (int64_t q = sp.off[c]; q < sp.off[c + 1]; ++q) {
-                    ll.push_back((int)(hl[q + 1] - hl[q]));
-                    ul.push_back((int)(hu[q + 1] - hu[q]));
-                    sp.lmax[c] = std::max<int>(sp.lmax[c], ll.back());
-                    sp.umax[c] = std::max<int>(sp.umax[c], ul.back());
-                }
-                // 90th percentile: the length one batch of loads should cover
-                if (!ll.empty()) {
-                    const size_t k = (ll.size() * 9) / 10;
-                    std::nth_element(ll.begin(), ll.begin() + k, ll.end());
-                    std::nth_element(ul.begin(), ul.begin() + k, ul.end());
-                    sp.l90[c] = ll[k];
-                    sp.u90[c] = ul[k];
-                }
-            }
-        }
-        sp.lcol = pool.get<int32_t>(sp.nnz_l > 0 ? sp.nnz_l : 1);
-        sp.lval = pool.get<double>(sp.nnz_l > 0 ? sp.nnz_l : 1);
-        sp.ucol = pool.get<int32_t>(sp.nnz_u > 0 ? sp.nnz_u : 1);
-        sp.uval = pool.get<double>(sp.nnz_u > 0 ? sp.nnz_u : 1);
-        sp.diag = pool.get<double>(n > 0 ? n : 1);
-        sp.dinv = pool.get<double>(n > 0 ? n : 1);
-        int *bad = tmp.get<int>(1);
-        PK_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
-        if (n > 0) {
-            k_split_fill<<<blocks_for(n, 256), 256, 0, s>>>(n, sp.perm, A.ptr, A.col, A.val, sp.colour, sp.lptr,
-                                                            sp.uptr, sp.lcol, sp.lval, sp.ucol, sp.uval, sp.diag,
-                                                            sp.dinv, bad);
-            PK_LAUNCH();
-        }
-        int hb = 0;
-        PK_CUDA(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
-        PK_CUDA(cudaStreamSynchronize(s));
-        if (hb == 1) fail(PKASP_EBREAKDOWN, "zero diagonal entry in a smoothed matrix");
-        if (hb == 2) fail(PKASP_ECUDA, "colouring left two neighbours with the same colour");
-        if (want32) {
-            sp.lval32 = pool.get<float>(sp.nnz_l > 0 ? sp.nnz_l : 1);
-            sp.uval32 = pool.get<float>(sp.nnz_u > 0 ? sp.nnz_u : 1);
-            sp.diag32 = pool.get<float>(n > 0 ? n : 1);
-            sp.dinv32 = pool.get<float>(n > 0 ? n : 1);
-            to32(sp.lval, sp.lval32, sp.nnz_l, s);
-            to32(sp.uval, sp.uval32, sp.nnz_u, s);
-            to32(sp.diag, sp.diag32, n, s);
-            to32(sp.dinv, sp.dinv32, n, s);
-        }
-        PK_CUDA(cudaStreamSynchronize(s));
-    } catch (...) {
-        cudaStreamSynchronize(s);
-        tmp.free_all();
-        throw;
-    }
-    tmp.free_all();
-}
 
 double *row_l1(DevPool &pool, const DCSR &A, cudaStream_t s) {
     double *l1 = pool.get<double>(A.n > 0 ? A.n : 1);
@@ -697,16 +647,13 @@ void spgemm(DevPool &pool, const DCSR &A, const DCSR &B, DCSR &C, cudaStream_t s
         if (tot > ((int64_t)1 << 31)) fail(PKASP_ENOMEM, "Galerkin product scratch above 2^31 entries");
         int32_t *scr = tmp.get<int32_t>(tot > 0 ? tot : 1);
         int64_t *cnt = tmp.get<int64_t>(n + 1);
-        if (n > 0) {
-            k_gemm_symbolic<<<blocks_for(n, 128), 128, 0, s>>>(n, A.ptr, A.col, B.ptr, B.col, ub, scr, cnt);
-            PK_LAUNCH();
-        }
+        union_rows(n, GemmCands{A.ptr, A.col, B.ptr, B.col}, ub, scr, cnt, tmp, s);
         exclusive_scan(cnt, n, s);
         int64_t nnz = read_i64(cnt + n, s);
         dcsr_alloc(pool, C, n, B.m, nnz);
         PK_CUDA(cudaMemcpyAsync(C.ptr, cnt, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
         if (n > 0) {
-            k_gemm_numeric<<<blocks_for(n, 128), 128, 0, s>>>(n, A.ptr, A.col, A.val, B.ptr, B.col, B.val, ub, scr,
+            k_gemm_numeric<<<blocks_for(n * 32, 128), 128, 0, s>>>(n, A.ptr, A.col, A.val, B.ptr, B.col, B.val, ub, scr,
                                                              C.ptr, C.col, C.val);
             PK_LAUNCH();
         }
@@ -732,13 +679,15 @@ void transpose(DevPool &pool, const DCSR &A, DCSR &T, cudaStream_t s) {
         static_assert(sizeof(unsigned long long) == sizeof(int64_t), "scan type");
         exclusive_scan(reinterpret_cast<int64_t *>(cnt), m, s);
         dcsr_alloc(pool, T, m, A.n, A.nnz);
+        int32_t *ucol = tmp.get<int32_t>(A.nnz > 0 ? A.nnz : 1);  // entries in the order of arrival
+        double *uval = tmp.get<double>(A.nnz > 0 ? A.nnz : 1);
         PK_CUDA(cudaMemcpyAsync(T.ptr, cnt, sizeof(int64_t) * (m + 1), cudaMemcpyDeviceToDevice, s));
         if (A.n > 0) {
-            k_transpose_scatter<<<blocks_for(A.n, 256), 256, 0, s>>>(A.n, A.ptr, A.col, A.val, cnt, T.col, T.val);
+            k_transpose_scatter<<<blocks_for(A.n, 256), 256, 0, s>>>(A.n, A.ptr, A.col, A.val, cnt, ucol, uval);
             PK_LAUNCH();
         }
         if (m > 0) {
-            k_sort_rows<<<blocks_for(m, 128), 128, 0, s>>>(m, T.ptr, T.col, T.val);
+            k_sort_rows<<<blocks_for(m * 32, 128), 128, 0, s>>>(m, T.ptr, ucol, uval, T.col, T.val);
             PK_LAUNCH();
         }
         PK_CUDA(cudaStreamSynchronize(s));
@@ -891,15 +840,14 @@ bool coarsen(DevPool &pool, Level &L, double theta, uint64_t pmis_stream, DCSR &
             if (tot > ((int64_t)1 << 31)) fail(PKASP_ENOMEM, "interpolation scratch above 2^31 entries");
             int32_t *scr = tmp.get<int32_t>(tot > 0 ? tot : 1);
             int64_t *cnt = tmp.get<int64_t>(n + 1);
-            k_extpi_hat<<<blocks_for(n, 128), 128, 0, s>>>(n, A.ptr, A.col, L.strong, L.cf, ub, scr, cnt, cc);
-            PK_LAUNCH();
+            union_rows(n, HatCands{A.ptr, A.col, L.strong, L.cf, cc}, ub, scr, cnt, tmp, s);
             exclusive_scan(cnt, n, s);
             int64_t pnnz = read_i64(cnt + n, s);
             const bool trunc = trunc_factor > 0.0 || pmax > 0;
             DCSR full;  // ext+i before truncation (scratch when truncating)
             dcsr_alloc(trunc ? tmp : pool, full, n, nc, pnnz);
             PK_CUDA(cudaMemcpyAsync(full.ptr, cnt, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
-            k_extpi_fill<<<blocks_for(n, 128), 128, 0, s>>>(n, A.ptr, A.col, A.val, L.strong, L.cf, cidx, ub, scr,
+            k_extpi_fill<<<blocks_for(n * 32, 128), 128, 0, s>>>(n, A.ptr, A.col, A.val, L.strong, L.cf, cidx, ub, scr,
                                                             full.ptr, full.col, full.val);
             PK_LAUNCH();
             if (trunc) {
@@ -941,20 +889,30 @@ bool coarsen(DevPool &pool, Level &L, double theta, uint64_t pmis_stream, DCSR &
     return ok;
 }
 
-// Dense inverse of the coarsest matrix.
+// Dense inverse of the coarsest matrix (block Gauss-Jordan, above).
 void coarse_inverse(DevPool &pool, const DCSR &A, double **inv, cudaStream_t s) {
     const int64_t n = A.n;
     if (n > 8192) fail(PKASP_ENOMEM, "coarsest level has more than 8192 rows; raise max_levels or coarse_size");
     DevPool tmp;
     try {
-        double *L = tmp.get<double>(n * n > 0 ? n * n : 1);
-        *inv = pool.get<double>(n * n > 0 ? n * n : 1);
+        double *A0 = pool.get<double>(n * n > 0 ? n * n : 1);
+        double *D = tmp.get<double>(kGj * kGj), *R = tmp.get<double>(kGj * std::max<int64_t>(n, 1)),
+               *C = tmp.get<double>(kGj * std::max<int64_t>(n, 1));
         int *bad = tmp.get<int>(1);
+        *inv = A0;
         PK_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
+        PK_CUDA(cudaMemsetAsync(A0, 0, sizeof(double) * n * n, s));
         if (n > 0) {
-            k_csr_to_dense<<<blocks_for(n, 128), 128, 0, s>>>(n, A.ptr, A.col, A.val, L);
+            k_csr_to_dense<<<blocks_for(n, 128), 128, 0, s>>>(n, A.ptr, A.col, A.val, A0);
             PK_LAUNCH();
-            k_cholesky_inverse<<<1, 1024, 0, s>>>(n, L, *inv, bad);
+        }
+        const unsigned tiles = blocks_for(n, kGj);
+        for (int64_t k0 = 0; k0 < n; k0 += kGj) {
+            k_gj_pivot<<<1, dim3(kGj, kGj), 0, s>>>(n, k0, A0, D, bad);
+            PK_LAUNCH();
+            k_gj_panels<<<blocks_for(n, 64), 64, 0, s>>>(n, k0, A0, D, R, C);
+            PK_LAUNCH();
+            k_gj_update<<<dim3(tiles, tiles), dim3(kGj, 8), 0, s>>>(n, k0, R, C, A0);
             PK_LAUNCH();
         }
         int hb = 0;

@@ -1060,7 +1060,7 @@ void autotune(pkasp_problem *p, cudaStream_t s) {
     // 769 vs 467 us; they stay selectable through smoother_layout)
     // 400 + t: t lanes, grid-stride over the resident blocks, the next row's static loads
     // in flight during the current row's gathers.
-    const int cand_fine[] = {-1, 0, 4, 8, 16, 104, 108, 116, 404, 408, 416};
+    const int cand_fine[] = {-1, 4, 8, 16, 104, 108, 116, 404, 408, 416};
     const int pick_spmv = tune(cand_spmv, 4, &p->spmv_tpr, [&] { spmv_fine(p, p->d_b, p->w_q, s); });
     p->spmv_tpr = pick_spmv;
     int pick_fine = -1;
@@ -1068,9 +1068,9 @@ void autotune(pkasp_problem *p, cudaStream_t s) {
         pick_fine = fixed_fine;
     } else if (p->opt.smoother == PKASP_SMOOTHER_SGS) {
         if (p->opt.precond_precision == PKASP_PREC_FP32)
-            pick_fine = tune(cand_fine, 11, &p->fine_tpr, [&] { smoother<float>(p, p->d_b, p->w_zs32, s); });
+            pick_fine = tune(cand_fine, 10, &p->fine_tpr, [&] { smoother<float>(p, p->d_b, p->w_zs32, s); });
         else
-            pick_fine = tune(cand_fine, 11, &p->fine_tpr, [&] { smoother<double>(p, p->d_b, p->w_zs, s); });
+            pick_fine = tune(cand_fine, 10, &p->fine_tpr, [&] { smoother<double>(p, p->d_b, p->w_zs, s); });
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1087,8 +1087,10 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
     // fine level: colour split of A_h, l1 norms, FP32 copies
     build_split(pool, p->Ah, stream_colour(o.seed, 0), want32, p->fine, s);
     build_sell_natural(pool, p->Ah, p->Asell, false, s);
-    build_sell_split(pool, p->fine, p->nh, false, p->fsl, want32, s);
-    build_sell_split(pool, p->fine, p->nh, true, p->fsu, want32, s);
+    if (o.smoother_layout == 2) {
+        build_sell_split(pool, p->fine, p->nh, false, p->fsl, want32, s);
+        build_sell_split(pool, p->fine, p->nh, true, p->fsu, want32, s);
+    }
     p->d_l1h = row_l1(pool, p->Ah, s);
     if (want32) {
         p->d_l1h32 = pool.get<float>(p->nh);

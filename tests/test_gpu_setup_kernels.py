@@ -1,0 +1,57 @@
+"""The device-side setup at the edges of its kernels, against the oracle: Galerkin and
+interpolation rows that overflow the first column table (more than 512 distinct columns,
+plain AMG on P4 matrices), and coarsest inverses whose size is below, at and above a
+multiple of the 32-row pivot block. Integer decisions are exact; values are held to the
+tolerance of the other setup tests (1e-12 of the largest entry), cycles to 1e-11."""
+import numpy as np
+import pytest
+
+from paper_1204_2586_gb300.inputs import kappa_lognormal, kuhn_mesh
+
+pytestmark = pytest.mark.gpu
+
+
+def _close(a, b, tol):
+    assert np.abs(a - b).max() <= tol * np.abs(b).max()
+
+
+def _pair(oracle_mod, k, n, **kw):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    kap = kappa_lognormal(t.shape[0], 1)
+    G, O = Problem(xyz, t, k, kap), oracle_mod.Problem(xyz, t, k, kap)
+    G.setup(**kw)
+    O.setup(**kw)
+    return torch, G, O
+
+
+@pytest.mark.parametrize("k,n,theta", [(4, 5, 0.0), (3, 6, 0.0)])
+def test_rows_with_many_columns(oracle_mod, k, n, theta):
+    _, G, O = _pair(oracle_mod, k, n, mode=2, theta=theta, coarse_size=20)
+    longest = 0
+    assert G.info.levels == O.levels()
+    for l in range(O.levels()):
+        Lo = O.level(l)
+        c, nc = G.colours(l)
+        assert np.array_equal(c, Lo["colour"]) and nc == Lo["ncolour"]
+        for which, key in ((3 + 2 * l, "A"), (4 + 2 * l, "P")):
+            if key not in Lo:
+                continue
+            ptr, col, val, shape = G.matrix(which)
+            assert shape == Lo[key].shape and np.array_equal(ptr, Lo[key].ptr) and np.array_equal(col, Lo[key].col)
+            _close(val, Lo[key].val, 1e-12)
+        if l > 0:
+            longest = max(longest, int(np.diff(Lo["A"].ptr).max()))
+    assert longest > 512  # the larger table was needed
+
+
+@pytest.mark.parametrize("n,coarse_size", [(4, 256), (5, 256), (6, 40), (7, 256), (9, 600)])
+def test_coarsest_inverse(oracle_mod, n, coarse_size):
+    torch, G, O = _pair(oracle_mod, 2, n, coarse_size=coarse_size, level_smoother=1)
+    assert G.info.coarse_rows == O.level(O.levels() - 1)["A"].shape[0]
+    b = np.random.default_rng(n).standard_normal(G.nH)
+    _close(G.apply_vcycle(torch.tensor(b, device="cuda")).cpu().numpy(), O.vcycle(b), 1e-11)
