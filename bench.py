@@ -338,6 +338,8 @@ def smoother_layout_name(code):
         return "CSR, lanes per colour"
     if code < -1:
         return f"one cooperative launch, CSR x{-code} lanes"
+    if code > 500:
+        return f"interleaved slices, {code - 500} lanes per ordinary row"
     if code > 400:
         return f"CSR x{code % 100} lanes, grid-stride over the resident blocks"
     if code > 100:

@@ -80,7 +80,8 @@ typedef struct {
                              while loop; 0: eager launches, host checks every iteration [1] */
     int spmv_threads;     /* threads per row of the fine SpMV and smoother: 4, 8, 16 or
                              32; 0 = pick by mean row length [0] */
-    int smoother_layout;  /* fine smoother layout (SGS): 0 = autotuned at setup [0];
+    int smoother_layout;  /* fine smoother layout (SGS): 0 = interleaved slices, one
+                             launch per colour phase, shaped by the sizes [0];
                              1 = one launch per colour phase, CSR, lanes fitted per colour;
                              2 = per phase, SELL-32; 3 = per phase, CSR with 2 lanes per
                              row; 4, 8, 16 = per phase, CSR with that many lanes per row;
@@ -138,7 +139,8 @@ typedef struct {
     double setup_ms, assemble_ms;
     int spmv_layout;        /* autotuned layout of the fine SpMV: 0 = SELL-32 (one thread
                                per row), t > 0 = CSR read by t lanes per row */
-    int smoother_layout;    /* same for the fine smoother's colour phases; -1 = CSR with
+    int smoother_layout;    /* same for the fine smoother's colour phases; 500 + t = interleaved
+                               slices, t lanes for an ordinary row; -1 = CSR with
                                lanes fitted per colour; 100 + t = t lanes, two rows per
                                lane group; 400 + t = t lanes, grid-stride over the resident
                                blocks; -t (t > 1) = the whole symmetric sweep in one

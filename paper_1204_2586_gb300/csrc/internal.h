@@ -105,6 +105,20 @@ struct DSell {
     std::vector<int64_t> coff;
 };
 
+// Interleaved slices of the parts of a colour split (slices.cu). Slice s is one warp's
+// work: meta[s] = {base low, base high, first place, steps | log2(lanes) << 20 | rows << 24};
+// row r of it is rows[first place + r]; colour c owns slices off[c]..off[c+1]-1.
+struct DSlices {
+    int t0 = 0, steps = 0, nb = 4;  // lanes of an ordinary row, most steps before its lanes
+                                    // double, steps loaded per batch
+    int64_t nslices = 0, entries = 0;
+    int4 *meta = nullptr;
+    int32_t *rows = nullptr, *col = nullptr;
+    double *val = nullptr, *dinv = nullptr;  // FP64 or FP32, as the smoother runs
+    float *val32 = nullptr, *dinv32 = nullptr;
+    std::vector<int64_t> off;  // first slice of each colour
+};
+
 struct Level {
     DCSR A;        // level matrix
     DSplit sp;     // colour split of A
@@ -187,6 +201,8 @@ struct pkasp_problem {
     pk::DSplit fine;      // colour split of A_h
     pk::DSell Asell;      // SELL-32 copy of A_h (natural order)
     pk::DSell fsl, fsu;   // SELL-32 colour-sorted lower / upper parts of A_h
+    pk::DSlices fll, flu, flf;  // interleaved slices of A_h: lower parts, upper parts, whole
+                                // rows (multiplicative form only)
     double *d_l1h = nullptr;
     float *d_l1h32 = nullptr;
     std::vector<pk::Level> lev;
@@ -197,7 +213,7 @@ struct pkasp_problem {
     unsigned *d_bar = nullptr;      // grid-barrier arrivals / exits of the persistent smoother
     int *d_bar_err = nullptr;       // set when one of its barriers timed out
     int spmv_tpr = 4;   // lanes per row of the fine SpMV (autotuned at setup)
-    int fine_tpr = 4;   // lanes per row of the fine smoother phases (autotuned at setup)
+    int fine_tpr = 4;   // layout code of the fine smoother phases (pkasp_info.smoother_layout)
     // solve work (sized for ncols = 1 at setup, grown on demand)
     int work_cols = 0;
     double *w_r = nullptr, *w_z = nullptr, *w_p = nullptr, *w_q = nullptr, *w_x = nullptr,
@@ -335,6 +351,10 @@ int stokes_solve(pkasp_problem *p, const double *b, double *x, pkasp_stats *st, 
 const DCSR *stokes_matrix(const pkasp_problem *p, int which);  // -1 B, -2 B^T, -3 M_p
 void stokes_sizes(const pkasp_problem *p, int64_t *out5);
 float time_kernel(pkasp_problem *p, int which, int reps, cudaStream_t s);
+
+// interleaved slices (slices.cu): part 0 lower, 1 upper parts of the split, 2 whole rows
+void build_slices(DevPool &pool, const DCSR &A, const DSplit &sp, int part, int t0, int steps, bool fp32, DSlices &S,
+                  cudaStream_t s);
 
 // SELL-32 builders (sell.cu)
 void build_sell_natural(DevPool &pool, const DCSR &A, DSell &S, bool want32, cudaStream_t s);

@@ -347,6 +347,67 @@ __global__ void __launch_bounds__(kBlock) k_gs_phase(int64_t pb, int64_t pe, con
     if (lead) y[i] = BACK ? own - acc * di : (own - acc) * di;
 }
 
+// One colour phase over interleaved slices (slices.cu), one warp per slice: W steps of 32
+// entries, T lanes per row; the sums are those of k_gs_phase with T lanes. Over whole rows
+// (r = b) the BACK = false form is a phase of a full sweep, y_i = (b_i - sum a_ij y_j) / a_ii.
+//
+// Small phases are bound by their chain of dependent accesses and FP64 adds, large ones by
+// the L2 sectors and L1 lines they touch. In the row-pointer layout a group of 4 lanes reads
+// 16 unaligned bytes of columns and 32 of values per step: 0.59 lines an entry besides the
+// 0.39 of the gathers (host count at P4 7^3). A slice's step is one line of columns and two
+// of values: 0.1 lines an entry. FP64 S_k, us before -> after (graph replays): P4 48^3
+// 2325 -> 1827, P4 24^3 597 -> 454, P3 32^3 359 -> 283, P2 33^3 129 -> 124, P2 8^3 46 -> 42;
+// FP32: P4 48^3 1379 -> 1240, P3 32^3 191 -> 170, P3 9^3 68 -> 66. At P4 48^3 FP64 it reads
+// about 1.0 sectors an entry at the 300 G sectors/s that random gathers reach there.
+template <int NB, typename PT, typename TR, bool BACK>
+__global__ void __launch_bounds__(kBlock) k_slice_phase(int64_t s0, int64_t s1, const int4 *__restrict__ meta,
+                                                        const int32_t *__restrict__ rows,
+                                                        const PT *__restrict__ dinv, const int32_t *__restrict__ col,
+                                                        const PT *__restrict__ val, const TR *r, PT *y) {
+    pdl_trigger();
+    const int64_t s = s0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (s >= s1) {  // a whole warp
+        pdl_wait();
+        return;
+    }
+    const int4 m = meta[s];
+    const int w = m.w & 0xfffff, lt = (m.w >> 20) & 15, nr = (m.w >> 24) & 255;
+    const int64_t e0 = (((int64_t)m.y << 32) | (uint32_t)m.x) + lane;
+    int c[NB];
+    PT v[NB];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+        const bool in = k < w;
+        c[k] = in ? ldst(&col[e0 + 32 * k]) : -1;
+        v[k] = in ? ldst(&val[e0 + 32 * k]) : PT(0);
+    }
+    const int q = lane >> lt;
+    const bool lead = (lane & ((1 << lt) - 1)) == 0 && q < nr;
+    const int32_t i = lead ? rows[m.z + q] : 0;
+    const PT di = lead ? dinv[m.z + q] : PT(1);
+    pdl_wait();
+    PT own = PT(0);
+    if (lead) own = BACK ? y[i] : (PT)r[i];
+    PT acc = PT(0);
+#pragma unroll
+    for (int k = 0; k < NB; ++k)
+        if (k < w && c[k] >= 0) acc += v[k] * y[c[k]];
+    for (int k0 = NB; k0 < w; k0 += NB) {
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            const bool in = k0 + k < w;
+            c[k] = in ? ldst(&col[e0 + 32 * (int64_t)(k0 + k)]) : -1;
+            v[k] = in ? ldst(&val[e0 + 32 * (int64_t)(k0 + k)]) : PT(0);
+        }
+#pragma unroll
+        for (int k = 0; k < NB; ++k)
+            if (k0 + k < w && c[k] >= 0) acc += v[k] * y[c[k]];
+    }
+    for (int o = 1 << lt >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+    if (lead) y[i] = BACK ? own - acc * di : (own - acc) * di;
+}
+
 // The loads of a colour phase without its dependency: every position of [0, n) at
 // once, out[i] = dinv_i * sum_part a_ij x_j with x read-only (a measurement of the
 // smoother's memory work without the barriers between colours; not used by a solve).

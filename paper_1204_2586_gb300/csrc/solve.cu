@@ -32,7 +32,7 @@ namespace {
 // ---------------------------------------------------------------------------------
 // Lanes per row. Short sub-warps keep more rows, and more independent loads per lane,
 // in flight: on GB300 four lanes beat sixteen by 1.7x on the P3 matrix (47 entries per
-// row). The fine SpMV and the fine smoother are autotuned at setup instead.
+// row). The fine SpMV is autotuned at setup instead, the fine smoother takes slices.
 int tpr_for(double mean_row) {
     if (mean_row <= 96) return 4;
     return 8;
@@ -272,6 +272,23 @@ void gs_backward0(const DSplit &sp, int tpr_fixed, PT *y, cudaStream_t s,
     }
 }
 
+// One sweep over the colours' interleaved slices, ascending or descending: BACK as in
+// k_slice_phase.
+template <typename PT, typename TR, bool BACK>
+void slice_sweep(const DSlices &S, bool ascending, const TR *r, PT *y, cudaStream_t s,
+                 const cudaAccessPolicyWindow *win) {
+    const int nc = (int)S.off.size() - 1;
+    auto kern = S.nb == 2 ? k_slice_phase<2, PT, TR, BACK>
+                : S.nb == 4 ? k_slice_phase<4, PT, TR, BACK> : k_slice_phase<6, PT, TR, BACK>;
+    for (int q = 0; q < nc; ++q) {
+        const int c = ascending ? q : nc - 1 - q;
+        const int64_t s0 = S.off[c], s1 = S.off[c + 1];
+        if (s1 <= s0) continue;
+        launch_pdl_w(kern, rows_grid(s1 - s0, 32), s, win, s0, s1, (const int4 *)S.meta, (const int32_t *)S.rows,
+                     pick<PT>(S.dinv, S.dinv32), (const int32_t *)S.col, pick<PT>(S.val, S.val32), r, y);
+    }
+}
+
 // full backward GS sweep on A x = b from the current x
 template <typename PT>
 void gs_backward_full(const DSplit &sp, int tpr_fixed, const PT *b, PT *x, cudaStream_t s,
@@ -479,6 +496,11 @@ void smoother(pkasp_problem *p, const double *r, PT *zs, cudaStream_t s) {
     }
     cudaAccessPolicyWindow wb;
     const cudaAccessPolicyWindow *win = smoother_window<PT>(p, zs, wb);
+    if (ts > 500) {
+        slice_sweep<PT, double, false>(p->fll, true, r, zs, s, win);
+        slice_sweep<PT, PT, true>(p->flu, false, zs, zs, s, win);
+        return;
+    }
     gs_forward0<PT, double>(p->fine, ts, r, zs, s, win);
     gs_backward0<PT>(p->fine, ts, zs, s, win);
 }
@@ -520,8 +542,10 @@ void precondition(pkasp_problem *p, const double *r, double *z, cudaStream_t s, 
     // multiplicative: forward GS (or l1 step) from zero, coarse correction of the new
     // residual, backward GS sweep (or l1 step) from the corrected iterate
     const bool jac = p->opt.smoother == PKASP_SMOOTHER_L1JACOBI;
-    // the forward half sweep takes the tuned layout (SELL-32 maps to lanes fitted per
-    // colour); the full backward sweep uses the CSR split with one row per lane group
+    // the forward half sweep takes the chosen layout (SELL-32 maps to lanes fitted per
+    // colour); the full backward sweep uses slices of whole rows, or with an explicit layout
+    // the CSR split with one row per lane group
+    const bool slices = p->fine_tpr > 500;
     const int tfw = p->fine_tpr > 0 ? p->fine_tpr : -1;
     const int ts = p->fine_tpr > 0 ? p->fine_tpr % 100 : -1;
     // the residuals read the CSR form (a SELL-32 choice of the autotuner maps to the
@@ -534,7 +558,9 @@ void precondition(pkasp_problem *p, const double *r, double *z, cudaStream_t s, 
         PK_LAUNCH();
     } else {
         cudaAccessPolicyWindow wb;
-        gs_forward0<PT, double>(p->fine, tfw, r, zs, s, smoother_window<PT>(p, zs, wb));
+        const cudaAccessPolicyWindow *win = smoother_window<PT>(p, zs, wb);
+        if (slices) slice_sweep<PT, double, false>(p->fll, true, r, zs, s, win);
+        else gs_forward0<PT, double>(p->fine, tfw, r, zs, s, win);
     }
     to_pt<PT>(r, rr, p->nh, s);
     PK_TPR_SWITCH(ta, (k_residual<TPR, PT, PT, PT><<<rows_grid(p->nh, TPR), kBlock, 0, s>>>(
@@ -554,7 +580,9 @@ void precondition(pkasp_problem *p, const double *r, double *z, cudaStream_t s, 
         PK_LAUNCH();
     } else {
         cudaAccessPolicyWindow wb;
-        gs_backward_full<PT>(p->fine, ts, (const PT *)rr, zs, s, smoother_window<PT>(p, zs, wb));
+        const cudaAccessPolicyWindow *win = smoother_window<PT>(p, zs, wb);
+        if (slices) slice_sweep<PT, PT, false>(p->flf, false, rr, zs, s, win);
+        else gs_backward_full<PT>(p->fine, ts, (const PT *)rr, zs, s, win);
     }
     k_copy_to<PT><<<elem_grid(p->nh), kBlock, 0, s>>>(p->nh, zs, z);
     PK_LAUNCH();
@@ -996,6 +1024,9 @@ void free_setup(pkasp_problem *p) {
     p->Asell = DSell{};
     p->fsl = DSell{};
     p->fsu = DSell{};
+    p->fll = DSlices{};
+    p->flu = DSlices{};
+    p->flf = DSlices{};
     p->d_l1h = nullptr;
     p->d_l1h32 = nullptr;
     p->d_cinv = nullptr;
@@ -1007,9 +1038,61 @@ void free_setup(pkasp_problem *p) {
     p->have_setup = false;
 }
 
-// Lanes-per-row autotuner for the two hot fine-level kernels: every candidate runs a few
-// times on the actual matrix (inputs f_h) and the fastest is kept. A fixed
-// options.spmv_threads bypasses it.
+// Shape of the interleaved slices: lanes t0 of an ordinary row, steps it takes before its
+// lanes double, entries loaded per batch. `entries` is the mean of a colour phase, `part`
+// the mean of a row's part. Measured with graph replays of S_k (us, all sizes in both
+// precisions; the lines lie between the sizes where the order changes):
+//  - small phases have too few rows to fill the chip: two steps, the shortest chain. FP64
+//    below 14000 entries (P2 8^3: 41 against 50 with 6 steps; P2 14^3, 14000: 60 against 64;
+//    P3 12^3, 41000: 149 against 122), FP32, whose adds cost nothing, with eight lanes below
+//    110000 (P3 16^3, 100000: 80 against 86 with 4 lanes and steps; P3 24^3, 330000: 118
+//    against 109) or, for the longer rows of P4, 60000 (8^3, 27000: 125 against 135; 12^3,
+//    95000: 159 against 147). P1's rows (parts of 7 entries) always (64^3 FP64: 68 with 2
+//    lanes against 74 with 6 steps; FP32: 35 with 4 lanes against 48).
+//  - then FP64 takes 2 lanes, since every shuffle add costs a warp-wide FP64 slot, and one
+//    batch of 6 steps (P3 32^3: 283 against 332 with 4 lanes and 4 steps); FP32 4 lanes and
+//    4 steps (P3 32^3: 170 against 183), or 2 and 6 for P4's rows (16^3: 163 against 176).
+//  - above 10^6 (FP64) and 2 10^6 (FP32) entries the L2 rate counts: fewer lanes that double
+//    late, so more of a step's entries belong to one row. FP64 P4 48^3 1827 with 4 lanes,
+//    16 steps and batches of 4 (fewer registers, so more warps) against 1948 with
+//    batches of 6; P4 32^3 769 with batches of 6 against 823; P2 64^3 298 with 2 lanes
+//    against 324 with 4. FP32 P4 48^3 1240 against 1276 with batches of 4.
+struct SliceShape {
+    int t0, steps, nb;
+};
+SliceShape slice_shape(bool fp32, double entries, double part) {
+    if (part < 9) return {fp32 ? 4 : 2, 2, 2};
+    if (fp32) {
+        if (entries < (part < 30 ? 110e3 : 60e3)) return {8, 2, 2};
+        if (entries >= 2e6) return {4, 16, 6};
+        return part < 30 || entries >= 1e6 ? SliceShape{4, 4, 4} : SliceShape{2, 6, 6};
+    }
+    if (entries < 14e3) return {2, 2, 2};
+    if (entries < 1e6) return {2, 6, 6};
+    if (part < 18) return {2, 16, 6};
+    return entries < 2.2e6 ? SliceShape{4, 16, 6} : SliceShape{4, 16, 4};
+}
+
+// builds the fine smoother's slices; returns the layout code 500 + lanes of an ordinary row
+int fine_slices(pkasp_problem *p, cudaStream_t s) {
+    const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
+    const double n = std::max<double>(1.0, (double)p->nh), nc = std::max(1, p->fine.ncol);
+    const double part = (double)(p->Ah.nnz - p->nh) / 2 / n;
+    const SliceShape h = slice_shape(fp32, n * part / nc, part);
+    auto build = [&](int which, const SliceShape &q, DSlices &S) {
+        build_slices(p->setup_pool, p->Ah, p->fine, which, q.t0, q.steps, fp32, S, s);
+        S.nb = q.nb;
+    };
+    build(0, h, p->fll);
+    build(1, h, p->flu);
+    if (p->opt.mode == PKASP_MODE_MULTIPLICATIVE) build(2, slice_shape(fp32, n * 2 * part / nc, 2 * part), p->flf);
+    return 500 + h.t0;
+}
+
+// Layouts of the two hot fine-level kernels. The SpMV's lanes per row are autotuned: every
+// candidate runs a few times on the actual matrix (inputs f_h) and the fastest is kept. The
+// smoother takes interleaved slices. A fixed options.spmv_threads bypasses both, a fixed
+// options.smoother_layout the second.
 void autotune(pkasp_problem *p, cudaStream_t s) {
     if (p->opt.spmv_threads) {
         p->spmv_tpr = p->fine_tpr = p->opt.spmv_threads;
@@ -1050,28 +1133,13 @@ void autotune(pkasp_problem *p, cudaStream_t s) {
             if (best[k] < best[pick]) pick = k;
         return cand[pick];
     };
-    // 0: SELL-32, one thread per row; t > 0: CSR with t lanes per row; -1 (smoother
-    // only): CSR with the lanes of each colour phase fitted to its longest row
+    // 0: SELL-32, one thread per row; t > 0: CSR with t lanes per row
     const int cand_spmv[] = {0, 2, 4, 8};
-    // 100 + t: t lanes, two rows per sub-warp. The one-launch cooperative sweep (-t) is
-    // not a candidate: its grid barrier cost more than a phase launch on every measured
-    // problem (P3 32^3, P4 48^3); smoother_layout selects it explicitly.
-    // (2 lanes per row, layouts 3 and 102, lost on every measured problem: P3 32^3 FP64
-    // 769 vs 467 us; they stay selectable through smoother_layout)
-    // 400 + t: t lanes, grid-stride over the resident blocks, the next row's static loads
-    // in flight during the current row's gathers.
-    const int cand_fine[] = {-1, 4, 8, 16, 104, 108, 116, 404, 408, 416};
     const int pick_spmv = tune(cand_spmv, 4, &p->spmv_tpr, [&] { spmv_fine(p, p->d_b, p->w_q, s); });
     p->spmv_tpr = pick_spmv;
     int pick_fine = -1;
-    if (p->opt.smoother == PKASP_SMOOTHER_SGS && p->opt.smoother_layout != 0) {
-        pick_fine = fixed_fine;
-    } else if (p->opt.smoother == PKASP_SMOOTHER_SGS) {
-        if (p->opt.precond_precision == PKASP_PREC_FP32)
-            pick_fine = tune(cand_fine, 10, &p->fine_tpr, [&] { smoother<float>(p, p->d_b, p->w_zs32, s); });
-        else
-            pick_fine = tune(cand_fine, 10, &p->fine_tpr, [&] { smoother<double>(p, p->d_b, p->w_zs, s); });
-    }
+    if (p->opt.smoother == PKASP_SMOOTHER_SGS)
+        pick_fine = p->opt.smoother_layout != 0 ? fixed_fine : fine_slices(p, s);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     p->spmv_tpr = pick_spmv;

@@ -1,8 +1,9 @@
-"""The device-side setup at the edges of its kernels, against the oracle: Galerkin and
+"""The device-side setup and its layouts at the edges of their kernels. Galerkin and
 interpolation rows that overflow the first column table (more than 512 distinct columns,
 plain AMG on P4 matrices), and coarsest inverses whose size is below, at and above a
-multiple of the 32-row pivot block. Integer decisions are exact; values are held to the
-tolerance of the other setup tests (1e-12 of the largest entry), cycles to 1e-11."""
+multiple of the 32-row pivot block, against the oracle; the interleaved slices. Integer
+decisions are exact; values are held to the tolerance of the other setup tests (1e-12 of
+the largest entry), cycles to 1e-11."""
 import numpy as np
 import pytest
 
@@ -29,7 +30,7 @@ def _pair(oracle_mod, k, n, **kw):
     return torch, G, O
 
 
-@pytest.mark.parametrize("k,n,theta", [(4, 5, 0.0), (3, 6, 0.0)])
+@pytest.mark.parametrize("k,n,theta", [(4, 6, 0.004), (3, 7, 0.01)])
 def test_rows_with_many_columns(oracle_mod, k, n, theta):
     _, G, O = _pair(oracle_mod, k, n, mode=2, theta=theta, coarse_size=20)
     longest = 0
@@ -55,3 +56,31 @@ def test_coarsest_inverse(oracle_mod, n, coarse_size):
     assert G.info.coarse_rows == O.level(O.levels() - 1)["A"].shape[0]
     b = np.random.default_rng(n).standard_normal(G.nH)
     _close(G.apply_vcycle(torch.tensor(b, device="cuda")).cpu().numpy(), O.vcycle(b), 1e-11)
+
+
+# one size for each shape of the interleaved slices (lanes, steps, batch), both precisions,
+# and the whole-row slices of the multiplicative form's full sweep
+@pytest.mark.parametrize("k,n,prec,mode", [(2, 2, 0, 0), (1, 9, 0, 0), (1, 9, 1, 0), (3, 12, 0, 0), (2, 64, 0, 0),
+                                           (3, 40, 0, 0), (4, 40, 0, 0), (3, 9, 1, 0), (3, 24, 1, 0), (4, 12, 1, 0),
+                                           (4, 40, 1, 0), (2, 5, 0, 1), (3, 12, 0, 1), (4, 10, 1, 1)])
+def test_slices_match_rows(k, n, prec, mode):
+    """The default sweep over slices against the row layout with 4 lanes (itself held to the
+    oracle elsewhere). Both add a row's products in some order: a sum of L terms is off by
+    at most L u sum|a y|, and the 2 C phases pass it on."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, k, kappa_lognormal(t.shape[0], 1))
+    r = torch.randn(P.nh, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    out = []
+    for layout in (4, 0):
+        P.setup(smoother_layout=layout, precond_precision=prec, mode=mode, level_smoother=1)
+        assert (P.info.smoother_layout > 500) == (layout == 0)
+        out.append(P.apply_prec(r) if mode else P.apply_smoother(r))
+    longest = 400 if k == 4 else 200
+    u = 2.0 ** -24 if prec else 2.0 ** -53
+    assert (out[1] - out[0]).norm() <= 2 * P.info.fine_colours * longest * u * out[0].norm()
+    P.close()
