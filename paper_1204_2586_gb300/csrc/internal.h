@@ -209,6 +209,9 @@ struct pkasp_problem {
     double *d_cinv = nullptr;  // dense inverse of the coarsest matrix
     float *d_cinv32 = nullptr;
     int64_t nc = 0;
+    int tail = 0;               // level from which one right-hand side's V-cycle is a dense product
+    double *d_tail = nullptr;   // its matrix (FP64 or FP32, as the cycle runs; tail.cu); the
+    float *d_tail32 = nullptr;  // coarsest inverse when tail is the coarsest level
     int64_t *d_fine_off = nullptr;  // device copy of fine.off (persistent smoother)
     unsigned *d_bar = nullptr;      // grid-barrier arrivals / exits of the persistent smoother
     int *d_bar_err = nullptr;       // set when one of its barriers timed out
@@ -355,6 +358,9 @@ float time_kernel(pkasp_problem *p, int which, int reps, cudaStream_t s);
 // interleaved slices (slices.cu): part 0 lower, 1 upper parts of the split, 2 whole rows
 void build_slices(DevPool &pool, const DCSR &A, const DSplit &sp, int part, int t0, int steps, bool fp32, DSlices &S,
                   cudaStream_t s);
+
+// the dense tail of the V-cycle (tail.cu); after the hierarchy and the coarsest inverse
+void build_tail(pkasp_problem *p, cudaStream_t s);
 
 // SELL-32 builders (sell.cu)
 void build_sell_natural(DevPool &pool, const DCSR &A, DSell &S, bool want32, cudaStream_t s);

@@ -327,12 +327,12 @@ template <typename PT>
 void vcycle(pkasp_problem *p, int l, cudaStream_t s, bool pre_done = false);
 
 // b_l = R x (R = I_P^T into level 0, or level l-1's restriction); with l1-Jacobi level
-// smoothing on a level that is not the coarsest, the same pass also takes the
+// smoothing on a level above the dense tail, the same pass also takes the
 // pre-smoothing step from zero, x_l = b_l / l1 (returns true then).
 template <typename PT, typename XT>
 bool restrict_to(pkasp_problem *p, const DCSR &R, const XT *x, int l, cudaStream_t s) {
     Level &L = p->lev[l];
-    const bool fuse = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI && l < (int)p->lev.size() - 1;
+    const bool fuse = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI && l < p->tail;
     if (!fuse || R.n == 0) {
         spmv<PT, PT>(R, x, lv_b<PT>(L), tpr_of(R), s);
         return false;
@@ -358,9 +358,9 @@ template <typename PT>
 void vcycle(pkasp_problem *p, int l, cudaStream_t s, bool pre_done) {
     Level &L = p->lev[l];
     const int64_t n = L.A.n;
-    if (l == (int)p->lev.size() - 1) {
-        k_dense_mv<PT><<<rows_grid(n, 32), kBlock, 0, s>>>(n, pick<PT>(p->d_cinv, p->d_cinv32), lv_b<PT>(L),
-                                                          lv_x<PT>(L));
+    if (l == p->tail) {
+        k_dense_mv<PT><<<(unsigned)((n + 3) / 4), 128, 0, s>>>(n, pick<PT>(p->d_tail, p->d_tail32), lv_b<PT>(L),
+                                                               lv_x<PT>(L));
         PK_LAUNCH();
         return;
     }
@@ -1030,6 +1030,9 @@ void free_setup(pkasp_problem *p) {
     p->d_l1h = nullptr;
     p->d_l1h32 = nullptr;
     p->d_cinv = nullptr;
+    p->d_tail = nullptr;
+    p->d_tail32 = nullptr;
+    p->tail = 0;
     p->d_fine_off = nullptr;
     p->d_bar = nullptr;
     p->d_bar_err = nullptr;
@@ -1220,6 +1223,7 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
         p->d_cinv32 = pool.get<float>(std::max<int64_t>(p->nc * p->nc, 1));
         to32(p->d_cinv, p->d_cinv32, p->nc * p->nc, s);
     }
+    build_tail(p, s);
     if (!p->aux_stream) PK_CUDA(cudaStreamCreateWithFlags(&p->aux_stream, cudaStreamNonBlocking));
     if (!p->cap_stream) PK_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
     if (!p->ev_fork) PK_CUDA(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));

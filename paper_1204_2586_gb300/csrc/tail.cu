@@ -1,0 +1,200 @@
+// tail.cu -- the dense tail of the V-cycle. On a small level the cycle from there down is a
+// chain of launches that each move a few kilobytes: with Gauss-Seidel levels one per colour
+// and sweep (402 rows still have 53 colours), each 2-4 us. But V is a fixed linear operator
+// of b, so setup applies it to the identity (all columns at once, from the coarsest level
+// up) and the solve multiplies by that n x n matrix, as it always did with the coarsest
+// inverse: one launch that reads n^2 entries. The matrix is formed in FP64.
+//
+// One column block of a level is 256 threads wide; a thread carries one column through the
+// row sums, so reads of the dense operand are coalesced and the matrix entry is a broadcast.
+#include <algorithm>
+
+#include "internal.h"
+
+namespace pk {
+namespace {
+
+constexpr int kCols = 128;  // columns of a block
+
+unsigned tiles(int64_t n) { return (unsigned)((n + kCols - 1) / kCols); }
+
+// Y_r = c0 * I_r + Y_r * keep + scale_r * (sum_e a_e X_e) with rows r = rows[p] (or p)
+//   rows/ptr per position p; one block per position and column block
+__global__ void __launch_bounds__(kCols) k_tail_rows(int64_t n, int64_t p0, const int32_t *__restrict__ rows,
+                                                     const int64_t *__restrict__ ptr,
+                                                     const int32_t *__restrict__ col, const double *__restrict__ val,
+                                                     const double *X, double *Y, double ident, double keep,
+                                                     double sign) {
+    const int64_t p = p0 + blockIdx.x, c = (int64_t)blockIdx.y * kCols + threadIdx.x;
+    if (c >= n) return;
+    const int64_t r = rows ? rows[p] : p;
+    double acc = 0.0;
+    const int64_t hi = ptr[p + 1];
+    for (int64_t e = ptr[p]; e < hi; ++e) acc += val[e] * X[(int64_t)col[e] * n + c];
+    const double own = keep != 0.0 ? keep * Y[r * n + c] : 0.0;
+    Y[r * n + c] = (r == c ? ident : 0.0) + own + sign * acc;
+}
+
+// one Gauss-Seidel colour: X_r = (I_r - sum_lower a X - [full] sum_upper a X) * dinv
+__global__ void __launch_bounds__(kCols) k_tail_gs(int64_t n, int64_t p0, const int32_t *__restrict__ rows,
+                                                   const int64_t *__restrict__ lptr,
+                                                   const int32_t *__restrict__ lcol,
+                                                   const double *__restrict__ lval, const int64_t *__restrict__ uptr,
+                                                   const int32_t *__restrict__ ucol,
+                                                   const double *__restrict__ uval, const double *__restrict__ dinv,
+                                                   int full, double *X) {
+    const int64_t p = p0 + blockIdx.x, c = (int64_t)blockIdx.y * kCols + threadIdx.x;
+    if (c >= n) return;
+    const int64_t r = rows[p];
+    double acc = 0.0;
+    for (int64_t e = lptr[p]; e < lptr[p + 1]; ++e) acc += lval[e] * X[(int64_t)lcol[e] * n + c];
+    if (full)
+        for (int64_t e = uptr[p]; e < uptr[p + 1]; ++e) acc += uval[e] * X[(int64_t)ucol[e] * n + c];
+    X[r * n + c] = ((r == c ? 1.0 : 0.0) - acc) * dinv[p];
+}
+
+// X = D^{-1} (the l1-Jacobi step from zero on the identity); X += D^{-1} R
+__global__ void k_tail_jacobi0(int64_t n, const double *__restrict__ d, double *__restrict__ X) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n * n) return;
+    const int64_t r = q / n;
+    X[q] = r == q % n ? 1.0 / d[r] : 0.0;
+}
+__global__ void k_tail_jacobi(int64_t n, const double *__restrict__ d, const double *__restrict__ R,
+                              double *__restrict__ X) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n * n) X[q] += R[q] / d[q / n];
+}
+
+// C[m][n] = A[m][k] B[k][n]: 32 x 32 tiles, four rows per thread
+__global__ void __launch_bounds__(256) k_tail_gemm(int64_t m, int64_t n, int64_t k, const double *__restrict__ A,
+                                                   const double *__restrict__ B, double *__restrict__ C) {
+    __shared__ double a[32][33], b[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
+    const int64_t i0 = (int64_t)blockIdx.y * 32, j = (int64_t)blockIdx.x * 32 + tx;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t k0 = 0; k0 < k; k0 += 32) {
+        for (int q = ty; q < 32; q += 8) {
+            a[q][tx] = i0 + q < m && k0 + tx < k ? A[(i0 + q) * k + k0 + tx] : 0.0;
+            b[q][tx] = k0 + q < k && j < n ? B[(k0 + q) * n + j] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int u = 0; u < 32; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[q] += a[ty + 8 * q][u] * b[u][tx];
+        __syncthreads();
+    }
+    if (j >= n) return;
+    for (int q = 0; q < 4; ++q)
+        if (i0 + ty + 8 * q < m) C[(i0 + ty + 8 * q) * n + j] = acc[q];
+}
+
+// Modelled time (us) of one cycle from level l down, as launches. Gauss-Seidel: a launch
+// per colour and sweep, 3.4 us each (P2 21^3 FP64, 202 phases of three levels: 709 us);
+// l1-Jacobi: five launches of 2 us each besides the next level (P2 8^3: 18 us over two
+// levels).
+double launches_us(const Level &L, bool jacobi) { return jacobi ? 11.0 : 10.0 + 2 * 3.4 * L.sp.ncol; }
+// and of the dense product: a launch, then n^2 FMAs at the FP64 pipe's 0.55 10^6 a us (the
+// reads of 8 n^2 bytes at 5 10^6 a us hide behind them), or 4 n^2 bytes at that rate in FP32
+double dense_us(double n, bool fp32) { return 2.5 + n * n / (fp32 ? 1.2e6 : 0.55e6); }
+
+}  // namespace
+
+// Level at which the cycle becomes one dense product: the highest where that is modelled
+// faster than the launches below it, within 5120 rows and 10^10 FMAs of setup work (about
+// 15 ms).
+int tail_level(const pkasp_problem *p) {
+    const bool jacobi = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
+    const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
+    const int last = (int)p->lev.size() - 1;
+    int best = last;
+    double below = dense_us((double)p->lev[last].A.n, fp32);
+    for (int l = last - 1; l >= 0; --l) {
+        const Level &L = p->lev[l];
+        const double n = (double)L.A.n;
+        below += launches_us(L, jacobi);
+        if (L.A.n > 5120 || n * (double)L.A.nnz > 4e9) break;
+        if (dense_us(n, fp32) < below) {
+            best = l;
+            below = dense_us(n, fp32);
+        }
+    }
+    return best;
+}
+
+// M = V on level p->tail, from the coarsest inverse up; into d_tail (or d_tail32)
+void build_tail(pkasp_problem *p, cudaStream_t s) {
+    const int last = (int)p->lev.size() - 1;
+    p->tail = tail_level(p);
+    p->d_tail = p->d_cinv;
+    p->d_tail32 = p->d_cinv32;
+    if (p->tail == last) return;
+    const bool jacobi = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
+    const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
+    DevPool tmp;
+    try {
+        const double *Mc = p->d_cinv;
+        for (int l = last - 1; l >= p->tail; --l) {
+            Level &L = p->lev[l];
+            const int64_t n = L.A.n, nc = L.R.n;
+            // the matrix of the tail itself outlives setup when it is the one in use
+            double *X = (l == p->tail && !fp32 ? p->setup_pool : tmp).get<double>(n * n);
+            double *R = tmp.get<double>(n * n), *B = tmp.get<double>(nc * n), *W = tmp.get<double>(nc * n);
+            const unsigned ct = tiles(n), flat = (unsigned)((n * n + 255) / 256);
+            const DSplit &sp = L.sp;
+            auto gs = [&](int c, int full) {
+                const int64_t pb = sp.off[c], m = sp.off[c + 1] - pb;
+                if (m == 0) return;
+                k_tail_gs<<<dim3((unsigned)m, ct), kCols, 0, s>>>(n, pb, sp.perm, sp.lptr, sp.lcol, sp.lval, sp.uptr,
+                                                                  sp.ucol, sp.uval, sp.dinv, full, X);
+                PK_LAUNCH();
+            };
+            auto residual = [&] {  // R = I - A X
+                k_tail_rows<<<dim3((unsigned)n, ct), kCols, 0, s>>>(n, 0, nullptr, L.A.ptr, L.A.col, L.A.val, X, R,
+                                                                    1.0, 0.0, -1.0);
+                PK_LAUNCH();
+            };
+            if (jacobi) {
+                k_tail_jacobi0<<<flat, 256, 0, s>>>(n, L.l1, X);
+                PK_LAUNCH();
+            } else {
+                for (int c = 0; c < sp.ncol; ++c) gs(c, 0);
+            }
+            residual();
+            k_tail_rows<<<dim3((unsigned)nc, ct), kCols, 0, s>>>(n, 0, nullptr, L.R.ptr, L.R.col, L.R.val, R, B, 0.0,
+                                                                 0.0, 1.0);
+            PK_LAUNCH();
+            k_tail_gemm<<<dim3((unsigned)((n + 31) / 32), (unsigned)((nc + 31) / 32)), 256, 0, s>>>(nc, n, nc, Mc, B,
+                                                                                                   W);
+            PK_LAUNCH();
+            k_tail_rows<<<dim3((unsigned)n, ct), kCols, 0, s>>>(n, 0, nullptr, L.P.ptr, L.P.col, L.P.val, W, X, 0.0,
+                                                                1.0, 1.0);
+            PK_LAUNCH();
+            if (jacobi) {
+                residual();
+                k_tail_jacobi<<<flat, 256, 0, s>>>(n, L.l1, R, X);
+                PK_LAUNCH();
+            } else {
+                for (int c = sp.ncol - 1; c >= 0; --c) gs(c, 1);
+            }
+            Mc = X;
+        }
+        const int64_t n = p->lev[p->tail].A.n;
+        if (fp32) {
+            p->d_tail32 = p->setup_pool.get<float>(n * n);
+            to32(Mc, p->d_tail32, n * n, s);
+            p->d_tail = nullptr;
+        } else {
+            p->d_tail = const_cast<double *>(Mc);
+        }
+        PK_CUDA(cudaStreamSynchronize(s));
+    } catch (...) {
+        cudaStreamSynchronize(s);
+        tmp.free_all();
+        throw;
+    }
+    tmp.free_all();
+}
+
+}  // namespace pk

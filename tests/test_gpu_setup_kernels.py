@@ -84,3 +84,16 @@ def test_slices_match_rows(k, n, prec, mode):
     u = 2.0 ** -24 if prec else 2.0 ** -53
     assert (out[1] - out[0]).norm() <= 2 * P.info.fine_colours * longest * u * out[0].norm()
     P.close()
+
+
+# cycles whose dense tail starts on the first, the second and a deeper level
+@pytest.mark.parametrize("n,level_smoother", [(6, 0), (12, 1), (21, 0), (21, 1), (17, 0)])
+def test_cycle_with_dense_tail(oracle_mod, n, level_smoother):
+    torch, G, O = _pair(oracle_mod, 1, n, level_smoother=level_smoother)
+    assert G.info.levels == O.levels()
+    b = np.random.default_rng(n).standard_normal(G.nH)
+    ref = O.vcycle(b)
+    _close(G.apply_vcycle(torch.tensor(b, device="cuda")).cpu().numpy(), ref, 1e-11)
+    # FP32: row sums of up to 5120 terms on the tail, u = 2^-24
+    G.setup(level_smoother=level_smoother, precond_precision=1)
+    _close(G.apply_vcycle(torch.tensor(b, device="cuda")).cpu().numpy(), ref, 5120 * 2.0 ** -24)
