@@ -152,8 +152,6 @@ struct Gmres {
         PK_CUDA(cudaGraphInstantiate(&p->gm_graph_exec, g, 0));
         cudaGraphDestroy(gi);
         p->gm_graph = g;
-        p->gm_key_b = b;
-        p->gm_key_x = x;
     }
 };
 
@@ -187,8 +185,6 @@ void free_gmres(pkasp_problem *p) {
     if (p->gm_graph) cudaGraphDestroy(p->gm_graph);
     p->gm_graph_exec = nullptr;
     p->gm_graph = nullptr;
-    p->gm_key_b = nullptr;
-    p->gm_key_x = nullptr;
     p->gm_pool.free_all();
     p->gm_V = p->gm_Z = p->gm_w = p->gm_vin = p->gm_zout = nullptr;
     p->gm_state = nullptr;
@@ -215,15 +211,21 @@ int solve_gmres(pkasp_problem *p, const double *b, double *x, pkasp_stats *st, c
     PK_CUDA(cudaEventCreate(&e1));
     PK_CUDA(cudaEventRecord(e0, s));
     const bool use_graph = p->opt.use_graph != 0;
-    if (use_graph && (!p->gm_graph_exec || p->gm_key_b != b || p->gm_key_x != x)) {
-        PK_CUDA(cudaStreamSynchronize(s));
-        Gmres::build_graph(p, b, x);
+    if (use_graph) {
+        // on the problem's own copies of b and x, as the CG graph (solve.cu)
+        if (!p->gm_graph_exec) {
+            PK_CUDA(cudaStreamSynchronize(s));
+            Gmres::build_graph(p, p->w_b, p->w_x);
+        }
+        PK_CUDA(cudaMemcpyAsync(p->w_b, b, sizeof(double) * p->nh, cudaMemcpyDeviceToDevice, s));
+        PK_CUDA(cudaMemcpyAsync(p->w_x, x, sizeof(double) * p->nh, cudaMemcpyDeviceToDevice, s));
     }
     GmresState hs;
     long long launches = 1;
     const long long eager0 = launch_count();
     if (use_graph) {
         PK_CUDA(cudaGraphLaunch(p->gm_graph_exec, s));
+        PK_CUDA(cudaMemcpyAsync(x, p->w_x, sizeof(double) * p->nh, cudaMemcpyDeviceToDevice, s));
     } else {
         Gmres::init(p, b, x, s);
         for (int pass = 0; pass < p->opt.max_iter + p->opt.max_iter / std::max(m, 1) + 4; ++pass) {

@@ -235,12 +235,7 @@ struct pkasp_problem {
     // graph cache
     cudaGraphExec_t graph_exec = nullptr;
     cudaGraph_t graph = nullptr;
-    int graph_cols = 0;
     long long g_init = 0, g_body = 0, g_final = 0;  // kernels per graph part
-    int64_t graph_ld = 0;
-    const void *graph_key_b = nullptr;
-    void *graph_key_x = nullptr;
-    cudaStream_t graph_stream = nullptr;
     // several right-hand sides: blocks [n][NC] (batched.cu), sized for one width NC
     pk::DevPool bwork_pool;
     int bwork_nc = -1, bwork_hist = 0;
@@ -265,8 +260,6 @@ struct pkasp_problem {
     pk::GmresState *gm_state = nullptr;
     cudaGraphExec_t gm_graph_exec = nullptr;
     cudaGraph_t gm_graph = nullptr;
-    const void *gm_key_b = nullptr;
-    void *gm_key_x = nullptr;
     long long gm_g_init = 0, gm_g_body = 0;
     // Taylor-Hood Stokes system (stokes.cpp, stokes.cu), built by pkasp_stokes_setup
     pk::StokesWork *st = nullptr;

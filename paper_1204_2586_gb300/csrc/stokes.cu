@@ -37,8 +37,7 @@ struct StokesWork {
     int hist_cap = 0;
     cudaGraphExec_t exec = nullptr;
     cudaGraph_t graph = nullptr;
-    const void *key_b = nullptr;
-    void *key_x = nullptr;
+    double *bin = nullptr, *xin = nullptr;  // the graph's copies of b and x
     long long g_init = 0, g_body = 0;
 };
 
@@ -372,8 +371,6 @@ struct StokesGmres {
         PK_CUDA(cudaGraphInstantiate(&S.exec, g, 0));
         cudaGraphDestroy(gi);
         S.graph = g;
-        S.key_b = b;
-        S.key_x = x;
     }
 };
 
@@ -393,6 +390,8 @@ void ensure_fgmres(StokesWork &S, int m, int hist_cap) {
     S.vin = w.get<double>(n);
     S.zout = w.get<double>(n);
     S.y = w.get<double>(n);
+    S.bin = w.get<double>(n);
+    S.xin = w.get<double>(n);
     S.H = w.get<double>((size_t)(m + 1) * m);
     S.g = w.get<double>(m + 1);
     S.cs = w.get<double>(m);
@@ -525,13 +524,19 @@ int stokes_solve(pkasp_problem *p, const double *b, double *x, pkasp_stats *st, 
     PK_CUDA(cudaEventCreate(&e1));
     PK_CUDA(cudaEventRecord(e0, s));
     const bool use_graph = p->opt.use_graph != 0;
-    if (use_graph && (!S.exec || S.key_b != b || S.key_x != x)) {
-        PK_CUDA(cudaStreamSynchronize(s));
-        StokesGmres::build_graph(p, b, x);
+    if (use_graph) {
+        // on the solver's own copies of b and x, as the CG graph (solve.cu)
+        if (!S.exec) {
+            PK_CUDA(cudaStreamSynchronize(s));
+            StokesGmres::build_graph(p, S.bin, S.xin);
+        }
+        PK_CUDA(cudaMemcpyAsync(S.bin, b, sizeof(double) * S.n, cudaMemcpyDeviceToDevice, s));
+        PK_CUDA(cudaMemcpyAsync(S.xin, x, sizeof(double) * S.n, cudaMemcpyDeviceToDevice, s));
     }
     const long long eager0 = launch_count();
     if (use_graph) {
         PK_CUDA(cudaGraphLaunch(S.exec, s));
+        PK_CUDA(cudaMemcpyAsync(x, S.xin, sizeof(double) * S.n, cudaMemcpyDeviceToDevice, s));
     } else {
         StokesGmres::init(p, b, x, s);
         for (int pass = 0; pass < p->opt.max_iter + p->opt.max_iter / m + 4; ++pass) {
