@@ -122,6 +122,7 @@ struct DSlices {
 struct Level {
     DCSR A;        // level matrix
     DSplit sp;     // colour split of A
+    DSlices fl, ff;  // its lower parts and whole rows (Gauss-Seidel levels above the tail)
     DCSR P, R;     // interpolation to the next level and its transpose
     double *l1 = nullptr;  // row 1-norms
     float *l132 = nullptr;

@@ -365,7 +365,7 @@ void vcycle(pkasp_problem *p, int l, cudaStream_t s, bool pre_done) {
         return;
     }
     const bool jac = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
-    const int ta = tpr_of(L.A), ts = -1;  // lanes per colour phase chosen per colour
+    const int ta = tpr_of(L.A);
     if (jac) {
         if (!pre_done) {
             k_jacobi0<PT, PT><<<elem_grid(n), kBlock, 0, s>>>(n, pick<PT>(L.l1, L.l132), lv_b<PT>(L),
@@ -373,7 +373,7 @@ void vcycle(pkasp_problem *p, int l, cudaStream_t s, bool pre_done) {
             PK_LAUNCH();
         }
     } else {
-        gs_forward0<PT, PT>(L.sp, ts, lv_b<PT>(L), lv_x<PT>(L), s);
+        slice_sweep<PT, PT, false>(L.fl, true, lv_b<PT>(L), lv_x<PT>(L), s, nullptr);
     }
     PK_TPR_SWITCH(ta, (k_residual<TPR, PT, PT, PT><<<rows_grid(n, TPR), kBlock, 0, s>>>(
                           n, L.A.ptr, L.A.col, pick<PT>(L.A.val, L.A.val32), lv_b<PT>(L), lv_x<PT>(L),
@@ -394,7 +394,7 @@ void vcycle(pkasp_problem *p, int l, cudaStream_t s, bool pre_done) {
         k_add_div<PT><<<elem_grid(n), kBlock, 0, s>>>(n, lv_r<PT>(L), pick<PT>(L.l1, L.l132), lv_x<PT>(L));
         PK_LAUNCH();
     } else {
-        gs_backward_full<PT>(L.sp, ts, lv_b<PT>(L), lv_x<PT>(L), s);
+        slice_sweep<PT, PT, false>(L.ff, false, lv_b<PT>(L), lv_x<PT>(L), s, nullptr);
     }
 }
 
@@ -1074,20 +1074,22 @@ SliceShape slice_shape(bool fp32, double entries, double part) {
     return entries < 2.2e6 ? SliceShape{4, 16, 6} : SliceShape{4, 16, 4};
 }
 
+// slices of part `which` (build_slices) of A's split, shaped for its mean phase and row
+void shaped_slices(pkasp_problem *p, const DCSR &A, const DSplit &sp, int which, DSlices &S, cudaStream_t s) {
+    const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
+    const double n = std::max<double>(1.0, (double)A.n), nc = std::max(1, sp.ncol);
+    const double part = (double)(A.nnz - A.n) / (which == 2 ? 1 : 2) / n;
+    const SliceShape h = slice_shape(fp32, n * part / nc, part);
+    build_slices(p->setup_pool, A, sp, which, h.t0, h.steps, fp32, S, s);
+    S.nb = h.nb;
+}
+
 // builds the fine smoother's slices; returns the layout code 500 + lanes of an ordinary row
 int fine_slices(pkasp_problem *p, cudaStream_t s) {
-    const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
-    const double n = std::max<double>(1.0, (double)p->nh), nc = std::max(1, p->fine.ncol);
-    const double part = (double)(p->Ah.nnz - p->nh) / 2 / n;
-    const SliceShape h = slice_shape(fp32, n * part / nc, part);
-    auto build = [&](int which, const SliceShape &q, DSlices &S) {
-        build_slices(p->setup_pool, p->Ah, p->fine, which, q.t0, q.steps, fp32, S, s);
-        S.nb = q.nb;
-    };
-    build(0, h, p->fll);
-    build(1, h, p->flu);
-    if (p->opt.mode == PKASP_MODE_MULTIPLICATIVE) build(2, slice_shape(fp32, n * 2 * part / nc, 2 * part), p->flf);
-    return 500 + h.t0;
+    shaped_slices(p, p->Ah, p->fine, 0, p->fll, s);
+    shaped_slices(p, p->Ah, p->fine, 1, p->flu, s);
+    if (p->opt.mode == PKASP_MODE_MULTIPLICATIVE) shaped_slices(p, p->Ah, p->fine, 2, p->flf, s);
+    return 500 + p->fll.t0;
 }
 
 // Layouts of the two hot fine-level kernels. The SpMV's lanes per row are autotuned: every
@@ -1222,6 +1224,14 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
         to32(p->d_cinv, p->d_cinv32, p->nc * p->nc, s);
     }
     build_tail(p, s);
+    // Gauss-Seidel levels above the tail sweep over slices as the fine smoother does: the
+    // lower parts forward, whole rows backward
+    if (o.level_smoother == PKASP_SMOOTHER_SGS)
+        for (int l = 0; l < p->tail; ++l) {
+            Level &L = p->lev[l];
+            shaped_slices(p, L.A, L.sp, 0, L.fl, s);
+            shaped_slices(p, L.A, L.sp, 2, L.ff, s);
+        }
     if (!p->aux_stream) PK_CUDA(cudaStreamCreateWithFlags(&p->aux_stream, cudaStreamNonBlocking));
     if (!p->cap_stream) PK_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
     if (!p->ev_fork) PK_CUDA(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
