@@ -65,6 +65,28 @@ __device__ __forceinline__ void bdotw(int64_t lo, int64_t hi, const int32_t *__r
     }
 }
 
+// the same with E entry groups per row, W * E lanes: group g adds entries lo + g, lo + g + E,
+// ..., and the groups' sums meet in a fixed shuffle tree (in every lane)
+template <int W, int E, int CPL, typename A, typename VT, typename XT>
+__device__ __forceinline__ void bdote(int64_t lo, int64_t hi, const int32_t *__restrict__ col,
+                                      const VT *__restrict__ val, const XT *X, int64_t ld, int lane, int g,
+                                      A (&acc)[CPL]) {
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) acc[k] = A(0);
+#pragma unroll 4
+    for (int64_t e = lo + g; e < hi; e += E) {
+        const int64_t j = __ldg(&col[e]);
+        const A a = (A)__ldg(&val[e]);
+        const XT *xr = X + j * ld + lane;
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) acc[k] += a * (A)xr[k * W];
+    }
+#pragma unroll
+    for (int k = 0; k < CPL; ++k)
+#pragma unroll
+        for (int o = W; o < W * E; o <<= 1) acc[k] += __shfl_xor_sync(kFull, acc[k], o);
+}
+
 // the same for the default task shape of an NC-wide block
 template <int NC, typename A, typename VT, typename XT>
 __device__ __forceinline__ void bdot(int64_t lo, int64_t hi, const int32_t *__restrict__ col,
@@ -585,48 +607,67 @@ __global__ void kb_add_div(int64_t n, const PT *R, const PT *__restrict__ d, PT 
     if (t < n * NC) X[t] += R[t] / d[t / NC];
 }
 
-// X = Ainv B (dense coarsest inverse), one task per row
+// X = M B for the dense tail of the V-cycle (tail.cu): one warp per row, 32 / W groups of
+// lanes share its entries, each with four partial sums per column
 template <int NC, typename PT>
-__global__ void kb_dense(int64_t n, const PT *__restrict__ Ainv, const PT *B, PT *X) {
-    constexpr int W = Tile<NC>::W, CPL = Tile<NC>::CPL;
-    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
-    const int lane = threadIdx.x % W;
-    if (row >= n) return;
-    PT acc[CPL];
+__global__ void __launch_bounds__(kBlock) kb_dense(int64_t n, const PT *__restrict__ M, const PT *B, PT *X) {
+    constexpr int W = Tile<NC>::W, CPL = Tile<NC>::CPL, E = 32 / W, U = CPL > 1 ? 2 : 4;
+    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x % W, g = (threadIdx.x & 31) / W;
+    if (row >= n) return;  // a whole warp
+    PT acc[U][CPL];
 #pragma unroll
-    for (int k = 0; k < CPL; ++k) acc[k] = PT(0);
-    for (int64_t j = 0; j < n; ++j) {
-        const PT a = Ainv[row * n + j];
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) acc[k] += a * B[j * NC + lane + k * W];
+        for (int k = 0; k < CPL; ++k) acc[u][k] = PT(0);
+    const PT *m = M + row * n;
+#pragma unroll 2
+    for (int64_t j0 = g; j0 < n; j0 += U * E) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t j = j0 + u * E;
+            if (j >= n) break;
+            const PT a = ldg(&m[j]);
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) acc[u][k] += a * B[j * NC + lane + k * W];
+        }
     }
 #pragma unroll
-    for (int k = 0; k < CPL; ++k) X[row * NC + lane + k * W] = acc[k];
+    for (int k = 0; k < CPL; ++k) {
+        PT t = acc[0][k];
+#pragma unroll
+        for (int u = 1; u < U; ++u) t += acc[u][k];
+#pragma unroll
+        for (int o = W; o < 32; o <<= 1) t += __shfl_xor_sync(kFull, t, o);
+        if (g == 0) X[row * NC + lane + k * W] = t;
+    }
 }
 
 // colour phase of the symmetric GS from zero on a group of CH columns of blocks with
 // row stride ld (R and Y point at the group's first column), W lanes per row, column
 // lane + k*W of the group in lane `lane` (PDL: the static loads come first):
 //   BACK = false: Y_i = (R_i - sum_L a_ij Y_j) * dinv_i ;  BACK = true: Y_i -= (sum_U a_ij Y_j) * dinv_i
-template <int CH, int W, typename PT, bool BACK>
+// E entry groups share a row (W * E lanes): a phase of few rows waits for its longest row,
+// and a vertex row of P3 has up to 170 entries on one chain of FP64 adds without them.
+template <int CH, int W, int E, typename PT, bool BACK>
 __global__ void __launch_bounds__(kBlock) kb_gs_phase(int64_t pb, int64_t pe, const int32_t *__restrict__ perm,
                                                       const int64_t *__restrict__ xptr,
                                                       const int32_t *__restrict__ xcol,
                                                       const PT *__restrict__ xval, const PT *__restrict__ dinv,
                                                       const PT *R, PT *Y, int64_t ld) {
-    static_assert(CH % W == 0 && 32 % W == 0, "lanes must divide the group and the warp");
+    static_assert(CH % W == 0 && 32 % (W * E) == 0, "lanes must divide the group and the warp");
     constexpr int CPL = CH / W;
     pdl_trigger();
-    const int64_t p = pb + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
-    const int lane = threadIdx.x % W;
+    const int64_t p = pb + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (W * E);
+    const int lane = threadIdx.x % W, g = threadIdx.x % (W * E) / W;
     const bool ok = p < pe;
     const int32_t i = ok ? perm[p] : 0;
     const PT di = ok ? dinv[p] : PT(1);
     const int64_t lo = ok ? xptr[p] : 0, hi = ok ? xptr[p + 1] : 0;
     pdl_wait();
-    if (!ok) return;
     PT acc[CPL];
-    bdotw<W, CPL, PT>(lo, hi, xcol, xval, (const PT *)Y, ld, lane, acc);
+    bdote<W, E, CPL, PT>(lo, hi, xcol, xval, (const PT *)Y, ld, lane, g, acc);
+    if (!ok || g != 0) return;
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
         const int64_t o = (int64_t)i * ld + lane + k * W;
@@ -635,20 +676,21 @@ __global__ void __launch_bounds__(kBlock) kb_gs_phase(int64_t pb, int64_t pe, co
 }
 
 // full backward GS sweep phase from the current X (level and multiplicative post-smoother)
-template <int NC, typename PT, typename TB>
+template <int NC, int E, typename PT, typename TB>
 __global__ void __launch_bounds__(kBlock) kb_gs_full(int64_t pb, int64_t pe, const int32_t *__restrict__ perm,
                                                      const int64_t *__restrict__ lptr, const int32_t *__restrict__ lcol,
                                                      const PT *__restrict__ lval, const int64_t *__restrict__ uptr,
                                                      const int32_t *__restrict__ ucol, const PT *__restrict__ uval,
                                                      const PT *__restrict__ diag, const TB *B, PT *X) {
     constexpr int W = Tile<NC>::W, CPL = Tile<NC>::CPL;
-    const int64_t p = pb + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
-    const int lane = threadIdx.x % W;
-    if (p >= pe) return;
-    const int32_t i = perm[p];
+    const int64_t p = pb + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (W * E);
+    const int lane = threadIdx.x % W, g = threadIdx.x % (W * E) / W;
+    const bool ok = p < pe;
+    const int32_t i = ok ? perm[p] : 0;
     PT sl[CPL], su[CPL];
-    bdot<NC, PT>(lptr[p], lptr[p + 1], lcol, lval, (const PT *)X, NC, lane, sl);
-    bdot<NC, PT>(uptr[p], uptr[p + 1], ucol, uval, (const PT *)X, NC, lane, su);
+    bdote<W, E, CPL, PT>(ok ? lptr[p] : 0, ok ? lptr[p + 1] : 0, lcol, lval, (const PT *)X, NC, lane, g, sl);
+    bdote<W, E, CPL, PT>(ok ? uptr[p] : 0, ok ? uptr[p + 1] : 0, ucol, uval, (const PT *)X, NC, lane, g, su);
+    if (!ok || g != 0) return;
     const PT d = diag[p];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
@@ -683,7 +725,7 @@ struct Batched {
     // every phase of a group reads the group's columns of Y, so a group small enough to
     // stay in L2 saves the re-reads from HBM that a full-width block costs on a large
     // fine level; fewer lanes per row put more rows (and loads) in flight per SM
-    template <int CH, int WL, typename PT>
+    template <int CH, int WL, int E, typename PT>
     static void gs_sym_group(const DSplit &sp, const PT *r, PT *y, bool backward, cudaStream_t s) {
         for (int c0 = 0; c0 < NC; c0 += CH) {
             const PT *rg = r + c0;
@@ -691,7 +733,7 @@ struct Batched {
             for (int c = 0; c < sp.ncol; ++c) {
                 const int64_t pb = sp.off[c], pe = sp.off[c + 1];
                 if (pe <= pb) continue;
-                blaunch_pdl(kb_gs_phase<CH, WL, PT, false>, tasks_grid(pe - pb, WL), s, pb, pe,
+                blaunch_pdl(kb_gs_phase<CH, WL, E, PT, false>, tasks_grid(pe - pb, WL * E), s, pb, pe,
                             (const int32_t *)sp.perm, (const int64_t *)sp.lptr, (const int32_t *)sp.lcol,
                             bpick<PT>(sp.lval, sp.lval32), bpick<PT>(sp.dinv, sp.dinv32), rg, yg, (int64_t)NC);
             }
@@ -699,12 +741,17 @@ struct Batched {
             for (int c = sp.ncol - 2; c >= 0; --c) {
                 const int64_t pb = sp.off[c], pe = sp.off[c + 1];
                 if (pe <= pb) continue;
-                blaunch_pdl(kb_gs_phase<CH, WL, PT, true>, tasks_grid(pe - pb, WL), s, pb, pe,
+                blaunch_pdl(kb_gs_phase<CH, WL, E, PT, true>, tasks_grid(pe - pb, WL * E), s, pb, pe,
                             (const int32_t *)sp.perm, (const int64_t *)sp.uptr, (const int32_t *)sp.ucol,
                             bpick<PT>(sp.uval, sp.uval32), bpick<PT>(sp.dinv, sp.dinv32), (const PT *)yg, yg,
                             (int64_t)NC);
             }
         }
+    }
+    // whole warps per row (32 / W entry groups) while a mean phase then has no more lanes
+    // than about two waves of the chip; wider phases have enough rows in flight without
+    static bool split_rows(const DSplit &sp) {
+        return sp.ncol > 0 && sp.off.back() / sp.ncol * 32 <= 600000;
     }
     // the layouts the autotuner tries: (group columns, lanes per row)
     static constexpr int kLayouts = 6;
@@ -718,12 +765,13 @@ struct Batched {
     }
     template <int K, typename PT>
     static void gs_layout(const DSplit &sp, const PT *r, PT *y, bool backward, cudaStream_t s) {
-        if constexpr (layout_ok(K)) gs_sym_group<layout_ch(K), layout_w(K), PT>(sp, r, y, backward, s);
+        if constexpr (layout_ok(K)) gs_sym_group<layout_ch(K), layout_w(K), 1, PT>(sp, r, y, backward, s);
         else fail(PKASP_EINVAL, "smoother layout not available for this block width");
     }
     // layout k of the list above (0: full width, the default lanes)
     template <typename PT>
     static void gs_sym(const DSplit &sp, const PT *r, PT *y, bool backward, int k, cudaStream_t s) {
+        if (split_rows(sp)) return gs_sym_group<NC, W, 32 / W, PT>(sp, r, y, backward, s);
         switch (k) {
             case 1: gs_layout<1, PT>(sp, r, y, backward, s); break;
             case 2: gs_layout<2, PT>(sp, r, y, backward, s); break;
@@ -738,7 +786,8 @@ struct Batched {
         for (int c = sp.ncol - 1; c >= 0; --c) {
             const int64_t pb = sp.off[c], pe = sp.off[c + 1];
             if (pe <= pb) continue;
-            kb_gs_full<NC, PT, TB><<<tasks_grid(pe - pb, W), kBlock, 0, s>>>(
+            auto kern = split_rows(sp) ? kb_gs_full<NC, 32 / W, PT, TB> : kb_gs_full<NC, 1, PT, TB>;
+            kern<<<tasks_grid(pe - pb, split_rows(sp) ? 32 : W), kBlock, 0, s>>>(
                 pb, pe, sp.perm, sp.lptr, sp.lcol, bpick<PT>(sp.lval, sp.lval32), sp.uptr, sp.ucol,
                 bpick<PT>(sp.uval, sp.uval32), bpick<PT>(sp.diag, sp.diag32), b, x);
             PK_LAUNCH();
@@ -759,12 +808,16 @@ struct Batched {
         PT *b = bpickw<PT>(p->bl_b[l], p->bl_b32[l]);
         PT *x = bpickw<PT>(p->bl_x[l], p->bl_x32[l]);
         PT *r = bpickw<PT>(p->bl_r[l], p->bl_r32[l]);
-        if (l == (int)p->lev.size() - 1) {
-            kb_dense<NC, PT><<<tasks_grid(n, W), kBlock, 0, s>>>(n, bpick<PT>(p->d_cinv, p->d_cinv32), b, x);
+        const bool jac = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
+        // the dense tail takes NC times the FMAs of one column; with l1-Jacobi levels, whose
+        // few launches it replaces, only while those stay below 10^7
+        const bool tail = l == p->tail && (!jac || (double)n * n * NC <= 1e7);
+        if (tail || l == (int)p->lev.size() - 1) {
+            kb_dense<NC, PT><<<tasks_grid(n, 32), kBlock, 0, s>>>(
+                n, tail ? bpick<PT>(p->d_tail, p->d_tail32) : bpick<PT>(p->d_cinv, p->d_cinv32), b, x);
             PK_LAUNCH();
             return;
         }
-        const bool jac = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
         const int64_t ne = n * NC;
         if (jac) {
             kb_jacobi0<NC, PT, PT><<<(unsigned)((ne + kBlock - 1) / kBlock), kBlock, 0, s>>>(
@@ -876,7 +929,7 @@ struct Batched {
     // layout: each column's sums run over the same entries in the same order. Returns
     // 1 + the index of the fastest layout.
     static int tune_group(pkasp_problem *p, cudaStream_t s) {
-        if (p->opt.smoother == PKASP_SMOOTHER_L1JACOBI) return 1;
+        if (p->opt.smoother == PKASP_SMOOTHER_L1JACOBI || split_rows(p->fine)) return 1;
         int best = 0;
         float best_ms = 1e30f;
         const bool f32 = p->opt.precond_precision == PKASP_PREC_FP32;

@@ -97,3 +97,26 @@ def test_cycle_with_dense_tail(oracle_mod, n, level_smoother):
     # FP32: row sums of up to 5120 terms on the tail, u = 2^-24
     G.setup(level_smoother=level_smoother, precond_precision=1)
     _close(G.apply_vcycle(torch.tensor(b, device="cuda")).cpu().numpy(), ref, 5120 * 2.0 ** -24)
+
+
+# every block width with rows shared by lane groups and a dense tail, against the
+# single-column solve of each column (both to 1e-8: the bound of the other block tests)
+@pytest.mark.parametrize("ncols,prec,level_smoother,mode", [(3, 0, 0, 0), (7, 1, 0, 0), (13, 0, 1, 0), (30, 1, 1, 0),
+                                                            (41, 0, 0, 1), (60, 1, 0, 0)])
+def test_block_widths(ncols, prec, level_smoother, mode):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(6, 0.2, 0)
+    P = Problem(xyz, t, 3, kappa_lognormal(t.shape[0], 1))
+    P.setup(precond_precision=prec, level_smoother=level_smoother, mode=mode)
+    b = torch.randn(P.nh, ncols, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(ncols))
+    x, st = P.solve(b)
+    assert max(st["true_rel"]) <= 1e-8
+    for c in (0, ncols // 2, ncols - 1):
+        xc, sc = P.solve(b[:, c].contiguous())
+        assert abs(sc["iters"][0] - st["iters"][c]) <= 1
+        assert (x[:, c] - xc).norm() <= 1e-8 * xc.norm()
+    P.close()
