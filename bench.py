@@ -563,7 +563,7 @@ def main():
                           "frac": s_tf / FP64_PEAK_TFLOPS, "flops_per_application": smoother_flops,
                           "peak_source": "derived: 152 SMs x 2.07 GHz x 4 FP64 flop/clk/SM"}}
     achieved = spmv_bytes / (spmv_ms / 1e3) / 1e9
-    roof_spmv = {"bound": "hbm", "kernel": "k_spmv_q / k_sell_spmv (fine SpMV, SELL-32, FP64)",
+    roof_spmv = {"bound": "hbm", "kernel": "k_spmv_q / k_spmv_y (fine SpMV, interleaved slices, FP64)",
                  "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                  "frac_of_nominal_8000": achieved / NOMINAL_HBM_GBS,
                  "traffic": SPMV_TRAFFIC.get((WORKLOAD["name"], WORKLOAD["n"])),
@@ -606,7 +606,7 @@ def main():
              "l2_persist_bytes": int(info64.l2_persist_bytes),
              "level_rows": [int(v) for v in info64.level_rows[: info64.levels]],
              "fine_colours": int(info64.fine_colours), "op_complexity": info64.op_complexity,
-             "spmv_layout": "SELL-32" if info64.spmv_layout == 0 else f"CSR x{info64.spmv_layout} lanes",
+             "spmv_layout": smoother_layout_name(info64.spmv_layout),
              "smoother_layout": smoother_layout_name(info64.smoother_layout),
              "smoother_ms": smoother_ms, "smoother_GBps": s_ach, "spmv_ms": spmv_ms,
              "fp32_preconditioner": fp32,

@@ -79,7 +79,7 @@ typedef struct {
     int use_graph;        /* 1: each solve runs as one CUDA graph with a device-side
                              while loop; 0: eager launches, host checks every iteration [1] */
     int spmv_threads;     /* threads per row of the fine SpMV and smoother: 4, 8, 16 or
-                             32; 0 = pick by mean row length [0] */
+                             32; 0 = interleaved slices shaped by the sizes [0] */
     int smoother_layout;  /* fine smoother layout (SGS): 0 = interleaved slices, one
                              launch per colour phase, shaped by the sizes [0];
                              1 = one launch per colour phase, CSR, lanes fitted per colour;
@@ -137,10 +137,10 @@ typedef struct {
     double op_complexity;   /* sum_l nnz(A_l) / nnz(A_0), A_0 = A_H (A_h in plain AMG
                                mode) (Sec. 6.2, Table 6) */
     double setup_ms, assemble_ms;
-    int spmv_layout;        /* autotuned layout of the fine SpMV: 0 = SELL-32 (one thread
-                               per row), t > 0 = CSR read by t lanes per row */
-    int smoother_layout;    /* same for the fine smoother's colour phases; 500 + t = interleaved
-                               slices, t lanes for an ordinary row; -1 = CSR with
+    int spmv_layout;        /* layout of the fine SpMV: 500 + t = interleaved slices, t lanes
+                               for an ordinary row; t < 500 = CSR read by t lanes per row
+                               (options.spmv_threads) */
+    int smoother_layout;    /* same for the fine smoother's colour phases; 0 = SELL-32; -1 = CSR with
                                lanes fitted per colour; 100 + t = t lanes, two rows per
                                lane group; 400 + t = t lanes, grid-stride over the resident
                                blocks; -t (t > 1) = the whole symmetric sweep in one

@@ -88,7 +88,7 @@ struct DSplit {
     std::vector<int> l90, u90;    // per colour: 90th percentile of those lengths (host)
 };
 
-// SELL-32: slices of 32 rows (one thread per row), entries column-major within a slice
+// SELL-32 (smoother_layout 2): slices of 32 rows (one thread per row), column-major within a slice
 // (entry k of slice row r at sptr[slice] + 32 k + r), padded with column -1. perm maps
 // a padded position to its row (natural order when null; -1 marks padding rows); coff
 // gives each colour's slice range when the rows are colour-sorted.
@@ -200,10 +200,10 @@ struct pkasp_problem {
     bool have_setup = false;
     pkasp_options opt{};
     pk::DSplit fine;      // colour split of A_h
-    pk::DSell Asell;      // SELL-32 copy of A_h (natural order)
-    pk::DSell fsl, fsu;   // SELL-32 colour-sorted lower / upper parts of A_h
+    pk::DSell fsl, fsu;   // SELL-32 colour-sorted lower / upper parts of A_h (smoother_layout 2)
     pk::DSlices fll, flu, flf;  // interleaved slices of A_h: lower parts, upper parts, whole
                                 // rows (multiplicative form only)
+    pk::DSlices fsv;            // and its rows with the diagonal (SpMV)
     double *d_l1h = nullptr;
     float *d_l1h32 = nullptr;
     std::vector<pk::Level> lev;
@@ -216,7 +216,7 @@ struct pkasp_problem {
     int64_t *d_fine_off = nullptr;  // device copy of fine.off (persistent smoother)
     unsigned *d_bar = nullptr;      // grid-barrier arrivals / exits of the persistent smoother
     int *d_bar_err = nullptr;       // set when one of its barriers timed out
-    int spmv_tpr = 4;   // lanes per row of the fine SpMV (autotuned at setup)
+    int spmv_tpr = 4;   // layout code of the fine SpMV (pkasp_info.spmv_layout)
     int fine_tpr = 4;   // layout code of the fine smoother phases (pkasp_info.smoother_layout)
     // solve work (sized for ncols = 1 at setup, grown on demand)
     int work_cols = 0;
@@ -350,14 +350,14 @@ void stokes_sizes(const pkasp_problem *p, int64_t *out5);
 float time_kernel(pkasp_problem *p, int which, int reps, cudaStream_t s);
 
 // interleaved slices (slices.cu): part 0 lower, 1 upper parts of the split, 2 whole rows
+// without the diagonal, 3 the rows of A
 void build_slices(DevPool &pool, const DCSR &A, const DSplit &sp, int part, int t0, int steps, bool fp32, DSlices &S,
                   cudaStream_t s);
 
 // the dense tail of the V-cycle (tail.cu); after the hierarchy and the coarsest inverse
 void build_tail(pkasp_problem *p, cudaStream_t s);
 
-// SELL-32 builders (sell.cu)
-void build_sell_natural(DevPool &pool, const DCSR &A, DSell &S, bool want32, cudaStream_t s);
+// SELL-32 builder (sell.cu)
 void build_sell_split(DevPool &pool, const DSplit &sp, int64_t n, bool upper, DSell &S, bool want32,
                       cudaStream_t s);
 

@@ -744,39 +744,6 @@ __global__ void __launch_bounds__(128) k_dense_mv(int64_t n, const PT *__restric
 // SELL-32 kernels: one thread per row; a warp is one slice, so every column and value
 // load of the warp is one contiguous access. Padding entries carry column -1.
 // ---------------------------------------------------------------------------------
-template <typename A, typename VT, typename XT>
-__device__ __forceinline__ A sell_dot(int64_t base, int w, const int32_t *__restrict__ col,
-                                      const VT *__restrict__ val, const XT *x) {
-    A acc = A(0);
-    for (int k0 = 0; k0 < w; k0 += kBatch) {
-        int c[kBatch];
-        A v[kBatch];
-#pragma unroll
-        for (int k = 0; k < kBatch; ++k) {
-            const int64_t e = base + 32 * (int64_t)(k0 + k);
-            const bool ok = k0 + k < w;
-            c[k] = ok ? ldst(&col[e]) : -1;
-            v[k] = ok ? (A)ldst(&val[e]) : A(0);
-        }
-#pragma unroll
-        for (int k = 0; k < kBatch; ++k)
-            if (c[k] >= 0) acc += v[k] * (A)x[c[k]];
-    }
-    return acc;
-}
-
-// y = A x, rows in natural order
-template <typename A, typename VT, typename XT, typename YT>
-__global__ void __launch_bounds__(kBlock) k_sell_spmv(int64_t n, const int64_t *__restrict__ sptr,
-                                                      const int32_t *__restrict__ sw, const int32_t *__restrict__ col,
-                                                      const VT *__restrict__ val, const XT *__restrict__ x,
-                                                      YT *__restrict__ y) {
-    const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= n) return;
-    const int64_t s = row >> 5;
-    y[row] = (YT)sell_dot<A>(sptr[s] + (row & 31), sw[s], col, val, x);
-}
-
 // One colour phase of the symmetric Gauss-Seidel sweep from zero over the SELL-32 slices
 // [s0, s1) of a colour-sorted split, one thread per row (no reduction across lanes):
 //   BACK = false: y_i = (r_i - sum_L a_ij y_j) * dinv_i

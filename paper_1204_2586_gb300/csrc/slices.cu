@@ -17,8 +17,8 @@
 namespace pk {
 namespace {
 
-constexpr int kSteps = 16;             // most steps (of DSlices::steps) of a row at T < 32
-constexpr int kKeys = 2 + 5 * kSteps;  // (T, W) classes of a colour: T = 32, 16 .. 1 by W, empty
+// (T, W) classes of a colour: T = 32, 16 .. 1 by W, empty
+int keys_of(int steps) { return 2 + 5 * steps; }
 
 unsigned blocks_for(int64_t n, int per) {
     int64_t b = (n + per - 1) / per;
@@ -32,20 +32,21 @@ __host__ __device__ inline int lanes_of(int64_t len, int t0, int steps) {
     return t;
 }
 
-// Class of a row part: 0 for 32 lanes, then 16 lanes with kSteps, kSteps - 1, ... steps, then
+// Class of a row part: 0 for 32 lanes, then 16 lanes with steps, steps - 1, ... steps, then
 // 8 lanes, ...; the last class holds the empty parts.
 __host__ __device__ inline int class_of(int64_t len, int t0, int steps) {
-    if (len == 0) return kKeys - 1;
+    if (len == 0) return 1 + 5 * steps;
     const int t = lanes_of(len, t0, steps);
     if (t == 32) return 0;
     const int w = (int)((len + t - 1) / t);
     int rank = 0;
     for (int u = 16; u > t; u >>= 1) ++rank;
-    return 1 + rank * kSteps + (kSteps - w);
+    return 1 + rank * steps + (steps - w);
 }
 
-// The parts that a layout is built from: the lower or upper parts of a colour split, or
-// whole rows without their diagonal (full: rows perm[p] of a matrix).
+// The parts that a layout is built from: the lower or upper parts of a colour split, whole
+// rows without their diagonal (full: rows perm[p] of a matrix), or the rows themselves (perm
+// is null).
 struct Parts {
     const int64_t *ptr;
     const int32_t *col;
@@ -55,6 +56,7 @@ struct Parts {
     __device__ int64_t lo(int64_t p) const { return ptr[full ? (int64_t)perm[p] : p]; }
     __device__ int64_t hi(int64_t p) const { return ptr[(full ? (int64_t)perm[p] : p) + 1]; }
     __device__ int64_t len(int64_t p) const { return hi(p) - lo(p) - (full ? 1 : 0); }
+    __device__ int32_t row(int64_t p) const { return perm ? perm[p] : (int32_t)p; }
 };
 
 __global__ void k_slice_keys(int64_t n, Parts A, int t0, int steps, const int32_t *__restrict__ colour,
@@ -63,7 +65,7 @@ __global__ void k_slice_keys(int64_t n, Parts A, int t0, int steps, const int32_
     int len = 0;
     if (p < n) {
         len = (int)A.len(p);
-        key[p] = colour[A.perm[p]] * kKeys + class_of(len, t0, steps);
+        key[p] = (colour ? colour[A.row(p)] * (2 + 5 * steps) : 0) + class_of(len, t0, steps);
     }
     len = __reduce_max_sync(0xffffffffu, len);
     if ((threadIdx.x & 31) == 0 && len > 0) atomicMax(maxlen, len);
@@ -122,7 +124,7 @@ __global__ void k_slice_fill(int64_t ns, const int4 *__restrict__ meta, Parts A,
     const int sub = lane & (t - 1), r = lane >> lt;
     const bool ok = r < nr;
     const int64_t p = ok ? order[m.z + r] : 0;
-    const int32_t i = ok ? A.perm[p] : -1;
+    const int32_t i = ok ? A.row(p) : -1;
     const int64_t lo = ok ? A.lo(p) : 0, len = ok ? A.len(p) : 0;
     // whole rows skip their diagonal: entries from there on move down by one
     int64_t skip = len;
@@ -144,47 +146,51 @@ __global__ void k_slice_fill(int64_t ns, const int4 *__restrict__ meta, Parts A,
     }
     if (ok && sub == 0) {
         rows[m.z + r] = i;
-        sdinv[m.z + r] = (PT)dinv[p];
+        if (dinv) sdinv[m.z + r] = (PT)dinv[p];
     }
 }
 
 }  // namespace
 
-// part: 0 lower, 1 upper, 2 whole rows of A. Rows whose upper part is empty are left out
-// (their phase would change nothing).
+// part: 0 lower, 1 upper, 2 whole rows of A without the diagonal, 3 the rows of A themselves
+// (no colours: one list of slices). Rows whose upper part is empty are left out (their phase
+// would change nothing).
 void build_slices(DevPool &pool, const DCSR &A, const DSplit &sp, int part, int t0, int steps, bool fp32, DSlices &S,
                   cudaStream_t s) {
     S = DSlices{};
     S.t0 = t0;
     S.steps = steps;
     const int64_t n = A.n;
-    const Parts P = part == 2 ? Parts{A.ptr, A.col, A.val, sp.perm, true}
+    const bool plain = part == 3;
+    const int ncol = plain ? 1 : sp.ncol, keys = keys_of(steps);
+    const Parts P = plain ? Parts{A.ptr, A.col, A.val, nullptr, false}
+                    : part == 2 ? Parts{A.ptr, A.col, A.val, sp.perm, true}
                     : part == 1 ? Parts{sp.uptr, sp.ucol, sp.uval, sp.perm, false}
                                 : Parts{sp.lptr, sp.lcol, sp.lval, sp.perm, false};
-    S.off.assign(sp.ncol + 1, 0);
+    S.off.assign(ncol + 1, 0);
     if (n == 0) return;
     DevPool tmp;
     try {
         int32_t *key = tmp.get<int32_t>(n), *order = tmp.get<int32_t>(n);
         int *maxlen = tmp.get<int>(1);
         PK_CUDA(cudaMemsetAsync(maxlen, 0, sizeof(int), s));
-        k_slice_keys<<<blocks_for(n, 256), 256, 0, s>>>(n, P, t0, steps, sp.colour, key, maxlen);
+        k_slice_keys<<<blocks_for(n, 256), 256, 0, s>>>(n, P, t0, steps, plain ? nullptr : sp.colour, key, maxlen);
         PK_LAUNCH();
         std::vector<int64_t> koff;
-        key_sort(n, key, (int64_t)sp.ncol * kKeys, order, koff, s);
+        key_sort(n, key, (int64_t)ncol * keys, order, koff, s);
         int longest = 0;
         PK_CUDA(cudaMemcpyAsync(&longest, maxlen, sizeof(int), cudaMemcpyDeviceToHost, s));
         PK_CUDA(cudaStreamSynchronize(s));
         if (longest >= (32 << 20)) fail(PKASP_ENOMEM, "a row of A_h has more than 2^25 entries");
         std::vector<Group> groups;
         int64_t ns = 0;
-        for (int c = 0; c < sp.ncol; ++c) {
-            for (int q = 0; q < kKeys; ++q) {
-                const int64_t p0 = koff[(int64_t)c * kKeys + q], m = koff[(int64_t)c * kKeys + q + 1] - p0;
-                if (m == 0 || (part == 1 && q == kKeys - 1)) continue;
+        for (int c = 0; c < ncol; ++c) {
+            for (int q = 0; q < keys; ++q) {
+                const int64_t p0 = koff[(int64_t)c * keys + q], m = koff[(int64_t)c * keys + q + 1] - p0;
+                if (m == 0 || (part == 1 && q == keys - 1)) continue;
                 int lt = 5;  // class 0: 32 lanes; empty parts: one lane
-                if (q == kKeys - 1) lt = 0;
-                else if (q > 0) lt = 4 - (q - 1) / kSteps;
+                if (q == keys - 1) lt = 0;
+                else if (q > 0) lt = 4 - (q - 1) / steps;
                 groups.push_back(Group{ns, p0, m, lt, 0});
                 const int rows = 32 >> lt;
                 ns += (m + rows - 1) / rows;
@@ -194,8 +200,8 @@ void build_slices(DevPool &pool, const DCSR &A, const DSplit &sp, int part, int 
         S.nslices = ns;
         S.meta = pool.get<int4>(std::max<int64_t>(ns, 1));
         S.rows = pool.get<int32_t>(n);
-        if (fp32) S.dinv32 = pool.get<float>(n);
-        else S.dinv = pool.get<double>(n);
+        if (!plain && fp32) S.dinv32 = pool.get<float>(n);
+        if (!plain && !fp32) S.dinv = pool.get<double>(n);
         Group *dg = tmp.get<Group>(std::max<size_t>(groups.size(), 1));
         int64_t *width = tmp.get<int64_t>(ns + 1);
         if (ns > 0) {
@@ -212,10 +218,10 @@ void build_slices(DevPool &pool, const DCSR &A, const DSplit &sp, int part, int 
         else S.val = pool.get<double>(std::max<int64_t>(S.entries, 1));
         if (ns > 0) {
             if (fp32)
-                k_slice_fill<float><<<blocks_for(ns * 32, 256), 256, 0, s>>>(ns, S.meta, P, order, sp.dinv, S.col,
+                k_slice_fill<float><<<blocks_for(ns * 32, 256), 256, 0, s>>>(ns, S.meta, P, order, plain ? nullptr : sp.dinv, S.col,
                                                                             S.val32, S.rows, S.dinv32);
             else
-                k_slice_fill<double><<<blocks_for(ns * 32, 256), 256, 0, s>>>(ns, S.meta, P, order, sp.dinv, S.col,
+                k_slice_fill<double><<<blocks_for(ns * 32, 256), 256, 0, s>>>(ns, S.meta, P, order, plain ? nullptr : sp.dinv, S.col,
                                                                              S.val, S.rows, S.dinv);
             PK_LAUNCH();
         }

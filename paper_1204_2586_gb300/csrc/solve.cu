@@ -32,7 +32,7 @@ namespace {
 // ---------------------------------------------------------------------------------
 // Lanes per row. Short sub-warps keep more rows, and more independent loads per lane,
 // in flight: on GB300 four lanes beat sixteen by 1.7x on the P3 matrix (47 entries per
-// row). The fine SpMV is autotuned at setup instead, the fine smoother takes slices.
+// row). The fine SpMV and smoother take interleaved slices instead.
 int tpr_for(double mean_row) {
     if (mean_row <= 96) return 4;
     return 8;
@@ -511,6 +511,13 @@ void restrict_vcycle(pkasp_problem *p, const double *r, cudaStream_t s) {
     vcycle<PT>(p, 0, s, pd);
 }
 
+// r = b - A x
+template <int TPR>
+__global__ void __launch_bounds__(kBlock) k_residual_fine(int64_t n, RowOp A, const double *__restrict__ b,
+                                                          const double *__restrict__ x, double *__restrict__ r) {
+    for_rows<TPR>(n, A, x, [&](int64_t row, double s) { r[row] = b[row] - s; });
+}
+
 // z = B r. tail = false (additive mode only) stops before the last step z = z_s + Pi w:
 // the PCG iteration then runs that step inside k_prolong_beta.
 template <typename PT>
@@ -548,11 +555,20 @@ void precondition(pkasp_problem *p, const double *r, double *z, cudaStream_t s, 
     const bool slices = p->fine_tpr > 500;
     const int tfw = p->fine_tpr > 0 ? p->fine_tpr : -1;
     const int ts = p->fine_tpr > 0 ? p->fine_tpr % 100 : -1;
-    // the residuals read the CSR form (a SELL-32 choice of the autotuner maps to the
-    // lanes fitted to the mean row length)
-    const int ta = p->spmv_tpr > 0 ? p->spmv_tpr : tpr_of(p->Ah);
     PT *t = pickw<PT>(p->w_t, p->w_t32);
     PT *rr = pickw<PT>(p->w_rr, p->w_rr32);
+    // the residuals read the fine operator as the outer iteration does, in FP32 its CSR form
+    auto fine_residual = [&] {
+        if constexpr (std::is_same<PT, double>::value) {
+            PK_FMT_SWITCH(p->spmv_tpr, (k_residual_fine<TPR><<<fine_grid(p), kBlock, 0, s>>>(p->nh, fine_op(p), rr, zs,
+                                                                                          t)));
+        } else {
+            const int ta = p->spmv_tpr < 500 ? p->spmv_tpr : tpr_of(p->Ah);
+            PK_TPR_SWITCH(ta, (k_residual<TPR, PT, PT, PT><<<rows_grid(p->nh, TPR), kBlock, 0, s>>>(
+                                  p->nh, p->Ah.ptr, p->Ah.col, p->Ah.val32, rr, zs, t)));
+        }
+        PK_LAUNCH();
+    };
     if (jac) {
         k_jacobi0<PT, double><<<elem_grid(p->nh), kBlock, 0, s>>>(p->nh, pick<PT>(p->d_l1h, p->d_l1h32), r, zs);
         PK_LAUNCH();
@@ -563,9 +579,7 @@ void precondition(pkasp_problem *p, const double *r, double *z, cudaStream_t s, 
         else gs_forward0<PT, double>(p->fine, tfw, r, zs, s, win);
     }
     to_pt<PT>(r, rr, p->nh, s);
-    PK_TPR_SWITCH(ta, (k_residual<TPR, PT, PT, PT><<<rows_grid(p->nh, TPR), kBlock, 0, s>>>(
-                          p->nh, p->Ah.ptr, p->Ah.col, pick<PT>(p->Ah.val, p->Ah.val32), rr, zs, t)));
-    PK_LAUNCH();
+    fine_residual();
     const bool pd = restrict_to<PT>(p, p->PiT, (const PT *)t, 0, s);
     vcycle<PT>(p, 0, s, pd);
     k_prolong_add<PT, PT><<<elem_grid(p->nh), kBlock, 0, s>>>(p->nh, p->Pi.ptr, p->Pi.col,
@@ -573,9 +587,7 @@ void precondition(pkasp_problem *p, const double *r, double *z, cudaStream_t s, 
                                                               zs, zs);
     PK_LAUNCH();
     if (jac) {
-        PK_TPR_SWITCH(ta, (k_residual<TPR, PT, PT, PT><<<rows_grid(p->nh, TPR), kBlock, 0, s>>>(
-                              p->nh, p->Ah.ptr, p->Ah.col, pick<PT>(p->Ah.val, p->Ah.val32), rr, zs, t)));
-        PK_LAUNCH();
+        fine_residual();
         k_add_div<PT><<<elem_grid(p->nh), kBlock, 0, s>>>(p->nh, t, pick<PT>(p->d_l1h, p->d_l1h32), zs);
         PK_LAUNCH();
     } else {
@@ -623,13 +635,6 @@ __global__ void k_state_restart(PcgState *st) {
 // (i, i + stride, ...) before it computes, and adds its terms in ascending i as a
 // one-at-a-time loop would.
 constexpr int kVec = 4;
-
-// r = b - A x
-template <int TPR>
-__global__ void __launch_bounds__(kBlock) k_residual_fine(int64_t n, RowOp A, const double *__restrict__ b,
-                                                          const double *__restrict__ x, double *__restrict__ r) {
-    for_rows<TPR>(n, A, x, [&](int64_t row, double s) { r[row] = b[row] - s; });
-}
 
 // ||v||^2 of the grid, in every thread of the last block (grid_reduce)
 __device__ __forceinline__ bool grid_norm2(int64_t n, const double *__restrict__ v, double *partials,
@@ -1019,12 +1024,13 @@ void free_setup(pkasp_problem *p) {
     p->work_pool.free_all();
     p->lev.clear();
     p->fine = DSplit{};
-    p->Asell = DSell{};
     p->fsl = DSell{};
     p->fsu = DSell{};
     p->fll = DSlices{};
     p->flu = DSlices{};
     p->flf = DSlices{};
+    p->fsv = DSlices{};
+    p->spmv_tpr = 4;  // A_h itself stays: pkasp_spmv reads its CSR form until the next setup
     p->d_l1h = nullptr;
     p->d_l1h32 = nullptr;
     p->d_cinv = nullptr;
@@ -1092,61 +1098,36 @@ int fine_slices(pkasp_problem *p, cudaStream_t s) {
     return 500 + p->fll.t0;
 }
 
-// Layouts of the two hot fine-level kernels. The SpMV's lanes per row are autotuned: every
-// candidate runs a few times on the actual matrix (inputs f_h) and the fastest is kept. The
-// smoother takes interleaved slices. A fixed options.spmv_threads bypasses both, a fixed
-// options.smoother_layout the second.
-void autotune(pkasp_problem *p, cudaStream_t s) {
-    if (p->opt.spmv_threads) {
-        p->spmv_tpr = p->fine_tpr = p->opt.spmv_threads;
+// Slices of the fine SpMV (steps is the most of a row at T0 lanes). Below 400,000 entries
+// the chip is nearly empty and the chain of a row counts (P2 8^3, 79,000: 3.3 us with 4
+// lanes and 8 steps against 4.2 with 2 and 16); then lanes give way to FP64 slots as rows
+// fill the chip: 2 lanes and 16 steps up to 4 10^6 (P2 21^3, 1.8 10^6: 8.7 against 9.6 with
+// 32 steps), 2 and 32 up to 10^7 (P3 16^3, 4.6 10^6: 14.4 against 16.4 and, with 1 and 64,
+// 20.4), above one lane a row, which doubles past 64 or, from 3 10^7 on, 96 entries (P3 24^3,
+// 1.6 10^7: 37.3 with 64 against 38.4 with 2 lanes and 42.0 with 96; P4 48^3: 989 with 96
+// against 1000 with 64 and 1076 with 2 lanes and 32).
+void spmv_slices(pkasp_problem *p, cudaStream_t s) {
+    const double nnz = (double)p->Ah.nnz;
+    const int t0 = nnz < 4e5 ? 4 : nnz < 1e7 ? 2 : 1, steps = nnz < 4e5 ? 8 : nnz < 4e6 ? 16 : nnz < 1e7 ? 32 : nnz < 3e7 ? 64 : 96;
+    build_slices(p->setup_pool, p->Ah, p->fine, 3, t0, steps, false, p->fsv, s);
+    p->spmv_tpr = 500 + t0;
+}
+
+// Layouts of the two hot fine-level kernels: interleaved slices, unless
+// options.spmv_threads fixes the lanes per row of both or options.smoother_layout the
+// smoother's layout (-1 here for lanes fitted per colour, 0 SELL-32; the other codes pass
+// through).
+void choose_layouts(pkasp_problem *p, cudaStream_t s) {
+    const pkasp_options &o = p->opt;
+    if (o.spmv_threads) {
+        p->spmv_tpr = p->fine_tpr = o.spmv_threads;
         return;
     }
-    // a fixed smoother layout: internal code -1 per-colour lanes, 0 SELL-32, t lanes
-    // 100 + t (t lanes, two rows per sub-warp) passes through
-    const int lay = p->opt.smoother_layout;
-    const int fixed_fine = lay == 1 ? -1 : lay == 2 ? 0 : lay == 3 ? 2 : lay;
-    cudaEvent_t e0, e1;
-    PK_CUDA(cudaEventCreate(&e0));
-    PK_CUDA(cudaEventCreate(&e1));
-    auto time3 = [&](auto fn) {  // three back-to-back runs
-        PK_CUDA(cudaEventRecord(e0, s));
-        for (int i = 0; i < 3; ++i) fn();
-        PK_CUDA(cudaEventRecord(e1, s));
-        PK_CUDA(cudaEventSynchronize(e1));
-        float ms = 0;
-        cudaEventElapsedTime(&ms, e0, e1);
-        return ms;
-    };
-    // Candidates are timed round-robin, three rounds, best round per candidate: the
-    // GPU's clock can still be ramping up during setup, and timing candidates one after
-    // another would favour the later ones.
-    auto tune = [&](const int *cand, int nc, int *slot, auto run) {
-        std::vector<float> best(nc, 1e30f);
-        for (int k = 0; k < nc; ++k) {
-            *slot = cand[k];
-            run();  // warm-up (first use of each variant)
-        }
-        for (int round = 0; round < 3; ++round)
-            for (int k = 0; k < nc; ++k) {
-                *slot = cand[k];
-                best[k] = std::min(best[k], time3(run));
-            }
-        int pick = 0;
-        for (int k = 1; k < nc; ++k)
-            if (best[k] < best[pick]) pick = k;
-        return cand[pick];
-    };
-    // 0: SELL-32, one thread per row; t > 0: CSR with t lanes per row
-    const int cand_spmv[] = {0, 2, 4, 8};
-    const int pick_spmv = tune(cand_spmv, 4, &p->spmv_tpr, [&] { spmv_fine(p, p->d_b, p->w_q, s); });
-    p->spmv_tpr = pick_spmv;
-    int pick_fine = -1;
-    if (p->opt.smoother == PKASP_SMOOTHER_SGS)
-        pick_fine = p->opt.smoother_layout != 0 ? fixed_fine : fine_slices(p, s);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    p->spmv_tpr = pick_spmv;
-    p->fine_tpr = pick_fine;
+    spmv_slices(p, s);
+    const int lay = o.smoother_layout;
+    p->fine_tpr = -1;
+    if (o.smoother != PKASP_SMOOTHER_SGS) return;
+    p->fine_tpr = lay == 0 ? fine_slices(p, s) : lay == 1 ? -1 : lay == 2 ? 0 : lay == 3 ? 2 : lay;
 }
 
 void setup_device(pkasp_problem *p, cudaStream_t s) {
@@ -1157,7 +1138,6 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
     DevPool &pool = p->setup_pool;
     // fine level: colour split of A_h, l1 norms, FP32 copies
     build_split(pool, p->Ah, stream_colour(o.seed, 0), want32, p->fine, s);
-    build_sell_natural(pool, p->Ah, p->Asell, false, s);
     if (o.smoother_layout == 2) {
         build_sell_split(pool, p->fine, p->nh, false, p->fsl, want32, s);
         build_sell_split(pool, p->fine, p->nh, true, p->fsu, want32, s);
@@ -1173,7 +1153,6 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
             else to32(M->val, M->val32, M->nnz, s);
         }
     }
-    p->spmv_tpr = o.spmv_threads ? o.spmv_threads : tpr_of(p->Ah);
     // P1 hierarchy
     const int maxl = std::max(1, std::min(o.max_levels, (int)PKASP_MAX_LEVELS));
     p->lev.clear();
@@ -1247,7 +1226,7 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
     PK_CUDA(cudaMemsetAsync(p->d_bar_err, 0, sizeof(int), s));
     PK_CUDA(cudaStreamSynchronize(s));
     p->have_setup = true;
-    autotune(p, s);
+    choose_layouts(p, s);
 }
 
 void ensure_work(pkasp_problem *p, int ncols) {
@@ -1283,15 +1262,18 @@ void ensure_work(pkasp_problem *p, int ncols) {
 // ---------------------------------------------------------------------------------
 // public pieces
 // ---------------------------------------------------------------------------------
+namespace {
+// y = A x
+template <int TPR>
+__global__ void __launch_bounds__(kBlock) k_spmv_y(int64_t n, RowOp A, const double *__restrict__ x,
+                                                   double *__restrict__ y) {
+    for_rows<TPR>(n, A, x, [&](int64_t row, double s) { y[row] = s; });
+}
+}  // namespace
+
 void spmv_fine(pkasp_problem *p, const double *x, double *y, cudaStream_t s) {
-    if (p->spmv_tpr == 0) {
-        const DSell &S = p->Asell;
-        k_sell_spmv<double, double, double, double><<<elem_grid(p->nh), kBlock, 0, s>>>(
-            p->nh, S.sptr, S.swidth, S.col, S.val, x, y);
-        PK_LAUNCH();
-        return;
-    }
-    spmv<double, double>(p->Ah, x, y, p->spmv_tpr, s);
+    PK_FMT_SWITCH(p->spmv_tpr, (k_spmv_y<TPR><<<fine_grid(p), kBlock, 0, s>>>(p->nh, fine_op(p), x, y)));
+    PK_LAUNCH();
 }
 
 void apply_prec(pkasp_problem *p, const double *r, double *z, cudaStream_t s) {

@@ -120,3 +120,26 @@ def test_block_widths(ncols, prec, level_smoother, mode):
         assert abs(sc["iters"][0] - st["iters"][c]) <= 1
         assert (x[:, c] - xc).norm() <= 1e-8 * xc.norm()
     P.close()
+
+
+# one size for each shape of the SpMV's slices, and the product between set_kappa and setup
+@pytest.mark.parametrize("k,n", [(2, 8), (3, 12), (3, 16), (3, 24), (4, 20)])
+def test_spmv_slices(k, n):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    kap = kappa_lognormal(t.shape[0], 1)
+    P = Problem(xyz, t, k, kap)
+    x = torch.randn(P.nh, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    y0 = P.spmv(x)  # rows of the CSR form
+    P.setup()
+    assert P.info.spmv_layout > 500
+    # a row sum of L terms is off by at most L u sum |a x|, either way
+    bound = 2 * 400 * 2.0 ** -53 * P.spmv(x.abs()).abs().max() * 4
+    assert (P.spmv(x) - y0).abs().max() <= bound
+    P.set_kappa(kap)
+    assert torch.equal(P.spmv(x), y0)
+    P.close()
