@@ -372,11 +372,16 @@ int pkasp_destroy(pkasp_problem *p) {
     cudaDeviceSynchronize();
     pk::free_setup(p);
     pk::stokes_free(p);
+    p->work_pool.free_all();
     p->stage_pool.free_all();
     p->pool.free_all();
     pk::l2_window_release(p);
     if (p->aux_stream) cudaStreamDestroy(p->aux_stream);
-    if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
+    if (p->cap_stream) {
+        cudaStreamSynchronize(p->cap_stream);  // the frees of the setup's blocks
+        cudaStreamDestroy(p->cap_stream);
+    }
+    if (p->mem) cudaMemPoolDestroy(p->mem);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_join) cudaEventDestroy(p->ev_join);
     delete p;

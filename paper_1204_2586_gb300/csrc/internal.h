@@ -28,10 +28,23 @@ void launched(const char *file, int line);
 long long launch_count();
 #define PK_LAUNCH() ::pk::launched(__FILE__, __LINE__)
 
-// Device allocation tracked by the owning problem (freed in one place).
+// Device allocations freed in one place: cudaMalloc blocks, or (pool set) stream-ordered
+// blocks of a memory pool. A setup allocates and frees hundreds of blocks, and cudaMalloc and
+// cudaFree with the synchronisations they imply were 11 of its 28 ms at P3 24^3, so
+// pkasp_setup works on a pool of its problem: scratch pools made while a PoolScope is in
+// force on the thread use its pool and stream.
+struct PoolScope {
+    PoolScope(cudaMemPool_t pool, cudaStream_t s);
+    ~PoolScope();
+    static cudaMemPool_t pool();     // of the innermost scope of this thread (or null)
+    static cudaStream_t stream();
+};
 struct DevPool {
     std::vector<void *> blocks;
     size_t bytes = 0;
+    cudaMemPool_t mp;
+    cudaStream_t ms;  // allocates and frees; outlives the pool's blocks
+    DevPool() : mp(PoolScope::pool()), ms(PoolScope::stream()) {}
     void *alloc(size_t n);
     void free_all();
     template <class T>
@@ -163,6 +176,7 @@ struct PcgState {
 struct pkasp_problem {
     pk::DevPool pool;       // assembly-lifetime memory
     pk::DevPool setup_pool; // freed and rebuilt by every pkasp_setup
+    cudaMemPool_t mem = nullptr;  // pool of setup_pool and of a setup's scratch
     int device = 0;
     int k = 0, nloc = 0;
     int64_t nv = 0, nt = 0, n_all = 0, nh = 0, nH = 0;

@@ -1013,6 +1013,7 @@ void l2_window_release(pkasp_problem *p) {
 // setup orchestration
 // ---------------------------------------------------------------------------------
 void free_setup(pkasp_problem *p) {
+    cudaDeviceSynchronize();  // stream-ordered frees below: nothing may still read the blocks
     free_batched(p);
     free_gmres(p);
     stokes_free(p);  // its solver captured the preconditioner being replaced
@@ -1021,7 +1022,6 @@ void free_setup(pkasp_problem *p) {
     p->graph_exec = nullptr;
     p->graph = nullptr;
     p->setup_pool.free_all();
-    p->work_pool.free_all();
     p->lev.clear();
     p->fine = DSplit{};
     p->fsl = DSell{};
@@ -1041,7 +1041,6 @@ void free_setup(pkasp_problem *p) {
     p->d_bar = nullptr;
     p->d_bar_err = nullptr;
     p->d_cinv32 = nullptr;
-    p->work_cols = 0;
     p->have_setup = false;
 }
 
@@ -1130,8 +1129,51 @@ void choose_layouts(pkasp_problem *p, cudaStream_t s) {
     p->fine_tpr = lay == 0 ? fine_slices(p, s) : lay == 1 ? -1 : lay == 2 ? 0 : lay == 3 ? 2 : lay;
 }
 
+// The problem's memory pool, made at its first setup (null where the device has none: blocks
+// then come from cudaMalloc). It keeps what a setup frees until the setup's end.
+void setup_pool_open(pkasp_problem *p) {
+    if (p->mem) return;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = p->device;
+    uint64_t keep = UINT64_MAX;
+    if (cudaMemPoolCreate(&p->mem, &props) != cudaSuccess) {
+        cudaGetLastError();
+        p->mem = nullptr;
+        return;
+    }
+    PK_CUDA(cudaMemPoolSetAttribute(p->mem, cudaMemPoolAttrReleaseThreshold, &keep));
+}
+
+// gives back what the pool holds beyond the blocks in use and 64 MB
+void setup_pool_trim(pkasp_problem *p) {
+    uint64_t used = 0;
+    if (p->mem && cudaMemPoolGetAttribute(p->mem, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+        cudaMemPoolTrimTo(p->mem, (size_t)used + (64u << 20));
+    cudaGetLastError();
+}
+
+void setup_build(pkasp_problem *p, cudaStream_t s);
+
 void setup_device(pkasp_problem *p, cudaStream_t s) {
     free_setup(p);
+    if (!p->cap_stream) PK_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
+    setup_pool_open(p);
+    p->setup_pool.mp = p->mem;  // its blocks are gone
+    p->setup_pool.ms = p->cap_stream;
+    try {
+        PoolScope scope(p->mem, s);
+        setup_build(p, s);
+    } catch (...) {
+        cudaStreamSynchronize(s);
+        setup_pool_trim(p);
+        throw;
+    }
+    setup_pool_trim(p);
+}
+
+void setup_build(pkasp_problem *p, cudaStream_t s) {
     const pkasp_options &o = p->opt;
     const bool want32 = o.precond_precision == PKASP_PREC_FP32;
     l2_window_setup(p);
@@ -1212,7 +1254,6 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
             shaped_slices(p, L.A, L.sp, 2, L.ff, s);
         }
     if (!p->aux_stream) PK_CUDA(cudaStreamCreateWithFlags(&p->aux_stream, cudaStreamNonBlocking));
-    if (!p->cap_stream) PK_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
     if (!p->ev_fork) PK_CUDA(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
     if (!p->ev_join) PK_CUDA(cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming));
     ensure_work(p, 1);

@@ -26,14 +26,30 @@ void launched(const char *file, int line) {
 
 long long launch_count() { return g_launches.load(std::memory_order_relaxed); }
 
+namespace {
+thread_local cudaMemPool_t tl_pool = nullptr;
+thread_local cudaStream_t tl_stream = nullptr;
+}  // namespace
+PoolScope::PoolScope(cudaMemPool_t pool, cudaStream_t s) {
+    tl_pool = pool;
+    tl_stream = s;
+}
+PoolScope::~PoolScope() {
+    tl_pool = nullptr;
+    tl_stream = nullptr;
+}
+cudaMemPool_t PoolScope::pool() { return tl_pool; }
+cudaStream_t PoolScope::stream() { return tl_stream; }
+
 void *DevPool::alloc(size_t n) {
     void *p = nullptr;
     if (n == 0) n = 16;
     n = (n + 255) & ~(size_t)255;
-    cudaError_t e = cudaMalloc(&p, n);
+    cudaError_t e = mp ? cudaMallocFromPoolAsync(&p, n, mp, PoolScope::pool() == mp ? PoolScope::stream() : ms)
+                       : cudaMalloc(&p, n);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        fail(PKASP_ENOMEM, "cudaMalloc of " + std::to_string(n) + " bytes failed");
+        fail(PKASP_ENOMEM, "device allocation of " + std::to_string(n) + " bytes failed");
     }
     blocks.push_back(p);
     bytes += n;
@@ -41,7 +57,10 @@ void *DevPool::alloc(size_t n) {
 }
 
 void DevPool::free_all() {
-    for (void *p : blocks) cudaFree(p);
+    for (void *p : blocks) {
+        if (mp) cudaFreeAsync(p, ms);
+        else cudaFree(p);
+    }
     blocks.clear();
     bytes = 0;
 }
@@ -106,7 +125,9 @@ __global__ void k_scan_add(int64_t *d, int64_t n, const int64_t *tile_off) {
 void scan_rec(int64_t *d, int64_t n, cudaStream_t s, int64_t *total_out_dev) {
     int64_t ntiles = (n + kScanTile - 1) / kScanTile;
     int64_t *sums = nullptr;
-    PK_CUDA(cudaMallocAsync((void **)&sums, sizeof(int64_t) * (ntiles + 1), s));
+    if (PoolScope::pool())
+        PK_CUDA(cudaMallocFromPoolAsync((void **)&sums, sizeof(int64_t) * (ntiles + 1), PoolScope::pool(), s));
+    else PK_CUDA(cudaMallocAsync((void **)&sums, sizeof(int64_t) * (ntiles + 1), s));
     k_scan_tile<<<(unsigned)ntiles, kScanThreads, 0, s>>>(d, n, sums);
     PK_LAUNCH();
     if (ntiles > 1) {
