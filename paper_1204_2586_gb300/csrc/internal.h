@@ -318,6 +318,7 @@ void free_setup(pkasp_problem *p);
 int solve_device(pkasp_problem *p, const double *b_dev, double *x_dev, int ncols, int64_t ld,
                  pkasp_stats *st, cudaStream_t s);
 void apply_prec(pkasp_problem *p, const double *r, double *z, cudaStream_t s);
+bool apply_prec3(pkasp_problem *p, const double *r, double *z, double *zs, double *w, cudaStream_t s);
 void apply_smoother(pkasp_problem *p, const double *r, double *z, cudaStream_t s);
 void apply_vcycle(pkasp_problem *p, const double *b, double *x, cudaStream_t s);
 void spmv_fine(pkasp_problem *p, const double *x, double *y, cudaStream_t s);

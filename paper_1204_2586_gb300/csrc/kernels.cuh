@@ -359,11 +359,13 @@ __global__ void __launch_bounds__(kBlock) k_gs_phase(int64_t pb, int64_t pe, con
 // 2325 -> 1827, P4 24^3 597 -> 454, P3 32^3 359 -> 283, P2 33^3 129 -> 124, P2 8^3 46 -> 42;
 // FP32: P4 48^3 1379 -> 1240, P3 32^3 191 -> 170, P3 9^3 68 -> 66. At P4 48^3 FP64 it reads
 // about 1.0 sectors an entry at the 300 G sectors/s that random gathers reach there.
-template <int NB, typename PT, typename TR, bool BACK>
+//
+// NV vectors at once (r and y of vector v at r + v n, y + v n): the slice is read once.
+template <int NB, int NV, typename PT, typename TR, bool BACK>
 __global__ void __launch_bounds__(kBlock) k_slice_phase(int64_t s0, int64_t s1, const int4 *__restrict__ meta,
                                                         const int32_t *__restrict__ rows,
                                                         const PT *__restrict__ dinv, const int32_t *__restrict__ col,
-                                                        const PT *__restrict__ val, const TR *r, PT *y) {
+                                                        const PT *__restrict__ val, const TR *r, PT *y, int64_t n) {
     pdl_trigger();
     const int64_t s = s0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
@@ -387,12 +389,19 @@ __global__ void __launch_bounds__(kBlock) k_slice_phase(int64_t s0, int64_t s1, 
     const int32_t i = lead ? rows[m.z + q] : 0;
     const PT di = lead ? dinv[m.z + q] : PT(1);
     pdl_wait();
-    PT own = PT(0);
-    if (lead) own = BACK ? y[i] : (PT)r[i];
-    PT acc = PT(0);
+    PT own[NV], acc[NV];
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+        own[u] = PT(0);
+        if (lead) own[u] = BACK ? y[u * n + i] : (PT)r[u * n + i];
+        acc[u] = PT(0);
+    }
 #pragma unroll
     for (int k = 0; k < NB; ++k)
-        if (k < w && c[k] >= 0) acc += v[k] * y[c[k]];
+        if (k < w && c[k] >= 0) {
+#pragma unroll
+            for (int u = 0; u < NV; ++u) acc[u] += v[k] * y[u * n + c[k]];
+        }
     for (int k0 = NB; k0 < w; k0 += NB) {
 #pragma unroll
         for (int k = 0; k < NB; ++k) {
@@ -402,10 +411,19 @@ __global__ void __launch_bounds__(kBlock) k_slice_phase(int64_t s0, int64_t s1, 
         }
 #pragma unroll
         for (int k = 0; k < NB; ++k)
-            if (k0 + k < w && c[k] >= 0) acc += v[k] * y[c[k]];
+            if (k0 + k < w && c[k] >= 0) {
+#pragma unroll
+                for (int u = 0; u < NV; ++u) acc[u] += v[k] * y[u * n + c[k]];
+            }
     }
-    for (int o = 1 << lt >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
-    if (lead) y[i] = BACK ? own - acc * di : (own - acc) * di;
+    for (int o = 1 << lt >> 1; o > 0; o >>= 1) {
+#pragma unroll
+        for (int u = 0; u < NV; ++u) acc[u] += __shfl_xor_sync(kFull, acc[u], o);
+    }
+    if (lead) {
+#pragma unroll
+        for (int u = 0; u < NV; ++u) y[u * n + i] = BACK ? own[u] - acc[u] * di : (own[u] - acc[u]) * di;
+    }
 }
 
 // The loads of a colour phase without its dependency: every position of [0, n) at

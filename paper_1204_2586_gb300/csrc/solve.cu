@@ -272,20 +272,20 @@ void gs_backward0(const DSplit &sp, int tpr_fixed, PT *y, cudaStream_t s,
     }
 }
 
-// One sweep over the colours' interleaved slices, ascending or descending: BACK as in
-// k_slice_phase.
-template <typename PT, typename TR, bool BACK>
+// One sweep over the colours' interleaved slices, ascending or descending: BACK and NV as
+// in k_slice_phase (n: the length of a vector).
+template <typename PT, typename TR, bool BACK, int NV = 1>
 void slice_sweep(const DSlices &S, bool ascending, const TR *r, PT *y, cudaStream_t s,
-                 const cudaAccessPolicyWindow *win) {
+                 const cudaAccessPolicyWindow *win, int64_t n = 0) {
     const int nc = (int)S.off.size() - 1;
-    auto kern = S.nb == 2 ? k_slice_phase<2, PT, TR, BACK>
-                : S.nb == 4 ? k_slice_phase<4, PT, TR, BACK> : k_slice_phase<6, PT, TR, BACK>;
+    auto kern = S.nb == 2 ? k_slice_phase<2, NV, PT, TR, BACK>
+                : S.nb == 4 ? k_slice_phase<4, NV, PT, TR, BACK> : k_slice_phase<6, NV, PT, TR, BACK>;
     for (int q = 0; q < nc; ++q) {
         const int c = ascending ? q : nc - 1 - q;
         const int64_t s0 = S.off[c], s1 = S.off[c + 1];
         if (s1 <= s0) continue;
         launch_pdl_w(kern, rows_grid(s1 - s0, 32), s, win, s0, s1, (const int4 *)S.meta, (const int32_t *)S.rows,
-                     pick<PT>(S.dinv, S.dinv32), (const int32_t *)S.col, pick<PT>(S.val, S.val32), r, y);
+                     pick<PT>(S.dinv, S.dinv32), (const int32_t *)S.col, pick<PT>(S.val, S.val32), r, y, n);
     }
 }
 
@@ -1320,6 +1320,41 @@ void spmv_fine(pkasp_problem *p, const double *x, double *y, cudaStream_t s) {
 void apply_prec(pkasp_problem *p, const double *r, double *z, cudaStream_t s) {
     if (p->opt.precond_precision == PKASP_PREC_FP32) precondition<float>(p, r, z, s);
     else precondition<double>(p, r, z, s);
+}
+
+namespace {
+template <typename PT>
+void precondition3(pkasp_problem *p, const double *r, double *z, PT *zs, PT *w, cudaStream_t s) {
+    const int64_t n = p->nh, nH = p->nH;
+    PK_CUDA(cudaEventRecord(p->ev_fork, s));
+    PK_CUDA(cudaStreamWaitEvent(p->aux_stream, p->ev_fork, 0));
+    for (int c = 0; c < 3; ++c) {
+        restrict_vcycle<PT>(p, r + c * n, p->aux_stream);
+        PK_CUDA(cudaMemcpyAsync(w + c * nH, lv_x<PT>(p->lev[0]), sizeof(PT) * nH, cudaMemcpyDeviceToDevice,
+                                p->aux_stream));
+    }
+    slice_sweep<PT, double, false, 3>(p->fll, true, r, zs, s, nullptr, n);
+    slice_sweep<PT, PT, true, 3>(p->flu, false, zs, zs, s, nullptr, n);
+    PK_CUDA(cudaEventRecord(p->ev_join, p->aux_stream));
+    PK_CUDA(cudaStreamWaitEvent(s, p->ev_join, 0));
+    for (int c = 0; c < 3; ++c) {
+        k_prolong_add<PT, double><<<elem_grid(n), kBlock, 0, s>>>(n, p->Pi.ptr, p->Pi.col,
+                                                                  pick<PT>(p->Pi.val, p->Pi.val32), w + c * nH,
+                                                                  zs + c * n, z + c * n);
+        PK_LAUNCH();
+    }
+}
+}  // namespace
+
+// z = B r for three vectors of n_h entries one after another, where their sweeps can share
+// the matrix (the additive form with slices); zs and w: 3 n_h and 3 n_H entries of scratch
+// (FP64 size). False: not this preconditioner, nothing done.
+bool apply_prec3(pkasp_problem *p, const double *r, double *z, double *zs, double *w, cudaStream_t s) {
+    if (p->opt.mode != PKASP_MODE_ADDITIVE || p->opt.smoother != PKASP_SMOOTHER_SGS || p->fine_tpr <= 500) return false;
+    if (p->opt.precond_precision == PKASP_PREC_FP32)
+        precondition3<float>(p, r, z, reinterpret_cast<float *>(zs), reinterpret_cast<float *>(w), s);
+    else precondition3<double>(p, r, z, zs, w, s);
+    return true;
 }
 
 void apply_smoother(pkasp_problem *p, const double *r, double *z, cudaStream_t s) {

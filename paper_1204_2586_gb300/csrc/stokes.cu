@@ -27,6 +27,7 @@ struct StokesWork {
     // preconditioner work
     double *t = nullptr, *rr = nullptr, *zz = nullptr, *pp = nullptr, *qq = nullptr, *xp = nullptr;
     double *scal = nullptr;  // rho, alpha, beta of the inner CG
+    double *zs3 = nullptr, *w3 = nullptr;  // the three components' smoothed and coarse parts
     // FGMRES
     int m = 0;
     double *V = nullptr, *Z = nullptr, *w = nullptr, *vin = nullptr, *zout = nullptr, *y = nullptr;
@@ -295,7 +296,10 @@ void prec(pkasp_problem *p, const double *r, double *z, cudaStream_t s) {
     PK_LAUNCH();
     ks_tsub<<<grid_for(nu), kBlock, 0, s>>>(nu, S.BT.ptr, S.BT.col, S.BT.val, z + nu, r, S.t);
     PK_LAUNCH();
-    for (int c = 0; c < 3; ++c) apply_prec(p, S.t + c * nh, z + c * nh, s);
+    // the components' sweeps share each read of a slice and each launch (a solve at P2 12^3:
+    // 20.5 ms against 23.1 with three applications one after another)
+    if (!apply_prec3(p, S.t, z, S.zs3, S.w3, s))
+        for (int c = 0; c < 3; ++c) apply_prec(p, S.t + c * nh, z + c * nh, s);
 }
 
 struct StokesGmres {
@@ -476,6 +480,8 @@ void stokes_setup(pkasp_problem *p, int mp_iters, cudaStream_t s) {
         tmp.free_all();
     }
     const int64_t nu = std::max<int64_t>(3 * p->nh, 1), npp = std::max<int64_t>(np, 1);
+    S.zs3 = S.pool.get<double>(3 * std::max<int64_t>(p->nh, 1));
+    S.w3 = S.pool.get<double>(3 * std::max<int64_t>(p->nH, 1));
     S.t = S.pool.get<double>(nu);
     S.rr = S.pool.get<double>(npp);
     S.zz = S.pool.get<double>(npp);
