@@ -227,6 +227,8 @@ struct pkasp_problem {
     int tail = 0;               // level from which one right-hand side's V-cycle is a dense product
     double *d_tail = nullptr;   // its matrix (FP64 or FP32, as the cycle runs; tail.cu); the
     float *d_tail32 = nullptr;  // coarsest inverse when tail is the coarsest level
+    double *d_dense = nullptr;   // B of a small problem (FP64 or FP32; tail.cu), else null
+    float *d_dense32 = nullptr;
     int64_t *d_fine_off = nullptr;  // device copy of fine.off (persistent smoother)
     unsigned *d_bar = nullptr;      // grid-barrier arrivals / exits of the persistent smoother
     int *d_bar_err = nullptr;       // set when one of its barriers timed out

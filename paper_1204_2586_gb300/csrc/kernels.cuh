@@ -720,12 +720,12 @@ __global__ void __launch_bounds__(kBlock) k_prolong_inplace(int64_t n, const int
     if (ok && sub == 0) x[row] = xi + s;
 }
 
-// x = M b for the dense tail of the V-cycle (one warp per row; small blocks, so that a few
+// x = M b for the dense tail of the V-cycle or a small problem's whole preconditioner (one warp per row; small blocks, so that a few
 // hundred rows spread over the chip). Bound by reading M: eight loads in flight per lane
 // and four partial sums.
-template <typename PT>
-__global__ void __launch_bounds__(128) k_dense_mv(int64_t n, const PT *__restrict__ M, const PT *__restrict__ b,
-                                                  PT *__restrict__ x) {
+template <typename PT, typename TB, typename TX>
+__global__ void __launch_bounds__(128) k_dense_mv(int64_t n, const PT *__restrict__ M, const TB *__restrict__ b,
+                                                  TX *__restrict__ x) {
     const int lane = threadIdx.x & 31;
     const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (row >= n) return;  // whole warp leaves together
@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(128) k_dense_mv(int64_t n, const PT *__restric
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             u[k] = ldg(&m[j + 32 * k]);
-            v[k] = ldg(&b[j + 32 * k]);
+            v[k] = (PT)ldg(&b[j + 32 * k]);
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) acc[k & 3] += u[k] * v[k];
@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(128) k_dense_mv(int64_t n, const PT *__restric
     for (int k = 0; k < 8; ++k) {
         const bool in = j + 32 * k < n;
         u[k] = in ? ldg(&m[j + 32 * k]) : PT(0);
-        v[k] = in ? ldg(&b[j + 32 * k]) : PT(0);
+        v[k] = in ? (PT)ldg(&b[j + 32 * k]) : PT(0);
     }
 #pragma unroll
     for (int k = 0; k < 8; ++k)
@@ -755,7 +755,7 @@ __global__ void __launch_bounds__(128) k_dense_mv(int64_t n, const PT *__restric
     PT s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    if (lane == 0) x[row] = s;
+    if (lane == 0) x[row] = (TX)s;
 }
 
 // ---------------------------------------------------------------------------------

@@ -359,7 +359,7 @@ void vcycle(pkasp_problem *p, int l, cudaStream_t s, bool pre_done) {
     Level &L = p->lev[l];
     const int64_t n = L.A.n;
     if (l == p->tail) {
-        k_dense_mv<PT><<<(unsigned)((n + 3) / 4), 128, 0, s>>>(n, pick<PT>(p->d_tail, p->d_tail32), lv_b<PT>(L),
+        k_dense_mv<PT, PT, PT><<<(unsigned)((n + 3) / 4), 128, 0, s>>>(n, pick<PT>(p->d_tail, p->d_tail32), lv_b<PT>(L),
                                                                lv_x<PT>(L));
         PK_LAUNCH();
         return;
@@ -529,6 +529,18 @@ void precondition(pkasp_problem *p, const double *r, double *z, cudaStream_t s, 
         to_pt<PT>(r, lv_b<PT>(L0), p->nh, s);
         vcycle<PT>(p, 0, s);
         k_copy_to<PT><<<elem_grid(p->nh), kBlock, 0, s>>>(p->nh, lv_x<PT>(L0), z);
+        PK_LAUNCH();
+        return;
+    }
+    if (pick<PT>(p->d_dense, p->d_dense32)) {
+        const unsigned g = (unsigned)((p->nh + 3) / 4);
+        if constexpr (std::is_same<PT, float>::value) {
+            // r rounded once: conversions run on the FP64 pipe
+            to_pt<float>(r, p->w_rr32, p->nh, s);
+            k_dense_mv<float, float, double><<<g, 128, 0, s>>>(p->nh, p->d_dense32, p->w_rr32, z);
+        } else {
+            k_dense_mv<double, double, double><<<g, 128, 0, s>>>(p->nh, p->d_dense, r, z);
+        }
         PK_LAUNCH();
         return;
     }
@@ -1036,6 +1048,8 @@ void free_setup(pkasp_problem *p) {
     p->d_cinv = nullptr;
     p->d_tail = nullptr;
     p->d_tail32 = nullptr;
+    p->d_dense = nullptr;
+    p->d_dense32 = nullptr;
     p->tail = 0;
     p->d_fine_off = nullptr;
     p->d_bar = nullptr;
@@ -1350,7 +1364,9 @@ void precondition3(pkasp_problem *p, const double *r, double *z, PT *zs, PT *w, 
 // the matrix (the additive form with slices); zs and w: 3 n_h and 3 n_H entries of scratch
 // (FP64 size). False: not this preconditioner, nothing done.
 bool apply_prec3(pkasp_problem *p, const double *r, double *z, double *zs, double *w, cudaStream_t s) {
-    if (p->opt.mode != PKASP_MODE_ADDITIVE || p->opt.smoother != PKASP_SMOOTHER_SGS || p->fine_tpr <= 500) return false;
+    if (p->opt.mode != PKASP_MODE_ADDITIVE || p->opt.smoother != PKASP_SMOOTHER_SGS || p->fine_tpr <= 500 ||
+        p->d_dense || p->d_dense32)
+        return false;
     if (p->opt.precond_precision == PKASP_PREC_FP32)
         precondition3<float>(p, r, z, reinterpret_cast<float *>(zs), reinterpret_cast<float *>(w), s);
     else precondition3<double>(p, r, z, zs, w, s);
@@ -1412,7 +1428,7 @@ void enqueue_iteration(pkasp_problem *p, double *x, cudaStream_t s) {
                                                   p->d_counter, p->d_hist);
     PK_LAUNCH();
     const int flex = (p->opt.flexible || p->opt.precond_precision == PKASP_PREC_FP32) ? 1 : 0;
-    if (p->opt.mode == PKASP_MODE_ADDITIVE) {
+    if (p->opt.mode == PKASP_MODE_ADDITIVE && !p->d_dense && !p->d_dense32) {
         // additive preconditioner up to z_s and w; z = z_s + Pi w inside the beta kernel
         const PiCodes &pc = p->pic;
         if (p->opt.precond_precision == PKASP_PREC_FP32) {

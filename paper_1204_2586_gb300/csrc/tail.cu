@@ -35,22 +35,24 @@ __global__ void __launch_bounds__(kCols) k_tail_rows(int64_t n, int64_t p0, cons
     Y[r * n + c] = (r == c ? ident : 0.0) + own + sign * acc;
 }
 
-// one Gauss-Seidel colour: X_r = (I_r - sum_lower a X - [full] sum_upper a X) * dinv
+// one Gauss-Seidel colour: X_r = (I_r - sum_lower a X - [full] sum_upper a X) * dinv; or
+// (back) the second half of the symmetric sweep, X_r -= (sum_upper a X) * dinv
 __global__ void __launch_bounds__(kCols) k_tail_gs(int64_t n, int64_t p0, const int32_t *__restrict__ rows,
                                                    const int64_t *__restrict__ lptr,
                                                    const int32_t *__restrict__ lcol,
                                                    const double *__restrict__ lval, const int64_t *__restrict__ uptr,
                                                    const int32_t *__restrict__ ucol,
                                                    const double *__restrict__ uval, const double *__restrict__ dinv,
-                                                   int full, double *X) {
+                                                   int full, int back, double *X) {
     const int64_t p = p0 + blockIdx.x, c = (int64_t)blockIdx.y * kCols + threadIdx.x;
     if (c >= n) return;
     const int64_t r = rows[p];
     double acc = 0.0;
-    for (int64_t e = lptr[p]; e < lptr[p + 1]; ++e) acc += lval[e] * X[(int64_t)lcol[e] * n + c];
-    if (full)
+    if (!back)
+        for (int64_t e = lptr[p]; e < lptr[p + 1]; ++e) acc += lval[e] * X[(int64_t)lcol[e] * n + c];
+    if (full || back)
         for (int64_t e = uptr[p]; e < uptr[p + 1]; ++e) acc += uval[e] * X[(int64_t)ucol[e] * n + c];
-    X[r * n + c] = ((r == c ? 1.0 : 0.0) - acc) * dinv[p];
+    X[r * n + c] = back ? X[r * n + c] - acc * dinv[p] : ((r == c ? 1.0 : 0.0) - acc) * dinv[p];
 }
 
 // X = D^{-1} (the l1-Jacobi step from zero on the identity); X += D^{-1} R
@@ -90,6 +92,22 @@ __global__ void __launch_bounds__(256) k_tail_gemm(int64_t m, int64_t n, int64_t
         if (i0 + ty + 8 * q < m) C[(i0 + ty + 8 * q) * n + j] = acc[q];
 }
 
+// X += I_P M I_P^T (rows of I_P have at most four entries)
+__global__ void __launch_bounds__(kCols) k_tail_coarse(int64_t n, int64_t nc, const int64_t *__restrict__ ptr,
+                                                       const int32_t *__restrict__ col,
+                                                       const double *__restrict__ val, const double *__restrict__ M,
+                                                       double *__restrict__ X) {
+    const int64_t r = blockIdx.x, c = (int64_t)blockIdx.y * kCols + threadIdx.x;
+    if (c >= n) return;
+    double acc = 0.0;
+    for (int64_t e = ptr[r]; e < ptr[r + 1]; ++e) {
+        double t = 0.0;
+        for (int64_t f = ptr[c]; f < ptr[c + 1]; ++f) t += M[(int64_t)col[e] * nc + col[f]] * val[f];
+        acc += val[e] * t;
+    }
+    X[r * n + c] += acc;
+}
+
 // Modelled time (us) of one cycle from level l down, as launches. Gauss-Seidel: a launch
 // per colour and sweep, 3.4 us each (P2 21^3 FP64, 202 phases of three levels: 709 us);
 // l1-Jacobi: five launches of 2 us each besides the next level (P2 8^3: 18 us over two
@@ -123,13 +141,53 @@ int tail_level(const pkasp_problem *p) {
     return best;
 }
 
-// M = V on level p->tail, from the coarsest inverse up; into d_tail (or d_tail32)
+// Whether the whole additive preconditioner B = S_k + I_P V I_P^T of a small problem is
+// applied as one dense product: its sweeps cost 1.5 us a phase (P2 8^3, 3375 unknowns, FP64:
+// B 42 us as launches; FP32 33). Within 3400 rows (92 MB, read from L2) and 6 10^8 FMAs of
+// setup work (about 1 ms). An explicit layout of the smoother keeps its sweeps.
+bool dense_prec(const pkasp_problem *p) {
+    const pkasp_options &o = p->opt;
+    if (o.mode != PKASP_MODE_ADDITIVE || o.smoother != PKASP_SMOOTHER_SGS || o.smoother_layout != 0 ||
+        o.spmv_threads != 0 || p->tail != 0)
+        return false;
+    const double n = (double)p->nh;
+    return p->nh <= 3400 && n * (double)p->Ah.nnz <= 6e8 &&
+           dense_us(n, o.precond_precision == PKASP_PREC_FP32) < 3.0 * p->fine.ncol;
+}
+
+// B from M = V on level 0 (n_H x n_H, FP64)
+void build_dense_prec(pkasp_problem *p, const double *M, DevPool &tmp, cudaStream_t s) {
+    const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
+    const int64_t n = p->nh;
+    double *X = (fp32 ? tmp : p->setup_pool).get<double>(n * n);
+    const DSplit &sp = p->fine;
+    for (int q = 0; q < 2 * sp.ncol; ++q) {
+        const int back = q >= sp.ncol, c = back ? 2 * sp.ncol - 1 - q : q;
+        const int64_t pb = sp.off[c], m = sp.off[c + 1] - pb;
+        if (m == 0) continue;
+        k_tail_gs<<<dim3((unsigned)m, tiles(n)), kCols, 0, s>>>(n, pb, sp.perm, sp.lptr, sp.lcol, sp.lval, sp.uptr,
+                                                                sp.ucol, sp.uval, sp.dinv, 0, back, X);
+        PK_LAUNCH();
+    }
+    k_tail_coarse<<<dim3((unsigned)n, tiles(n)), kCols, 0, s>>>(n, p->nH, p->Pi.ptr, p->Pi.col, p->Pi.val, M, X);
+    PK_LAUNCH();
+    if (fp32) {
+        p->d_dense32 = p->setup_pool.get<float>(n * n);
+        to32(X, p->d_dense32, n * n, s);
+    } else {
+        p->d_dense = X;
+    }
+}
+
+// M = V on level p->tail, from the coarsest inverse up; into d_tail (or d_tail32); then the
+// whole preconditioner of a small problem
 void build_tail(pkasp_problem *p, cudaStream_t s) {
     const int last = (int)p->lev.size() - 1;
     p->tail = tail_level(p);
     p->d_tail = p->d_cinv;
     p->d_tail32 = p->d_cinv32;
-    if (p->tail == last) return;
+    const bool dense = dense_prec(p);
+    if (p->tail == last && !dense) return;
     const bool jacobi = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
     const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
     DevPool tmp;
@@ -147,7 +205,7 @@ void build_tail(pkasp_problem *p, cudaStream_t s) {
                 const int64_t pb = sp.off[c], m = sp.off[c + 1] - pb;
                 if (m == 0) return;
                 k_tail_gs<<<dim3((unsigned)m, ct), kCols, 0, s>>>(n, pb, sp.perm, sp.lptr, sp.lcol, sp.lval, sp.uptr,
-                                                                  sp.ucol, sp.uval, sp.dinv, full, X);
+                                                                  sp.ucol, sp.uval, sp.dinv, full, 0, X);
                 PK_LAUNCH();
             };
             auto residual = [&] {  // R = I - A X
@@ -180,8 +238,11 @@ void build_tail(pkasp_problem *p, cudaStream_t s) {
             }
             Mc = X;
         }
+        if (dense) build_dense_prec(p, Mc, tmp, s);
         const int64_t n = p->lev[p->tail].A.n;
-        if (fp32) {
+        if (p->tail == last) {
+            // the coarsest inverse itself
+        } else if (fp32) {
             p->d_tail32 = p->setup_pool.get<float>(n * n);
             to32(Mc, p->d_tail32, n * n, s);
             p->d_tail = nullptr;
