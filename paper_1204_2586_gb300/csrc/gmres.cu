@@ -94,12 +94,12 @@ struct Gmres {
         PK_FMT_SWITCH(p->spmv_tpr, (kg_spmv_w<TPR><<<fine_grid(p), kBlock, 0, s>>>(n, A, p->gm_zout, p->gm_w, p->gm_Z,
                                                                               p->gm_state)));
         PK_LAUNCH();
-        const dim3 dg(kDotChunks, p->gm_m + 1);
+        const dim3 dg(dot_chunks(n), p->gm_m + 1);
         for (int pass = 0; pass < 2; ++pass) {
             kg_dots<<<dg, kBlock, 0, s>>>(n, p->gm_V, p->gm_w, p->gm_state, p->gm_part, p->gm_cnt, p->gm_hc,
                                           p->gm_H, pass);
             PK_LAUNCH();
-            kg_axpy<<<kRedGrid, kBlock, 0, s>>>(n, p->gm_V, p->gm_w, p->gm_state, p->gm_hc, p->gm_H, p->d_partials,
+            kg_axpy<<<red_grid(n), kBlock, 0, s>>>(n, p->gm_V, p->gm_w, p->gm_state, p->gm_hc, p->gm_H, p->d_partials,
                                                 p->d_counter, pass);
             PK_LAUNCH();
         }

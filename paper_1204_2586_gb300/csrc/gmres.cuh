@@ -192,6 +192,8 @@ __global__ void kg_loop_control(GmresState *st, cudaGraphConditionalHandle h) {
     cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
+// chunks of kg_dots: at most kDotChunks, at least 512 elements each
+unsigned dot_chunks(int64_t n) { return (unsigned)std::min<int64_t>(kDotChunks, std::max<int64_t>(1, (n + 511) / 512)); }
 unsigned elem_blocks(int64_t n) { return (unsigned)std::min<int64_t>(152 * 8, std::max<int64_t>(1, (n + kBlock - 1) / kBlock)); }
 
 // v0 = b - y (y = A x computed by the caller) and its norm. first: the solve's start

@@ -18,7 +18,12 @@ namespace pk {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kBlock = 256;
-constexpr int kRedGrid = 152 * 4;  // fixed grid of the reduction kernels
+constexpr int kRedGrid = 152 * 4;  // most blocks of the reduction kernels
+// Grid of an element-wise reduction over n elements: one element a thread up to kRedGrid
+// blocks. On a short vector the atomics of 608 arriving blocks cost more than the sums.
+inline unsigned red_grid(int64_t n) {
+    return (unsigned)(n <= kBlock ? 1 : n >= (int64_t)kRedGrid * kBlock ? kRedGrid : (n + kBlock - 1) / kBlock);
+}
 
 template <typename T>
 __device__ __forceinline__ T ldg(const T *p) {
@@ -78,7 +83,7 @@ __device__ __forceinline__ A row_dot(int64_t lo, int64_t hi, int sub, const int3
 //    partials[block].
 //  - grid_reduce: the last block to arrive (fence and atomic counter) adds the block
 //    partials with strided_sum and a block tree.
-// The PCG's reductions run in element-wise kernels of kRedGrid blocks. GB300 issues one
+// The PCG's reductions run in element-wise kernels of at most kRedGrid blocks. GB300 issues one
 // warp-wide FP64 instruction per 16 cycles per SM, so a shuffle tree of doubles at the
 // end of every warp of a one-row-per-thread SpMV (5 adds per 32 rows) costs about as
 // much as streaming the operand vectors once more: the PCG's fine SpMV writes q only,

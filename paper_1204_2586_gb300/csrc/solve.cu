@@ -643,7 +643,7 @@ __global__ void k_state_restart(PcgState *st) {
 
 // The fine-operator kernels (one thread or lane group per row, tens of thousands of
 // blocks) only write vectors; every dot product and norm is taken by an element-wise
-// kernel of kRedGrid blocks (grid_reduce). Each thread of those loads kVec elements
+// kernel of red_grid blocks (grid_reduce). Each thread of those loads kVec elements
 // (i, i + stride, ...) before it computes, and adds its terms in ascending i as a
 // one-at-a-time loop would.
 constexpr int kVec = 4;
@@ -760,12 +760,30 @@ __global__ void __launch_bounds__(kBlock) k_pq_alpha(int64_t n, const double *__
     }
 }
 
+// Loop control of the captured while node: continue unless stopped; a safety bound on the
+// number of passes stops the loop even if no kernel set the flag. The kernel that decides
+// the stop sets the condition itself: a kernel of its own cost a launch of 1.7 us in every
+// pass. graph = 0: eager launches, the host reads the flag.
+struct LoopNode {
+    cudaGraphConditionalHandle h;
+    int graph;
+};
+__device__ __forceinline__ void loop_control(PcgState *st, const LoopNode &loop) {
+    if (!loop.graph) return;
+    const int loops = ++st->loops;
+    const bool go = !st->all_done && loops <= st->maxit + 2;
+    cudaGraphSetConditional(loop.h, go ? 1u : 0u);
+}
+
 // x += alpha p, r -= alpha q, ||r||, convergence test
 __global__ void __launch_bounds__(kBlock) k_update_xr(int64_t n, double *__restrict__ x, double *__restrict__ r,
                                                       const double *__restrict__ p, const double *__restrict__ q,
                                                       PcgState *st, double *partials, unsigned *counter,
-                                                      double *hist) {
-    if (st->done[0]) return;
+                                                      double *hist, LoopNode loop) {
+    if (st->done[0]) {  // stopped before this pass: no block writes the flag in it
+        if (blockIdx.x == 0 && threadIdx.x == 0) loop_control(st, loop);
+        return;
+    }
     const double a = st->alpha[0];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     double part = 0.0;
@@ -808,6 +826,7 @@ __global__ void __launch_bounds__(kBlock) k_update_xr(int64_t n, double *__restr
             st->status[0] = PKASP_ENOTCONV;
             st->all_done = 1;
         }
+        loop_control(st, loop);
     }
 }
 
@@ -927,15 +946,6 @@ __global__ void __launch_bounds__(kBlock) k_update_p(int64_t n, const double *__
             if (i < n) p[i] = zv[u] + b * pv[u];
         }
     }
-}
-
-// loop control of the captured while node: continue unless stopped; a safety bound on
-// the number of passes stops the loop even if no kernel set the flag
-__global__ void k_loop_control(PcgState *st, cudaGraphConditionalHandle h) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int loops = ++st->loops;
-    bool go = !st->all_done && loops <= st->maxit + 2;
-    cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
 // true residual norm ||t|| (t = b - A x) into st->tnorm
@@ -1407,25 +1417,25 @@ void enqueue_init(pkasp_problem *p, const double *b, double *x, cudaStream_t s) 
     const unsigned fg = fine_grid(p);
     PK_FMT_SWITCH(tpr, (k_residual_fine<TPR><<<fg, kBlock, 0, s>>>(p->nh, A, b, x, p->w_r)));
     PK_LAUNCH();
-    k_init_norm<<<kRedGrid, kBlock, 0, s>>>(p->nh, p->w_r, p->d_state, p->d_partials, p->d_counter, p->d_hist);
+    k_init_norm<<<red_grid(p->nh), kBlock, 0, s>>>(p->nh, p->w_r, p->d_state, p->d_partials, p->d_counter, p->d_hist);
     PK_LAUNCH();
     apply_prec(p, p->w_r, p->w_z, s);
-    k_start<<<kRedGrid, kBlock, 0, s>>>(p->nh, p->w_r, p->w_z, p->w_p, p->d_state, p->d_partials,
+    k_start<<<red_grid(p->nh), kBlock, 0, s>>>(p->nh, p->w_r, p->w_z, p->w_p, p->d_state, p->d_partials,
                                               p->d_counter);
     PK_LAUNCH();
 }
 
 
-void enqueue_iteration(pkasp_problem *p, double *x, cudaStream_t s) {
+void enqueue_iteration(pkasp_problem *p, double *x, const LoopNode &loop, cudaStream_t s) {
     const int tpr = p->spmv_tpr;
     const RowOp A = fine_op(p);
     const unsigned fg = fine_grid(p);
     PK_FMT_SWITCH(tpr, (k_spmv_q<TPR><<<fg, kBlock, 0, s>>>(p->nh, A, p->w_p, p->w_q, p->d_state)));
     PK_LAUNCH();
-    k_pq_alpha<<<kRedGrid, kBlock, 0, s>>>(p->nh, p->w_p, p->w_q, p->d_state, p->d_partials, p->d_counter);
+    k_pq_alpha<<<red_grid(p->nh), kBlock, 0, s>>>(p->nh, p->w_p, p->w_q, p->d_state, p->d_partials, p->d_counter);
     PK_LAUNCH();
-    k_update_xr<<<kRedGrid, kBlock, 0, s>>>(p->nh, x, p->w_r, p->w_p, p->w_q, p->d_state, p->d_partials,
-                                                  p->d_counter, p->d_hist);
+    k_update_xr<<<red_grid(p->nh), kBlock, 0, s>>>(p->nh, x, p->w_r, p->w_p, p->w_q, p->d_state, p->d_partials,
+                                                  p->d_counter, p->d_hist, loop);
     PK_LAUNCH();
     const int flex = (p->opt.flexible || p->opt.precond_precision == PKASP_PREC_FP32) ? 1 : 0;
     if (p->opt.mode == PKASP_MODE_ADDITIVE && !p->d_dense && !p->d_dense32) {
@@ -1433,22 +1443,22 @@ void enqueue_iteration(pkasp_problem *p, double *x, cudaStream_t s) {
         const PiCodes &pc = p->pic;
         if (p->opt.precond_precision == PKASP_PREC_FP32) {
             precondition<float>(p, p->w_r, p->w_z, s, false);
-            k_prolong_beta<float><<<kRedGrid, kBlock, 0, s>>>(
+            k_prolong_beta<float><<<red_grid(p->nh), kBlock, 0, s>>>(
                 p->nh, (const int4 *)pc.ell_col, pc.ell_code, pc.tab32, p->lev[0].x32, p->w_zs32, p->w_r, p->w_q,
                 p->w_z, flex, p->d_state, p->d_partials, p->d_counter);
         } else {
             precondition<double>(p, p->w_r, p->w_z, s, false);
-            k_prolong_beta<double><<<kRedGrid, kBlock, 0, s>>>(
+            k_prolong_beta<double><<<red_grid(p->nh), kBlock, 0, s>>>(
                 p->nh, (const int4 *)pc.ell_col, pc.ell_code, pc.tab, p->lev[0].x, p->w_zs, p->w_r, p->w_q,
                 p->w_z, flex, p->d_state, p->d_partials, p->d_counter);
         }
     } else {
         apply_prec(p, p->w_r, p->w_z, s);
-        k_beta<<<kRedGrid, kBlock, 0, s>>>(p->nh, p->w_r, p->w_z, p->w_q, flex, p->d_state, p->d_partials,
+        k_beta<<<red_grid(p->nh), kBlock, 0, s>>>(p->nh, p->w_r, p->w_z, p->w_q, flex, p->d_state, p->d_partials,
                                                  p->d_counter);
     }
     PK_LAUNCH();
-    k_update_p<<<kRedGrid, kBlock, 0, s>>>(p->nh, p->w_z, p->w_p, p->d_state);
+    k_update_p<<<red_grid(p->nh), kBlock, 0, s>>>(p->nh, p->w_z, p->w_p, p->d_state);
     PK_LAUNCH();
 }
 
@@ -1459,7 +1469,7 @@ void enqueue_final(pkasp_problem *p, const double *b, const double *x, cudaStrea
     // the residual goes to a work vector the iteration no longer needs
     PK_FMT_SWITCH(tpr, (k_residual_fine<TPR><<<fg, kBlock, 0, s>>>(p->nh, A, b, x, p->w_t)));
     PK_LAUNCH();
-    k_true_norm<<<kRedGrid, kBlock, 0, s>>>(p->nh, p->w_t, p->d_state, p->d_partials, p->d_counter);
+    k_true_norm<<<red_grid(p->nh), kBlock, 0, s>>>(p->nh, p->w_t, p->d_state, p->d_partials, p->d_counter);
     PK_LAUNCH();
 }
 
@@ -1490,9 +1500,7 @@ void build_graph(pkasp_problem *p, const double *b, double *x) {
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     PK_CUDA(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     c0 = launch_count();
-    enqueue_iteration(p, x, cs);
-    k_loop_control<<<1, 32, 0, cs>>>(p->d_state, h);
-    PK_LAUNCH();
+    enqueue_iteration(p, x, LoopNode{h, 1}, cs);
     p->g_body = launch_count() - c0;
     PK_CUDA(cudaStreamEndCapture(cs, &body));
     // final true residual
@@ -1557,7 +1565,7 @@ int solve_device(pkasp_problem *p, const double *b, double *x, int ncols, int64_
         } else {
             enqueue_init(p, b, x, s);
             for (int it = 0; it <= p->opt.max_iter + 1; ++it) {
-                enqueue_iteration(p, x, s);
+                enqueue_iteration(p, x, LoopNode{}, s);
                 int ad = 0;
                 PK_CUDA(cudaMemcpyAsync(&ad, &p->d_state->all_done, sizeof(int), cudaMemcpyDeviceToHost, s));
                 PK_CUDA(cudaStreamSynchronize(s));

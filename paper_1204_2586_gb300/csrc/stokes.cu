@@ -270,7 +270,7 @@ void op(pkasp_problem *p, const double *x, double *y, const int *gate, cudaStrea
     }
     ks_add_csr<<<grid_for(nu), kBlock, 0, s>>>(nu, S.BT.ptr, S.BT.col, S.BT.val, x + nu, y, gate);
     PK_LAUNCH();
-    ks_spmv_rows<<<kRedGrid, kBlock, 0, s>>>(S.np, S.B.ptr, S.B.col, S.B.val, x, y + nu, gate);
+    ks_spmv_rows<<<red_grid(S.np * 8), kBlock, 0, s>>>(S.np, S.B.ptr, S.B.col, S.B.val, x, y + nu, gate);
     PK_LAUNCH();
 }
 
@@ -278,15 +278,15 @@ void op(pkasp_problem *p, const double *x, double *y, const int *gate, cudaStrea
 void prec(pkasp_problem *p, const double *r, double *z, cudaStream_t s) {
     StokesWork &S = *p->st;
     const int64_t nh = S.nh, nu = 3 * nh, np = S.np;
-    ks_mp_start<<<kRedGrid, kBlock, 0, s>>>(np, r + nu, S.mdiag, S.rr, S.zz, S.pp, S.xp, S.scal, p->d_partials,
+    ks_mp_start<<<red_grid(np), kBlock, 0, s>>>(np, r + nu, S.mdiag, S.rr, S.zz, S.pp, S.xp, S.scal, p->d_partials,
                                             p->d_counter);
     PK_LAUNCH();
     for (int it = 0; it < S.mp_iters; ++it) {
-        ks_spmv_rows<<<kRedGrid, kBlock, 0, s>>>(np, S.M.ptr, S.M.col, S.M.val, S.pp, S.qq, nullptr);
+        ks_spmv_rows<<<red_grid(np * 8), kBlock, 0, s>>>(np, S.M.ptr, S.M.col, S.M.val, S.pp, S.qq, nullptr);
         PK_LAUNCH();
-        ks_mp_alpha<<<kRedGrid, kBlock, 0, s>>>(np, S.pp, S.qq, S.scal, p->d_partials, p->d_counter);
+        ks_mp_alpha<<<red_grid(np), kBlock, 0, s>>>(np, S.pp, S.qq, S.scal, p->d_partials, p->d_counter);
         PK_LAUNCH();
-        ks_mp_update<<<kRedGrid, kBlock, 0, s>>>(np, S.xp, S.rr, S.zz, S.pp, S.qq, S.mdiag, S.scal, p->d_partials,
+        ks_mp_update<<<red_grid(np), kBlock, 0, s>>>(np, S.xp, S.rr, S.zz, S.pp, S.qq, S.mdiag, S.scal, p->d_partials,
                                                  p->d_counter);
         PK_LAUNCH();
         ks_mp_p<<<grid_for(np), kBlock, 0, s>>>(np, S.zz, S.pp, S.scal);
@@ -306,7 +306,7 @@ struct StokesGmres {
     static void init(pkasp_problem *p, const double *b, double *x, cudaStream_t s) {
         StokesWork &S = *p->st;
         op(p, x, S.y, nullptr, s);
-        kg_residual_y<<<kRedGrid, kBlock, 0, s>>>(S.n, b, S.y, S.V, S.state, S.g, p->d_partials, p->d_counter, S.hist,
+        kg_residual_y<<<red_grid(S.n), kBlock, 0, s>>>(S.n, b, S.y, S.V, S.state, S.g, p->d_partials, p->d_counter, S.hist,
                                                   1);
         PK_LAUNCH();
         kg_scale_v0<<<elem_blocks(S.n), kBlock, 0, s>>>(S.n, S.V, S.vin, S.state);
@@ -319,11 +319,11 @@ struct StokesGmres {
         kg_store_z<<<elem_blocks(n), kBlock, 0, s>>>(n, S.zout, S.Z, S.state);
         PK_LAUNCH();
         op(p, S.zout, S.w, nullptr, s);
-        const dim3 dg(kDotChunks, S.m + 1);
+        const dim3 dg(dot_chunks(n), S.m + 1);
         for (int pass = 0; pass < 2; ++pass) {
             kg_dots<<<dg, kBlock, 0, s>>>(n, S.V, S.w, S.state, S.part, S.cnt, S.hc, S.H, pass);
             PK_LAUNCH();
-            kg_axpy<<<kRedGrid, kBlock, 0, s>>>(n, S.V, S.w, S.state, S.hc, S.H, p->d_partials, p->d_counter, pass);
+            kg_axpy<<<red_grid(n), kBlock, 0, s>>>(n, S.V, S.w, S.state, S.hc, S.H, p->d_partials, p->d_counter, pass);
             PK_LAUNCH();
         }
         kg_scale_next<<<elem_blocks(n), kBlock, 0, s>>>(n, S.V, S.w, S.vin, S.state);
@@ -335,7 +335,7 @@ struct StokesGmres {
         kg_update_x<<<elem_blocks(n), kBlock, 0, s>>>(n, x, S.Z, S.yv, S.state);
         PK_LAUNCH();
         op(p, x, S.y, &S.state->cycle_end, s);
-        kg_residual_y<<<kRedGrid, kBlock, 0, s>>>(n, b, S.y, S.V, S.state, S.g, p->d_partials, p->d_counter, S.hist,
+        kg_residual_y<<<red_grid(S.n), kBlock, 0, s>>>(n, b, S.y, S.V, S.state, S.g, p->d_partials, p->d_counter, S.hist,
                                                   0);
         PK_LAUNCH();
         kg_scale_v0<<<elem_blocks(n), kBlock, 0, s>>>(n, S.V, S.vin, S.state);

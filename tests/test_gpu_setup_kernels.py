@@ -143,3 +143,51 @@ def test_spmv_slices(k, n):
     P.set_kappa(kap)
     assert torch.equal(P.spmv(x), y0)
     P.close()
+
+
+def _sweep_bound(P, prec):
+    """Rounding of a symmetric sweep and a dense tail: 2 C phases of sums of up to 400 terms,
+    then one of up to 5120, either way."""
+    u = 2.0 ** -24 if prec else 2.0 ** -53
+    return (2 * 2 * P.info.fine_colours * 400 + 2 * 5120) * u
+
+
+# the whole preconditioner as one dense product (up to 3400 unknowns; 4913 keep the sweeps)
+# against the row layout's sweeps
+@pytest.mark.parametrize("k,n,prec,level_smoother", [(2, 8, 0, 0), (2, 8, 1, 1), (4, 4, 0, 1), (3, 5, 1, 0), (2, 9, 0, 0),
+                                                     (1, 4, 0, 0)])
+def test_dense_preconditioner(k, n, prec, level_smoother):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, k, kappa_lognormal(t.shape[0], 1))
+    r = torch.randn(P.nh, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    out = []
+    for layout in (4, 0):
+        P.setup(smoother_layout=layout, precond_precision=prec, level_smoother=level_smoother)
+        out.append(P.apply_prec(r))
+    assert (out[1] - out[0]).norm() <= _sweep_bound(P, prec) * out[0].norm()
+    P.close()
+
+
+# the three velocity components in one sweep (above 3400 unknowns) against one at a time
+@pytest.mark.parametrize("k,n,prec", [(2, 9, 0), (3, 6, 1)])
+def test_stokes_components_share_sweeps(k, n, prec):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, k)
+    out = []
+    for layout in (4, 0):
+        P.setup(smoother_layout=layout, precond_precision=prec, level_smoother=1)
+        P.stokes_setup()
+        r = torch.randn(P.stokes_n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+        out.append(P.stokes_prec(r)[: 3 * P.nh])
+    assert (out[1] - out[0]).norm() <= _sweep_bound(P, prec) * out[0].norm()
+    P.close()
