@@ -124,6 +124,7 @@ struct DSell {
 struct DSlices {
     int t0 = 0, steps = 0, nb = 4;  // lanes of an ordinary row, most steps before its lanes
                                     // double, steps loaded per batch
+    bool late = false;              // late programmatic launch of the next phase (solve.cu)
     int64_t nslices = 0, entries = 0;
     int4 *meta = nullptr;
     int32_t *rows = nullptr, *col = nullptr;

@@ -366,12 +366,15 @@ __global__ void __launch_bounds__(kBlock) k_gs_phase(int64_t pb, int64_t pe, con
 // about 1.0 sectors an entry at the 300 G sectors/s that random gathers reach there.
 //
 // NV vectors at once (r and y of vector v at r + v n, y + v n): the slice is read once.
-template <int NB, int NV, typename PT, typename TR, bool BACK>
+//
+// LATE: the successor may launch only once this phase's wait is over, so no more than one
+// phase waits at a time (slice_late in solve.cu says when that is faster).
+template <int NB, int NV, bool LATE, typename PT, typename TR, bool BACK>
 __global__ void __launch_bounds__(kBlock) k_slice_phase(int64_t s0, int64_t s1, const int4 *__restrict__ meta,
                                                         const int32_t *__restrict__ rows,
                                                         const PT *__restrict__ dinv, const int32_t *__restrict__ col,
                                                         const PT *__restrict__ val, const TR *r, PT *y, int64_t n) {
-    pdl_trigger();
+    if (!LATE) pdl_trigger();
     const int64_t s = s0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (s >= s1) {  // a whole warp
@@ -394,6 +397,7 @@ __global__ void __launch_bounds__(kBlock) k_slice_phase(int64_t s0, int64_t s1, 
     const int32_t i = lead ? rows[m.z + q] : 0;
     const PT di = lead ? dinv[m.z + q] : PT(1);
     pdl_wait();
+    if (LATE) pdl_trigger();
     PT own[NV], acc[NV];
 #pragma unroll
     for (int u = 0; u < NV; ++u) {

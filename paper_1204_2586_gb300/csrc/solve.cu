@@ -94,11 +94,11 @@ void spmv(const DCSR &A, const X *x, Y *y, int tpr, cudaStream_t s) {
 // an earlier kernel wrote (k_gs_phase does).
 // win (optional): an L2 access-policy window for the launch
 template <typename... KArgs, typename... Args>
-void launch_pdl_w(void (*kern)(KArgs...), unsigned grid, cudaStream_t s, const cudaAccessPolicyWindow *win,
-                  Args... args) {
+void launch_pdl_b(void (*kern)(KArgs...), unsigned grid, unsigned block, cudaStream_t s,
+                  const cudaAccessPolicyWindow *win, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kBlock);
+    cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
@@ -113,6 +113,12 @@ void launch_pdl_w(void (*kern)(KArgs...), unsigned grid, cudaStream_t s, const c
     }
     PK_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
     PK_LAUNCH();
+}
+
+template <typename... KArgs, typename... Args>
+void launch_pdl_w(void (*kern)(KArgs...), unsigned grid, cudaStream_t s, const cudaAccessPolicyWindow *win,
+                  Args... args) {
+    launch_pdl_b(kern, grid, (unsigned)kBlock, s, win, args...);
 }
 
 template <typename... KArgs, typename... Args>
@@ -278,13 +284,21 @@ template <typename PT, typename TR, bool BACK, int NV = 1>
 void slice_sweep(const DSlices &S, bool ascending, const TR *r, PT *y, cudaStream_t s,
                  const cudaAccessPolicyWindow *win, int64_t n = 0) {
     const int nc = (int)S.off.size() - 1;
-    auto kern = S.nb == 2 ? k_slice_phase<2, NV, PT, TR, BACK>
-                : S.nb == 4 ? k_slice_phase<4, NV, PT, TR, BACK> : k_slice_phase<6, NV, PT, TR, BACK>;
+    auto kern = S.nb == 2 ? k_slice_phase<2, NV, false, PT, TR, BACK>
+                : S.nb == 4 ? k_slice_phase<4, NV, false, PT, TR, BACK> : k_slice_phase<6, NV, false, PT, TR, BACK>;
+    if (S.late)
+        kern = S.nb == 2 ? k_slice_phase<2, NV, true, PT, TR, BACK>
+               : S.nb == 4 ? k_slice_phase<4, NV, true, PT, TR, BACK> : k_slice_phase<6, NV, true, PT, TR, BACK>;
+    // four warps to a block where a phase is bound by its gathers or FP64 adds: a finished
+    // block makes room sooner (FP64 P4 48^3 1823 -> 1799 us, P4 32^3 766 -> 748, P3 32^3 281 ->
+    // 276; FP32 P4 48^3 1230 -> 1200); the short FP32 slices keep eight (P3 32^3 169 against 181)
+    const unsigned block = std::is_same<PT, double>::value || S.nb == 6 ? 128 : 256;
     for (int q = 0; q < nc; ++q) {
         const int c = ascending ? q : nc - 1 - q;
         const int64_t s0 = S.off[c], s1 = S.off[c + 1];
         if (s1 <= s0) continue;
-        launch_pdl_w(kern, rows_grid(s1 - s0, 32), s, win, s0, s1, (const int4 *)S.meta, (const int32_t *)S.rows,
+        const unsigned grid = (unsigned)(((s1 - s0) * 32 + block - 1) / block);
+        launch_pdl_b(kern, grid, block, s, win, s0, s1, (const int4 *)S.meta, (const int32_t *)S.rows,
                      pick<PT>(S.dinv, S.dinv32), (const int32_t *)S.col, pick<PT>(S.val, S.val32), r, y, n);
     }
 }
@@ -762,8 +776,7 @@ __global__ void __launch_bounds__(kBlock) k_pq_alpha(int64_t n, const double *__
 
 // Loop control of the captured while node: continue unless stopped; a safety bound on the
 // number of passes stops the loop even if no kernel set the flag. The kernel that decides
-// the stop sets the condition itself: a kernel of its own cost a launch of 1.7 us in every
-// pass. graph = 0: eager launches, the host reads the flag.
+// the stop sets the condition itself, instead of a launch of its own in every pass. graph = 0: eager launches, the host reads the flag.
 struct LoopNode {
     cudaGraphConditionalHandle h;
     int graph;
@@ -1073,15 +1086,17 @@ void free_setup(pkasp_problem *p) {
 // the mean of a row's part. Measured with graph replays of S_k (us, all sizes in both
 // precisions; the lines lie between the sizes where the order changes):
 //  - small phases have too few rows to fill the chip: two steps, the shortest chain. FP64
-//    below 14000 entries (P2 8^3: 41 against 50 with 6 steps; P2 14^3, 14000: 60 against 64;
-//    P3 12^3, 41000: 149 against 122), FP32, whose adds cost nothing, with eight lanes below
-//    110000 (P3 16^3, 100000: 80 against 86 with 4 lanes and steps; P3 24^3, 330000: 118
-//    against 109) or, for the longer rows of P4, 60000 (8^3, 27000: 125 against 135; 12^3,
-//    95000: 159 against 147). P1's rows (parts of 7 entries) always (64^3 FP64: 68 with 2
-//    lanes against 74 with 6 steps; FP32: 35 with 4 lanes against 48).
+//    below 20000 entries (P2 14^3, 17000: B 53 against 61 with 6 steps; P3 9^3, 15000: 82
+//    against 88; P4 8^3, 27000: 164 against 156), FP32, whose adds cost nothing, with eight
+//    lanes below 110000 (P3 16^3, 100000: 80 against 86 with 4 lanes and steps; P3 24^3,
+//    330000: 118 against 109) or, for the longer rows of P4, 60000 (8^3, 27000: 125 against
+//    135; 12^3, 95000: 159 against 147). P1's rows (parts of 7 entries) always (64^3 FP64: 68
+//    with 2 lanes against 74 with 6 steps; FP32: 35 with 4 lanes against 48).
 //  - then FP64 takes 2 lanes, since every shuffle add costs a warp-wide FP64 slot, and one
-//    batch of 6 steps (P3 32^3: 283 against 332 with 4 lanes and 4 steps); FP32 4 lanes and
-//    4 steps (P3 32^3: 170 against 183), or 2 and 6 for P4's rows (16^3: 163 against 176).
+//    batch of 6 steps (P3 32^3: 283 against 332 with 4 lanes and 4 steps); FP32 the same up to
+//    500000 entries for P3's rows and 10^6 for P4's (P3 24^3: B 108 against 114 with 4 lanes
+//    and steps; P4 16^3: 163 against 176), else 4 lanes and 4 steps (P3 32^3: 170 against 183;
+//    P2 48^3: B 148 against 154).
 //  - above 10^6 (FP64) and 2 10^6 (FP32) entries the L2 rate counts: fewer lanes that double
 //    late, so more of a step's entries belong to one row. FP64 P4 48^3 1827 with 4 lanes,
 //    16 steps and batches of 4 (fewer registers, so more warps) against 1948 with
@@ -1095,13 +1110,24 @@ SliceShape slice_shape(bool fp32, double entries, double part) {
     if (fp32) {
         if (entries < (part < 30 ? 110e3 : 60e3)) return {8, 2, 2};
         if (entries >= 2e6) return {4, 16, 6};
-        return part < 30 || entries >= 1e6 ? SliceShape{4, 4, 4} : SliceShape{2, 6, 6};
+        if (part >= 18 && entries < (part < 30 ? 5e5 : 1e6)) return {2, 6, 6};
+        return {4, 4, 4};
     }
-    if (entries < 14e3) return {2, 2, 2};
+    if (entries < 20e3) return {2, 2, 2};
     if (entries < 1e6) return {2, 6, 6};
     if (part < 18) return {2, 16, 6};
     return entries < 2.2e6 ? SliceShape{4, 16, 6} : SliceShape{4, 16, 4};
 }
+
+// Whether a phase lets its successor launch only after its own wait (k_slice_phase). Early,
+// every following phase that fits the chip is resident and loads its entries while the
+// current one gathers; for FP64 phases of middling size those loads are in the way. S_k and
+// B as graphs, us, early -> late: P4 16^3 (220,000 entries a phase) 329 -> 246, B 315 -> 256;
+// P2 33^3 (226,000) 119 -> 89, B 133 -> 112; P3 16^3 (98,000) 159 -> 107, B 118 -> 110; P2 48^3
+// (720,000) B 252 -> 236. Smaller ones need the head start (P2 21^3, 56,000: B 74 -> 77), larger
+// ones do not mind (P3 32^3, 780,000: B 313 -> 316; P4 32^3: 751 -> 777), FP32 loses (P3 16^3:
+// 79 -> 85).
+bool slice_late(bool fp32, double entries) { return !fp32 && entries >= 80e3 && entries < 750e3; }
 
 // slices of part `which` (build_slices) of A's split, shaped for its mean phase and row
 void shaped_slices(pkasp_problem *p, const DCSR &A, const DSplit &sp, int which, DSlices &S, cudaStream_t s) {
@@ -1111,6 +1137,7 @@ void shaped_slices(pkasp_problem *p, const DCSR &A, const DSplit &sp, int which,
     const SliceShape h = slice_shape(fp32, n * part / nc, part);
     build_slices(p->setup_pool, A, sp, which, h.t0, h.steps, fp32, S, s);
     S.nb = h.nb;
+    S.late = slice_late(fp32, n * part / nc);
 }
 
 // builds the fine smoother's slices; returns the layout code 500 + lanes of an ordinary row
