@@ -25,7 +25,7 @@ struct StokesWork {
     DCSR B, BT, M;
     double *mdiag = nullptr;
     // preconditioner work
-    double *t = nullptr, *rr = nullptr, *zz = nullptr, *pp = nullptr, *qq = nullptr, *xp = nullptr;
+    double *t = nullptr, *rr = nullptr, *zz = nullptr, *pp = nullptr, *pn = nullptr, *qq = nullptr, *xp = nullptr;
     double *scal = nullptr;  // rho, alpha, beta of the inner CG
     double *zs3 = nullptr, *w3 = nullptr;  // the three components' smoothed and coarse parts
     // FGMRES
@@ -183,7 +183,11 @@ __global__ void __launch_bounds__(kBlock) ks_spmv_rows(int64_t n, const int64_t 
 }
 
 // ---- inner CG on M_p with the diagonal as preconditioner (device scalars) ----------
-// start: r = r_p, z = r / d, p = z, x = 0, rho = (r, z)
+// A step is two launches: ks_mp_step forms p = z + beta p on the fly where a row gathers it
+// (into the other of two buffers), q = M p and alpha; ks_mp_update the rest. With the p
+// update, the product and the dot product as launches of their own, the 41 launches of ten
+// steps were a third of an FGMRES step at P2 12^3.
+// start: r = r_p, z = r / d, p = 0, x = 0, beta = 0, rho = (r, z)
 __global__ void __launch_bounds__(kBlock) ks_mp_start(int64_t n, const double *__restrict__ rp,
                                                       const double *__restrict__ d, double *rr, double *zz, double *pp,
                                                       double *xp, double *scal, double *partials, unsigned *counter) {
@@ -192,20 +196,48 @@ __global__ void __launch_bounds__(kBlock) ks_mp_start(int64_t n, const double *_
         const double r = rp[i], z = r / d[i];
         rr[i] = r;
         zz[i] = z;
-        pp[i] = z;
+        pp[i] = 0.0;
         xp[i] = 0.0;
         part += r * z;
     }
     double v[1] = {part}, tot[1];
-    if (grid_reduce<1>(v, partials, counter, tot) && threadIdx.x == 0) scal[0] = tot[0];
+    if (grid_reduce<1>(v, partials, counter, tot) && threadIdx.x == 0) {
+        scal[0] = tot[0];
+        scal[2] = 0.0;
+    }
 }
 
-// alpha = rho / (p, q) (0 once rho is 0)
-__global__ void __launch_bounds__(kBlock) ks_mp_alpha(int64_t n, const double *pp, const double *qq, double *scal,
-                                                      double *partials, unsigned *counter) {
+// pn = z + beta p, q = M pn (8 lanes per row), alpha = rho / (pn, q) (0 once rho is 0)
+__global__ void __launch_bounds__(kBlock) ks_mp_step(int64_t n, const int64_t *__restrict__ ptr,
+                                                     const int32_t *__restrict__ col, const double *__restrict__ val,
+                                                     const double *__restrict__ zz, const double *__restrict__ pp,
+                                                     double *__restrict__ pn, double *__restrict__ qq, double *scal,
+                                                     double *partials, unsigned *counter) {
+    constexpr int TPR = 8;
+    const double beta = scal[2];
+    const int sub = threadIdx.x & (TPR - 1), sg = (threadIdx.x & 31) / TPR;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    constexpr int rpw = 32 / TPR;
     double part = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        part += pp[i] * qq[i];
+    for (int64_t base = warp * rpw; base < n; base += nwarps * rpw) {
+        const int64_t row = base + sg;
+        const bool ok = row < n;
+        double s = 0.0;
+        if (ok)
+#pragma unroll 4
+            for (int64_t e = ptr[row] + sub; e < ptr[row + 1]; e += TPR) {
+                const int32_t j = col[e];
+                s += val[e] * (zz[j] + beta * pp[j]);
+            }
+        s = subwarp_sum<TPR>(s);
+        if (ok && sub == 0) {
+            const double p = zz[row] + beta * pp[row];
+            pn[row] = p;
+            qq[row] = s;
+            part += p * s;
+        }
+    }
     double v[1] = {part}, tot[1];
     if (grid_reduce<1>(v, partials, counter, tot) && threadIdx.x == 0)
         scal[1] = scal[0] != 0.0 ? scal[0] / tot[0] : 0.0;
@@ -230,12 +262,6 @@ __global__ void __launch_bounds__(kBlock) ks_mp_update(int64_t n, double *xp, do
         scal[2] = scal[0] != 0.0 ? tot[0] / scal[0] : 0.0;
         scal[0] = tot[0];
     }
-}
-
-__global__ void ks_mp_p(int64_t n, const double *zz, double *pp, const double *scal) {
-    const double beta = scal[2];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        pp[i] = zz[i] + beta * pp[i];
 }
 
 // z_p = -x; t = r_u - B^T z_p (one thread per velocity row)
@@ -281,16 +307,15 @@ void prec(pkasp_problem *p, const double *r, double *z, cudaStream_t s) {
     ks_mp_start<<<red_grid(np), kBlock, 0, s>>>(np, r + nu, S.mdiag, S.rr, S.zz, S.pp, S.xp, S.scal, p->d_partials,
                                             p->d_counter);
     PK_LAUNCH();
+    double *p0 = S.pp, *p1 = S.pn;
     for (int it = 0; it < S.mp_iters; ++it) {
-        ks_spmv_rows<<<red_grid(np * 8), kBlock, 0, s>>>(np, S.M.ptr, S.M.col, S.M.val, S.pp, S.qq, nullptr);
+        ks_mp_step<<<red_grid(np * 8), kBlock, 0, s>>>(np, S.M.ptr, S.M.col, S.M.val, S.zz, p0, p1, S.qq, S.scal,
+                                                       p->d_partials, p->d_counter);
         PK_LAUNCH();
-        ks_mp_alpha<<<red_grid(np), kBlock, 0, s>>>(np, S.pp, S.qq, S.scal, p->d_partials, p->d_counter);
+        ks_mp_update<<<red_grid(np), kBlock, 0, s>>>(np, S.xp, S.rr, S.zz, p1, S.qq, S.mdiag, S.scal, p->d_partials,
+                                                     p->d_counter);
         PK_LAUNCH();
-        ks_mp_update<<<red_grid(np), kBlock, 0, s>>>(np, S.xp, S.rr, S.zz, S.pp, S.qq, S.mdiag, S.scal, p->d_partials,
-                                                 p->d_counter);
-        PK_LAUNCH();
-        ks_mp_p<<<grid_for(np), kBlock, 0, s>>>(np, S.zz, S.pp, S.scal);
-        PK_LAUNCH();
+        std::swap(p0, p1);
     }
     ks_neg<<<grid_for(np), kBlock, 0, s>>>(np, S.xp, z + nu);
     PK_LAUNCH();
@@ -486,6 +511,7 @@ void stokes_setup(pkasp_problem *p, int mp_iters, cudaStream_t s) {
     S.rr = S.pool.get<double>(npp);
     S.zz = S.pool.get<double>(npp);
     S.pp = S.pool.get<double>(npp);
+    S.pn = S.pool.get<double>(npp);
     S.qq = S.pool.get<double>(npp);
     S.xp = S.pool.get<double>(npp);
     S.scal = S.pool.get<double>(4);
