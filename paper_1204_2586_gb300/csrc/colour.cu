@@ -113,6 +113,73 @@ __global__ void k_jp_round(const int64_t *__restrict__ ptr, const int32_t *__res
     if (most > 0 && sub == 0) atomicMax(maxcol, most);
 }
 
+// The same rounds in one block, with colours, counts and lists in shared memory, one warp per
+// row. A coarse level is nearly dense, so its rounds are many (592 rows with 124 entries each:
+// hundreds) and hold a row or two: a launch each took 3.2 ms of a 17 ms setup for those rows
+// at P3 24^3. Up to kJpSmall rows; with more a block is the smaller part of the chip.
+constexpr int kJpSmall = 4096;
+
+__global__ void __launch_bounds__(1024) k_jp_small(int n, const int64_t *__restrict__ ptr,
+                                                   const int32_t *__restrict__ col, const int32_t *__restrict__ cnt0,
+                                                   const int32_t *__restrict__ list0, const unsigned *__restrict__ nlist,
+                                                   int32_t *__restrict__ colour, int *__restrict__ maxcol) {
+    extern __shared__ int32_t jp_smem[];
+    int32_t *clr = jp_smem, *cnt = clr + n, *in = cnt + n, *out = in + n;
+    __shared__ int num[2];
+    __shared__ int most;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        num[0] = (int)*nlist;
+        num[1] = 0;
+        most = 0;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < n; q += blockDim.x) {
+        clr[q] = -1;
+        cnt[q] = cnt0[q];
+        if (q < num[0]) in[q] = list0[q];
+    }
+    __syncthreads();
+    // every row enters a list once, so the rounds end
+    for (int cur = 0; num[cur] > 0; cur ^= 1) {
+        const int nf = num[cur];
+        for (int q = warp; q < nf; q += 32) {
+            const int32_t i = in[q];
+            const int64_t lo = ptr[i], hi = ptr[i + 1];
+            int base = 0, c = -1;
+            while (c < 0) {
+                unsigned long long used = 0ull;
+                for (int64_t e = lo + lane; e < hi; e += 32) {
+                    const int32_t j = col[e];
+                    const int cj = j == i ? -1 : clr[j] - base;
+                    if (cj >= 0 && cj < 64) used |= 1ull << cj;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) used |= __shfl_xor_sync(0xffffffffu, used, o);
+                if (~used != 0ull) c = base + __ffsll((long long)~used) - 1;
+                else base += 64;
+            }
+            for (int64_t e = lo + lane; e < hi; e += 32) {
+                const int32_t j = col[e];
+                if (j == i || clr[j] >= 0) continue;
+                if (atomicSub(&cnt[j], 1) == 1) out[atomicAdd(&num[cur ^ 1], 1)] = j;
+            }
+            if (lane == 0) {
+                clr[i] = c;
+                atomicMax(&most, c + 1);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) num[cur] = 0;
+        int32_t *t = in;
+        in = out;
+        out = t;
+        __syncthreads();
+    }
+    for (int q = threadIdx.x; q < n; q += blockDim.x) colour[q] = clr[q];
+    if (threadIdx.x == 0) *maxcol = most;
+}
+
 int jp_colour(int64_t n, const int64_t *ptr, const int32_t *col, uint64_t stream, int32_t *colour, DevPool &tmp,
               cudaStream_t s) {
     int32_t *deg = tmp.get<int32_t>(n), *cnt = tmp.get<int32_t>(n);
@@ -125,6 +192,17 @@ int jp_colour(int64_t n, const int64_t *ptr, const int32_t *col, uint64_t stream
     PK_LAUNCH();
     k_jp_count<<<blocks_for(n * kJpLanes, 256), 256, 0, s>>>(n, ptr, col, deg, stream, cnt, list[0], ctr);
     PK_LAUNCH();
+    if (n <= kJpSmall) {
+        const size_t smem = sizeof(int32_t) * 4 * (size_t)n;
+        PK_CUDA(cudaFuncSetAttribute(k_jp_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(sizeof(int32_t) * 4 * kJpSmall)));
+        k_jp_small<<<1, 1024, smem, s>>>((int)n, ptr, col, cnt, list[0], ctr, colour, maxc);
+        PK_LAUNCH();
+        int h = 0;
+        PK_CUDA(cudaMemcpyAsync(&h, maxc, sizeof(int), cudaMemcpyDeviceToHost, s));
+        PK_CUDA(cudaStreamSynchronize(s));
+        return h;
+    }
     // a round's list is rarely longer than a few percent of the rows; rounds run in
     // batches of 32 between two looks at the list length (an empty round costs a launch)
     const unsigned grid = (unsigned)std::min<int64_t>(152 * 4, blocks_for(n * kJpLanes, 256));

@@ -191,3 +191,12 @@ def test_stokes_components_share_sweeps(k, n, prec):
         out.append(P.stokes_prec(r)[: 3 * P.nh])
     assert (out[1] - out[0]).norm() <= _sweep_bound(P, prec) * out[0].norm()
     P.close()
+
+
+@pytest.mark.parametrize("n", [2, 16, 17, 18])
+def test_colouring_in_one_block_and_in_rounds(oracle_mod, n):
+    """P1 problems of 1, 3375, 4096 and 4913 rows: up to 4096 the colouring runs in one block."""
+    _, G, O = _pair(oracle_mod, 1, n)
+    c, nc = G.colours(-1)
+    assert np.array_equal(c, O.fine_colour()) and nc == c.max() + 1
+    assert np.array_equal(G.colours(0)[0], O.level(0)["colour"])
