@@ -402,8 +402,7 @@ def main():
                              "theta_study", "cop_study", "stokes_study"])
     ap.add_argument("--smoother-layout", type=int, default=0,
                     help="pin the fine smoother layout (pkasp_options.smoother_layout) instead of "
-                         "autotuning it; for profiler runs, under which the autotuner's timings "
-                         "are distorted")
+                         "the slices that setup shapes by the sizes")
     ap.add_argument("--smoother-layout-fp32", type=int, default=0,
                     help="the same for the FP32-preconditioner solves")
     ap.add_argument("--mesh-n", type=int, default=0,

@@ -263,26 +263,6 @@ __global__ void __launch_bounds__(kBlock) k_residual(int64_t n, const int64_t *_
 // backward from there: y_i = y_i - (sum_U a_ij y_j) / a_ii
 // backward full sweep: x_i = (b_i - sum_L a_ij x_j - sum_U a_ij x_j) / a_ii
 // ---------------------------------------------------------------------------------
-template <int TPR, typename PT, typename TR>
-__global__ void __launch_bounds__(kBlock) k_gs_fwd0(int64_t pb, int64_t pe, const int32_t *__restrict__ perm,
-                                                    const int64_t *__restrict__ lptr, const int32_t *__restrict__ lcol,
-                                                    const PT *__restrict__ lval, const PT *__restrict__ diag,
-                                                    const TR *__restrict__ r, PT *y) {
-    // every per-row load that does not depend on the row sum is issued first, so the
-    // phase costs one round trip for them plus the entry loads and gathers
-    const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t p = pb + gt / TPR;
-    const int sub = threadIdx.x & (TPR - 1);
-    const bool ok = p < pe;
-    const bool lead = ok && sub == 0;
-    const int32_t i = lead ? perm[p] : 0;
-    const PT d = lead ? diag[p] : PT(1);
-    int64_t lo = ok ? lptr[p] : 0, hi = ok ? lptr[p + 1] : 0;
-    const PT ri = lead ? (PT)r[i] : PT(0);
-    PT s = row_dot<TPR, PT>(lo, hi, sub, lcol, lval, (const PT *)y);
-    if (lead) y[i] = (ri - s) / d;
-}
-
 // Programmatic dependent launch (sm_90+): a kernel launched with programmatic stream
 // serialization may start while its predecessor is still running. It lets its own
 // successor launch at once, loads the data no kernel of the solve writes (the matrix),
@@ -641,24 +621,6 @@ __global__ void __launch_bounds__(kBlock) k_gs_phase2(int64_t pb, int64_t pe, co
         if (lead[q]) y[i[q]] = BACK ? own[q] - acc[q] * di[q] : (own[q] - acc[q]) * di[q];
 }
 
-template <int TPR, typename PT>
-__global__ void __launch_bounds__(kBlock) k_gs_bwd0(int64_t pb, int64_t pe, const int32_t *__restrict__ perm,
-                                                    const int64_t *__restrict__ uptr, const int32_t *__restrict__ ucol,
-                                                    const PT *__restrict__ uval, const PT *__restrict__ diag,
-                                                    PT *y) {
-    const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t p = pb + gt / TPR;
-    const int sub = threadIdx.x & (TPR - 1);
-    const bool ok = p < pe;
-    const bool lead = ok && sub == 0;
-    const int32_t i = lead ? perm[p] : 0;
-    const PT d = lead ? diag[p] : PT(1);
-    int64_t lo = ok ? uptr[p] : 0, hi = ok ? uptr[p + 1] : 0;
-    const PT yi = lead ? y[i] : PT(0);
-    PT s = row_dot<TPR, PT>(lo, hi, sub, ucol, uval, (const PT *)y);
-    if (lead) y[i] = yi - s / d;
-}
-
 template <int TPR, int NB, typename PT>
 __global__ void __launch_bounds__(kBlock) k_gs_bwd_full(int64_t pb, int64_t pe, const int32_t *__restrict__ perm,
                                                         const int64_t *__restrict__ lptr, const int32_t *__restrict__ lcol,
@@ -681,25 +643,11 @@ __global__ void __launch_bounds__(kBlock) k_gs_bwd_full(int64_t pb, int64_t pe, 
     if (lead) x[i] = (bi - sl - su) / d;
 }
 
-// l1-Jacobi: x = r / d (from zero) and x += (b - A x) / d
+// l1-Jacobi from zero: x = r / d
 template <typename PT, typename TR>
 __global__ void k_jacobi0(int64_t n, const PT *__restrict__ d, const TR *__restrict__ r, PT *__restrict__ x) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) x[i] = (PT)r[i] / d[i];
-}
-
-template <int TPR, typename PT>
-__global__ void __launch_bounds__(kBlock) k_jacobi_step(int64_t n, const int64_t *__restrict__ ptr,
-                                                        const int32_t *__restrict__ col, const PT *__restrict__ val,
-                                                        const PT *__restrict__ d, const PT *__restrict__ b,
-                                                        const PT *__restrict__ xin, PT *__restrict__ xout) {
-    const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = gt / TPR;
-    const int sub = threadIdx.x & (TPR - 1);
-    const bool ok = row < n;
-    int64_t lo = ok ? ptr[row] : 0, hi = ok ? ptr[row + 1] : 0;
-    PT s = row_dot<TPR, PT>(lo, hi, sub, col, val, xin);
-    if (ok && sub == 0) xout[row] = xin[row] + (b[row] - s) / d[row];
 }
 
 // z_i = zs_i + sum_j Pi_ij w_j (I_P has at most 4 entries per row: one thread per row)

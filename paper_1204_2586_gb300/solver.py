@@ -79,7 +79,7 @@ class Problem:
 
     @property
     def info(self):
-        """pkasp_info of the problem as it is now (sizes, hierarchy, autotuned layouts)."""
+        """pkasp_info of the problem as it is now (sizes, hierarchy, layouts)."""
         return self._info()
 
     def _info(self):
