@@ -542,7 +542,7 @@ def main():
     src = "measured (MEASURED_PEAKS.json hbm_gbs)" if hbm else "fallback"
     s_ach = smoother_bytes / (smoother_ms / 1e3) / 1e9
     s_tf = smoother_flops / (smoother_ms / 1e3) / 1e12
-    roof = {"bound": "hbm", "kernel": "k_gs_phase (colour phases of the fine SGS S_k, FP64)",
+    roof = {"bound": "hbm", "kernel": "k_slice_phase (colour phases of the fine SGS S_k, FP64)",
             "achieved": s_ach, "peak": peak, "unit": "GB/s", "frac": s_ach / peak,
             "traffic": SMOOTHER_TRAFFIC.get((WORKLOAD["name"], WORKLOAD["n"], smoother_layout_name(
                 info64.smoother_layout))),
