@@ -193,8 +193,11 @@ __global__ void __launch_bounds__(kBlock) kb_init_residual(int64_t n, const int6
     }
 }
 
-// Q = A P and alpha_c = rho_c / (p_c, q_c) for the columns still running
-template <int NC>
+// Q = A P and alpha_c = rho_c / (p_c, q_c) for the columns still running; E entry groups
+// share a row (W * E = 32 lanes, or E = 1): with fewer rows than two passes of the grid the
+// longest row's chain is the kernel's time (P3 9^3, 5 columns: 76 -> 59 us; P4 6^3, 3 columns:
+// 115 -> 53)
+template <int NC, int E>
 __global__ void __launch_bounds__(kBlock) kb_spmv_pq(int64_t n, const int64_t *__restrict__ ptr,
                                                      const int32_t *__restrict__ col, const double *__restrict__ val,
                                                      const double *P, double *Q, PcgState *st, double *partials,
@@ -203,14 +206,15 @@ __global__ void __launch_bounds__(kBlock) kb_spmv_pq(int64_t n, const int64_t *_
     __shared__ double tot[NC];
     if (st->all_done) return;
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x % W;
-    const int64_t ntask = ((int64_t)gridDim.x * blockDim.x) / W;
+    const int lane = threadIdx.x % W, g = threadIdx.x % (W * E) / W;
+    const int64_t ntask = ((int64_t)gridDim.x * blockDim.x) / (W * E);
     double v[1][CPL];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) v[0][k] = 0.0;
-    for (int64_t row = gt / W; row < n; row += ntask) {
+    for (int64_t row = gt / (W * E); row < n; row += ntask) {
         double acc[CPL];
-        bdot<NC, double>(ptr[row], ptr[row + 1], col, val, P, NC, lane, acc);
+        bdote<W, E, CPL, double>(ptr[row], ptr[row + 1], col, val, P, NC, lane, g, acc);
+        if (g != 0) continue;
 #pragma unroll
         for (int k = 0; k < CPL; ++k) {
             const int64_t o = row * NC + lane + k * W;
@@ -924,6 +928,13 @@ struct Batched {
         PK_LAUNCH();
     }
 
+    static void spmm_pq(pkasp_problem *p, cudaStream_t s) {
+        auto kern = p->nh * W <= 2 * (int64_t)kRedGrid * kBlock ? kb_spmv_pq<NC, 32 / W> : kb_spmv_pq<NC, 1>;
+        kern<<<kRedGrid, kBlock, 0, s>>>(p->nh, p->Ah.ptr, p->Ah.col, p->Ah.val, p->bw_p, p->bw_q, p->d_state,
+                                         p->d_partials, p->d_counter);
+        PK_LAUNCH();
+    }
+
     // the autotuner of the fine smoother's layout (column group width, lanes per row):
     // times one symmetric sweep per candidate. Results are the same bits for every
     // layout: each column's sums run over the same entries in the same order. Returns
@@ -981,9 +992,7 @@ struct Batched {
         PK_LAUNCH();
         auto once = [&]() {
             if (which == 4) {
-                kb_spmv_pq<NC><<<kRedGrid, kBlock, 0, s>>>(p->nh, p->Ah.ptr, p->Ah.col, p->Ah.val, p->bw_p,
-                                                           p->bw_q, p->d_state, p->d_partials, p->d_counter);
-                PK_LAUNCH();
+                spmm_pq(p, s);
             } else if (which == 5) {
                 if (f32) gs_sym<float>(p->fine, p->bw_r32, p->bw_zs32, true, p->bchunk - 1, s);
                 else gs_sym<double>(p->fine, p->bw_b, p->bw_zs, true, p->bchunk - 1, s);
@@ -1028,9 +1037,7 @@ struct Batched {
     }
 
     static void iteration(pkasp_problem *p, double *X, cudaStream_t s) {
-        kb_spmv_pq<NC><<<kRedGrid, kBlock, 0, s>>>(p->nh, p->Ah.ptr, p->Ah.col, p->Ah.val, p->bw_p, p->bw_q,
-                                                   p->d_state, p->d_partials, p->d_counter);
-        PK_LAUNCH();
+        spmm_pq(p, s);
         kb_update_xr<NC><<<kRedGrid, FlatBT<NC>, 0, s>>>(p->nh * NC, X, p->bw_r, r32_out(p), p->bw_p, p->bw_q,
                                                          p->d_state, p->d_partials, p->d_counter, p->d_hist);
         PK_LAUNCH();
