@@ -24,8 +24,7 @@ unsigned blocks_for(int64_t n, int per) {
 // list, takes its colour, and takes one off the count of each uncoloured neighbour, which
 // joins the next round's list when its count reaches zero. (Rescanning every uncoloured
 // row each round, with each neighbour's degree counted from its row, took 116 ms of a
-// 312 ms setup at P3 24^3; now the whole splits, colours included, take 3.8 ms for A_h
-// and 9.3 ms for the four levels, whose rounds are short and many.)
+// 312 ms setup at P3 24^3; now the whole split of A_h, colours included, takes 2.6 ms.)
 //
 // kJpLanes lanes share a row: rows have 15 (P1) to 75 (P4) entries on average, so eight
 // lanes read them in a few coalesced steps and leave enough rows in flight.

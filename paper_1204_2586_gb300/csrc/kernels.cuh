@@ -341,8 +341,8 @@ __global__ void __launch_bounds__(kBlock) k_gs_phase(int64_t pb, int64_t pe, con
 // 16 unaligned bytes of columns and 32 of values per step: 0.59 lines an entry besides the
 // 0.39 of the gathers (host count at P4 7^3). A slice's step is one line of columns and two
 // of values: 0.1 lines an entry. FP64 S_k, us before -> after (graph replays): P4 48^3
-// 2325 -> 1827, P4 24^3 597 -> 454, P3 32^3 359 -> 283, P2 33^3 129 -> 124, P2 8^3 46 -> 42;
-// FP32: P4 48^3 1379 -> 1240, P3 32^3 191 -> 170, P3 9^3 68 -> 66. At P4 48^3 FP64 it reads
+// 2325 -> 1804, P4 24^3 597 -> 446, P3 32^3 359 -> 276, P2 33^3 129 -> 89, P2 8^3 46 -> 38;
+// FP32: P4 48^3 1379 -> 1204, P3 32^3 191 -> 170, P3 9^3 68 -> 65. At P4 48^3 FP64 it reads
 // about 1.0 sectors an entry at the 300 G sectors/s that random gathers reach there.
 //
 // NV vectors at once (r and y of vector v at r + v n, y + v n): the slice is read once.

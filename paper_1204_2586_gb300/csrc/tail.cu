@@ -109,7 +109,9 @@ __global__ void __launch_bounds__(kCols) k_tail_coarse(int64_t n, int64_t nc, co
 }
 
 // Modelled time (us) of one cycle from level l down, as launches. Gauss-Seidel: a launch
-// per colour and sweep, 3.4 us each (P2 21^3 FP64, 202 phases of three levels: 709 us);
+// per colour and sweep, 3.4 us each in the row layout (P2 21^3 FP64, 202 phases of three
+// levels: 709 us) and 1.6 to 2.4 in slices, which picks the same levels on the hierarchies of
+// P1 problems from 17^3 to 64^3;
 // l1-Jacobi: five launches of 2 us each besides the next level (P2 8^3: 18 us over two
 // levels).
 double launches_us(const Level &L, bool jacobi) { return jacobi ? 11.0 : 10.0 + 2 * 3.4 * L.sp.ncol; }
