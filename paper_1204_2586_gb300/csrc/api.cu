@@ -239,6 +239,7 @@ int pkasp_set_kappa(pkasp_problem *p, const double *kappa, pkasp_stream_t stream
         cudaStream_t s = (cudaStream_t)stream;
         PK_CUDA(cudaMemcpyAsync(p->d_kappa, kappa, sizeof(double) * p->nt, cudaMemcpyDefault, s));
         pk::free_setup(p);  // the preconditioner belongs to the old kappa
+        pk::setup_pool_trim(p, pk::kKeepKappa);
         pk::assemble_values(p, false, s);
         return PKASP_OK;
     });

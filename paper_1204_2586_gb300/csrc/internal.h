@@ -318,6 +318,11 @@ void assemble_device(pkasp_problem *p, cudaStream_t s);
 void assemble_values(pkasp_problem *p, bool first, cudaStream_t s);
 void setup_device(pkasp_problem *p, cudaStream_t s);
 void free_setup(pkasp_problem *p);
+// What pkasp_set_kappa leaves in the pool for the setup that follows as a rule. Mapping memory
+// again costs 2.3 ms a GB: P3 24^3 (0.7 GB) set_kappa and setup take 19.3 ms with it and 20.8
+// with all of it given back; of the 24 GB of P4 48^3 no more than this stays.
+constexpr size_t kKeepKappa = size_t(1) << 30;
+void setup_pool_trim(pkasp_problem *p, size_t keep);
 int solve_device(pkasp_problem *p, const double *b_dev, double *x_dev, int ncols, int64_t ld,
                  pkasp_stats *st, cudaStream_t s);
 void apply_prec(pkasp_problem *p, const double *r, double *z, cudaStream_t s);

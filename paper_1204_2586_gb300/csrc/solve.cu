@@ -1181,7 +1181,9 @@ void choose_layouts(pkasp_problem *p, cudaStream_t s) {
 }
 
 // The problem's memory pool, made at its first setup (null where the device has none: blocks
-// then come from cudaMalloc). It keeps what a setup frees until the setup's end.
+// then come from cudaMalloc). It keeps what a setup frees until the setup's end, and 64 MB
+// from then on (pkasp_set_kappa: kKeepKappa).
+constexpr size_t kKeepSetup = size_t(64) << 20;
 void setup_pool_open(pkasp_problem *p) {
     if (p->mem) return;
     cudaMemPoolProps props = {};
@@ -1197,11 +1199,14 @@ void setup_pool_open(pkasp_problem *p) {
     PK_CUDA(cudaMemPoolSetAttribute(p->mem, cudaMemPoolAttrReleaseThreshold, &keep));
 }
 
-// gives back what the pool holds beyond the blocks in use and 64 MB
-void setup_pool_trim(pkasp_problem *p) {
+// Gives back what the pool holds beyond the blocks in use and `keep` bytes. The frees are
+// stream-ordered: what cap_stream has not freed yet counts as in use, so it is waited for.
+void setup_pool_trim(pkasp_problem *p, size_t keep) {
+    if (!p->mem) return;
+    cudaStreamSynchronize(p->cap_stream);
     uint64_t used = 0;
-    if (p->mem && cudaMemPoolGetAttribute(p->mem, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
-        cudaMemPoolTrimTo(p->mem, (size_t)used + (64u << 20));
+    if (cudaMemPoolGetAttribute(p->mem, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+        cudaMemPoolTrimTo(p->mem, (size_t)used + keep);
     cudaGetLastError();
 }
 
@@ -1218,10 +1223,10 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
         setup_build(p, s);
     } catch (...) {
         cudaStreamSynchronize(s);
-        setup_pool_trim(p);
+        setup_pool_trim(p, kKeepSetup);
         throw;
     }
-    setup_pool_trim(p);
+    setup_pool_trim(p, kKeepSetup);
 }
 
 void setup_build(pkasp_problem *p, cudaStream_t s) {

@@ -45,8 +45,18 @@ void *DevPool::alloc(size_t n) {
     void *p = nullptr;
     if (n == 0) n = 16;
     n = (n + 255) & ~(size_t)255;
-    cudaError_t e = mp ? cudaMallocFromPoolAsync(&p, n, mp, PoolScope::pool() == mp ? PoolScope::stream() : ms)
-                       : cudaMalloc(&p, n);
+    auto get = [&] {
+        return mp ? cudaMallocFromPoolAsync(&p, n, mp, PoolScope::pool() == mp ? PoolScope::stream() : ms)
+                  : cudaMalloc(&p, n);
+    };
+    cudaError_t e = get();
+    if (e != cudaSuccess && PoolScope::pool()) {
+        // what the scratch of this setup has freed may be what is missing
+        cudaGetLastError();
+        cudaStreamSynchronize(PoolScope::stream());
+        cudaMemPoolTrimTo(PoolScope::pool(), 0);
+        e = get();
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         fail(PKASP_ENOMEM, "device allocation of " + std::to_string(n) + " bytes failed");

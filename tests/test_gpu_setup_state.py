@@ -1,0 +1,57 @@
+"""What a problem holds before, between and after its setups: memory that is no longer in use
+goes back."""
+import pytest
+
+from paper_1204_2586_gb300 import _lib as L
+from paper_1204_2586_gb300.inputs import kappa_lognormal, kuhn_mesh
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch
+
+
+def _problem(k, n):
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    return Problem(xyz, t, k, kappa_lognormal(t.shape[0], 1))
+
+
+def _free(torch):
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.cuda.mem_get_info()[0]
+
+
+MB = 1 << 20
+
+
+def test_set_kappa_gives_memory_back(torch_cuda):
+    """pkasp_set_kappa discards the setup: of its 36 bytes an entry of A_h (FP32 preconditioner:
+    split 16, SpMV slices 12, smoother slices 8) no more than 1 GB stays for the next one."""
+    torch = torch_cuda
+    P = _problem(4, 32)
+    P.setup(precond_precision=1, level_smoother=1)
+    held = _free(torch)
+    P.set_kappa(kappa_lognormal(P.nt, 2))
+    assert _free(torch) - held >= 36 * P.info.nnz_h - 1024 * MB
+    P.close()
+
+
+def test_smaller_setup_gives_memory_back(torch_cuda):
+    """A setup with fewer copies of A_h than the one before it holds less: 28 bytes an entry of
+    slices are gone (SpMV 12, smoother 8, whole rows 8), 64 MB of it may stay in the pool, as
+    much again in the parts of its blocks that the smaller setup uses."""
+    torch = torch_cuda
+    P = _problem(4, 20)
+    P.setup(mode=1, precond_precision=1, level_smoother=1)
+    held = _free(torch)
+    P.setup(smoother=1, precond_precision=1, spmv_threads=4, level_smoother=1)
+    assert _free(torch) - held >= 28 * P.info.nnz_h - 128 * MB
+    P.close()
