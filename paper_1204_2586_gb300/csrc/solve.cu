@@ -1065,7 +1065,8 @@ void free_setup(pkasp_problem *p) {
     p->flu = DSlices{};
     p->flf = DSlices{};
     p->fsv = DSlices{};
-    p->spmv_tpr = 4;  // A_h itself stays: pkasp_spmv reads its CSR form until the next setup
+    // A_h itself stays: pkasp_spmv reads its CSR form until the next setup
+    p->spmv_tpr = p->fine_tpr = 4;
     p->d_l1h = nullptr;
     p->d_l1h32 = nullptr;
     p->d_cinv = nullptr;
@@ -1223,9 +1224,11 @@ void setup_device(pkasp_problem *p, cudaStream_t s) {
         setup_build(p, s);
     } catch (...) {
         cudaStreamSynchronize(s);
+        free_setup(p);  // nothing half-built stays: calls that need a setup are refused
         setup_pool_trim(p, kKeepSetup);
         throw;
     }
+    p->have_setup = true;
     setup_pool_trim(p, kKeepSetup);
 }
 
@@ -1322,7 +1325,6 @@ void setup_build(pkasp_problem *p, cudaStream_t s) {
     PK_CUDA(cudaMemsetAsync(p->d_bar, 0, sizeof(unsigned) * 2, s));
     PK_CUDA(cudaMemsetAsync(p->d_bar_err, 0, sizeof(int), s));
     PK_CUDA(cudaStreamSynchronize(s));
-    p->have_setup = true;
     choose_layouts(p, s);
 }
 

@@ -11,6 +11,7 @@ void fail(int code, const std::string &msg) { throw Error{code, msg}; }
 
 void cuda_check(cudaError_t e, const char *what, const char *file, int line) {
     if (e == cudaSuccess) return;
+    cudaGetLastError();  // reported here; the next launch's check must not find it again
     char buf[512];
     snprintf(buf, sizeof(buf), "%s failed at %s:%d: %s", what, file, line, cudaGetErrorString(e));
     int code = (e == cudaErrorMemoryAllocation) ? PKASP_ENOMEM : PKASP_ECUDA;

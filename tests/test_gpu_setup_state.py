@@ -1,5 +1,5 @@
 """What a problem holds before, between and after its setups: memory that is no longer in use
-goes back."""
+goes back, and a setup that fails leaves none."""
 import pytest
 
 from paper_1204_2586_gb300 import _lib as L
@@ -54,4 +54,43 @@ def test_smaller_setup_gives_memory_back(torch_cuda):
     held = _free(torch)
     P.setup(smoother=1, precond_precision=1, spmv_threads=4, level_smoother=1)
     assert _free(torch) - held >= 28 * P.info.nnz_h - 128 * MB
+    P.close()
+
+
+def test_setup_out_of_memory_leaves_no_setup(torch_cuda):
+    """A second setup with more and more device memory left to it, from almost none to almost
+    enough, so that it fails at every stage, the layouts of the last one included. Every
+    failure is reported, and no call that needs a setup runs on what is left of either."""
+    torch = torch_cuda
+    P = _problem(4, 18)
+    b = P.rhs()
+    y = P.spmv(b)
+    small = dict(smoother=1, spmv_threads=4, level_smoother=1)
+    big = dict(mode=1, precond_precision=1, level_smoother=1)
+    P.setup(**big)
+    x = P.solve(b)[0]
+    held = _free(torch)
+    P.setup(**small)
+    need = _free(torch) - held  # what the larger setup takes on top
+    assert need > 100 * MB
+    failed = 0
+    for part in range(24):
+        P.setup(**small)
+        ballast = torch.empty(_free(torch) - 16 * MB - part * need // 20, dtype=torch.uint8, device="cuda")
+        try:
+            P.setup(**big)
+        except L.PkaspError as e:
+            failed += 1
+            assert e.code in (L.PKASP_ENOMEM, L.PKASP_ECUDA)
+            for call in (P.solve, P.apply_prec, P.apply_smoother, P.stokes_setup):
+                with pytest.raises(L.PkaspError) as e:
+                    call() if call == P.stokes_setup else call(b)
+                assert e.value.code == L.PKASP_ESTATE
+            assert P.info.levels == 0
+            assert torch.equal(P.spmv(b), y)  # A_h is the problem's, not the setup's
+        del ballast
+        torch.cuda.empty_cache()
+    assert 8 <= failed < 24
+    P.setup(**big)
+    assert torch.equal(P.solve(b)[0], x)
     P.close()
