@@ -374,6 +374,7 @@ int pkasp_destroy(pkasp_problem *p) {
     pk::free_setup(p);
     pk::stokes_free(p);
     p->work_pool.free_all();
+    p->hist_pool.free_all();
     p->stage_pool.free_all();
     p->pool.free_all();
     pk::l2_window_release(p);

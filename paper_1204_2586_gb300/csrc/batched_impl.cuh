@@ -1028,7 +1028,7 @@ struct Batched {
     static void init(pkasp_problem *p, const double *B, double *X, cudaStream_t s) {
         kb_init_residual<NC><<<kRedGrid, kBlock, 0, s>>>(p->nh, p->Ah.ptr, p->Ah.col, p->Ah.val, B, X, p->bw_r,
                                                          r32_out(p), p->d_state, p->d_partials, p->d_counter,
-                                                         p->d_hist);
+                                                         p->bw_hist);
         PK_LAUNCH();
         prec(p, p->bw_r, p->bw_z, s);
         kb_start<NC><<<kRedGrid, FlatBT<NC>, 0, s>>>(p->nh * NC, p->bw_r, p->bw_z, p->bw_p, p->d_state,
@@ -1039,7 +1039,7 @@ struct Batched {
     static void iteration(pkasp_problem *p, double *X, cudaStream_t s) {
         spmm_pq(p, s);
         kb_update_xr<NC><<<kRedGrid, FlatBT<NC>, 0, s>>>(p->nh * NC, X, p->bw_r, r32_out(p), p->bw_p, p->bw_q,
-                                                         p->d_state, p->d_partials, p->d_counter, p->d_hist);
+                                                         p->d_state, p->d_partials, p->d_counter, p->bw_hist);
         PK_LAUNCH();
         prec(p, p->bw_r, p->bw_z, s);
         const int flex = (p->opt.flexible || p->opt.precond_precision == PKASP_PREC_FP32) ? 1 : 0;
@@ -1114,8 +1114,6 @@ int solve_nc(pkasp_problem *p, const double *b, double *x, int ncols, int64_t ld
     PK_LAUNCH();
     kb_gather<<<eg, kBlock, 0, s>>>(n, ncols, ld, NC, x, p->bw_x);
     PK_LAUNCH();
-    double *saved_hist = p->d_hist;
-    p->d_hist = p->bw_hist;
     kb_state_reset<<<1, PKASP_MAX_COLS, 0, s>>>(p->d_state, NC, ncols, p->opt.tol, p->opt.max_iter, hist_rows);
     PK_LAUNCH();
     cudaEvent_t e0, e1;
@@ -1175,7 +1173,6 @@ int solve_nc(pkasp_problem *p, const double *b, double *x, int ncols, int64_t ld
     cudaEventDestroy(e1);
     kb_scatter<<<eg, kBlock, 0, s>>>(n, ncols, ld, NC, p->bw_x, x);
     PK_LAUNCH();
-    p->d_hist = saved_hist;
     int rc = PKASP_OK;
     for (int c = 0; c < ncols; ++c) {
         int stc = hs.status[c] < 0 ? PKASP_ENOTCONV : hs.status[c];

@@ -120,10 +120,7 @@ struct Gmres {
         PK_LAUNCH();
     }
     static void build_graph(pkasp_problem *p, const double *b, double *x) {
-        if (p->gm_graph_exec) cudaGraphExecDestroy(p->gm_graph_exec);
-        if (p->gm_graph) cudaGraphDestroy(p->gm_graph);
-        p->gm_graph_exec = nullptr;
-        p->gm_graph = nullptr;
+        free_gmres_graph(p);
         cudaStream_t cs = p->cap_stream;
         cudaGraph_t g, gi;
         PK_CUDA(cudaGraphCreate(&g, 0));
@@ -180,11 +177,15 @@ void ensure_gmres(pkasp_problem *p, int m) {
 
 }  // namespace
 
-void free_gmres(pkasp_problem *p) {
+void free_gmres_graph(pkasp_problem *p) {
     if (p->gm_graph_exec) cudaGraphExecDestroy(p->gm_graph_exec);
     if (p->gm_graph) cudaGraphDestroy(p->gm_graph);
     p->gm_graph_exec = nullptr;
     p->gm_graph = nullptr;
+}
+
+void free_gmres(pkasp_problem *p) {
+    free_gmres_graph(p);
     p->gm_pool.free_all();
     p->gm_V = p->gm_Z = p->gm_w = p->gm_vin = p->gm_zout = nullptr;
     p->gm_state = nullptr;
@@ -196,14 +197,7 @@ int solve_gmres(pkasp_problem *p, const double *b, double *x, pkasp_stats *st, c
     ensure_work(p, 1);
     ensure_gmres(p, m);
     const int cap = (st && st->hist_cap > 0) ? st->hist_cap : 1;
-    if (cap > p->hist_cap) {
-        p->d_hist = p->work_pool.get<double>(cap);
-        p->hist_cap = cap;
-        if (p->gm_graph_exec) cudaGraphExecDestroy(p->gm_graph_exec);
-        if (p->gm_graph) cudaGraphDestroy(p->gm_graph);
-        p->gm_graph_exec = nullptr;
-        p->gm_graph = nullptr;
-    }
+    ensure_hist(p, cap);
     kg_state_reset<<<1, 32, 0, s>>>(p->gm_state, m, p->opt.tol, p->opt.max_iter, p->hist_cap);
     PK_LAUNCH();
     cudaEvent_t e0, e1;

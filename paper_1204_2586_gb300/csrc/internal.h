@@ -247,9 +247,9 @@ struct pkasp_problem {
     double *d_partials = nullptr;
     unsigned int *d_counter = nullptr;
     pk::PcgState *d_state = nullptr;
-    double *d_hist = nullptr;
+    double *d_hist = nullptr;  // [hist_cap] in hist_pool (ensure_hist)
     int hist_cap = 0;
-    pk::DevPool work_pool;
+    pk::DevPool work_pool, hist_pool;
     // graph cache
     cudaGraphExec_t graph_exec = nullptr;
     cudaGraph_t graph = nullptr;
@@ -337,6 +337,7 @@ void pmis_device(int64_t n, const int64_t *ptr, const int32_t *col, const uint8_
 void pmis_noalloc(int64_t n, const int64_t *ptr, const int32_t *col, const uint8_t *strong, uint64_t stream_id,
                   int8_t *cf, cudaStream_t s);
 void ensure_work(pkasp_problem *p, int ncols);
+void ensure_hist(pkasp_problem *p, int cap);
 void check_barrier(pkasp_problem *p, cudaStream_t s);
 // PCG on several right-hand sides (batched.cu); b and x device arrays [n_h][ld]
 int solve_batched(pkasp_problem *p, const double *b, double *x, int ncols, int64_t ld, pkasp_stats *st,
@@ -346,6 +347,7 @@ float time_batched(pkasp_problem *p, int which, int reps, cudaStream_t s);
 // FGMRES(m) outer iteration (gmres.cu); b and x device vectors [n_h]
 int solve_gmres(pkasp_problem *p, const double *b, double *x, pkasp_stats *st, cudaStream_t s);
 void free_gmres(pkasp_problem *p);
+void free_gmres_graph(pkasp_problem *p);
 // Stokes (stokes.cpp: patterns of B = -div_h, B^T and the pressure mass matrix, and
 // their host values for the host-only entry point; stokes.cu: device assembly of the
 // values, operator, block preconditioner, FGMRES)

@@ -1047,15 +1047,21 @@ void l2_window_release(pkasp_problem *p) {
 // ---------------------------------------------------------------------------------
 // setup orchestration
 // ---------------------------------------------------------------------------------
+namespace {
+void free_graph(pkasp_problem *p) {
+    if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
+    if (p->graph) cudaGraphDestroy(p->graph);
+    p->graph_exec = nullptr;
+    p->graph = nullptr;
+}
+}  // namespace
+
 void free_setup(pkasp_problem *p) {
     cudaDeviceSynchronize();  // stream-ordered frees below: nothing may still read the blocks
     free_batched(p);
     free_gmres(p);
     stokes_free(p);  // its solver captured the preconditioner being replaced
-    if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
-    if (p->graph) cudaGraphDestroy(p->graph);
-    p->graph_exec = nullptr;
-    p->graph = nullptr;
+    free_graph(p);
     p->setup_pool.free_all();
     p->lev.clear();
     p->fine = DSplit{};
@@ -1316,6 +1322,9 @@ void setup_build(pkasp_problem *p, cudaStream_t s) {
     if (!p->ev_fork) PK_CUDA(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
     if (!p->ev_join) PK_CUDA(cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming));
     ensure_work(p, 1);
+    // the work vectors outlive a setup; the arrival counts of the reductions start from zero
+    // with each all the same, whatever an aborted run left in them
+    PK_CUDA(cudaMemsetAsync(p->d_counter, 0, sizeof(unsigned) * 4, s));
     // colour offsets on the device and the grid-barrier state of the persistent smoother
     p->d_fine_off = pool.get<int64_t>(p->fine.off.size());
     PK_CUDA(cudaMemcpyAsync(p->d_fine_off, p->fine.off.data(), sizeof(int64_t) * p->fine.off.size(),
@@ -1349,13 +1358,21 @@ void ensure_work(pkasp_problem *p, int ncols) {
     p->d_counter = w.get<unsigned>(4);
     PK_CUDA(cudaMemset(p->d_counter, 0, sizeof(unsigned) * 4));
     p->d_state = w.get<PcgState>(1);
+    p->work_cols = ncols;
+    free_graph(p);
+}
+
+// The residual history of single-column solves, one block that grows: the graphs hold its
+// address, so they go when it moves.
+void ensure_hist(pkasp_problem *p, int cap) {
+    if (cap <= p->hist_cap) return;
+    free_graph(p);
+    free_gmres_graph(p);
+    p->hist_pool.free_all();
     p->hist_cap = 0;
     p->d_hist = nullptr;
-    p->work_cols = ncols;
-    if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
-    if (p->graph) cudaGraphDestroy(p->graph);
-    p->graph_exec = nullptr;
-    p->graph = nullptr;
+    p->d_hist = p->hist_pool.get<double>(cap);
+    p->hist_cap = cap;
 }
 
 // ---------------------------------------------------------------------------------
@@ -1508,10 +1525,7 @@ void enqueue_final(pkasp_problem *p, const double *b, const double *x, cudaStrea
 }
 
 void build_graph(pkasp_problem *p, const double *b, double *x) {
-    if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
-    if (p->graph) cudaGraphDestroy(p->graph);
-    p->graph_exec = nullptr;
-    p->graph = nullptr;
+    free_graph(p);
     cudaStream_t cs = p->cap_stream;
     cudaGraph_t g, gi, gf;
     PK_CUDA(cudaGraphCreate(&g, 0));
@@ -1561,14 +1575,7 @@ int solve_device(pkasp_problem *p, const double *b, double *x, int ncols, int64_
     if (ncols != 1 || ld != 1) return solve_batched(p, b, x, ncols, ld, st, s);
     ensure_work(p, 1);
     const int cap = (st && st->hist_cap > 0) ? st->hist_cap : 1;
-    if (cap > p->hist_cap) {
-        p->d_hist = p->work_pool.get<double>(cap);
-        p->hist_cap = cap;
-        if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
-        if (p->graph) cudaGraphDestroy(p->graph);
-        p->graph_exec = nullptr;
-        p->graph = nullptr;
-    }
+    ensure_hist(p, cap);
     cudaEvent_t e0, e1;
     PK_CUDA(cudaEventCreate(&e0));
     PK_CUDA(cudaEventCreate(&e1));

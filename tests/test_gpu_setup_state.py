@@ -94,3 +94,48 @@ def test_setup_out_of_memory_leaves_no_setup(torch_cuda):
     P.setup(**big)
     assert torch.equal(P.solve(b)[0], x)
     P.close()
+
+
+@pytest.mark.parametrize("krylov", [0, 1])
+def test_history_is_one_block(torch_cuda, krylov):
+    """Solves that ask for longer and longer histories: 40 of 0.8 to 32 MB, 656 MB in all, of which
+    the longest is held, and what they return does not change."""
+    torch = torch_cuda
+    P = _problem(2, 6)
+    b = P.rhs()
+    P.setup(krylov=krylov)
+    first = P.solve(b, hist_cap=64)[1]["hist"]
+    free = _free(torch)
+    for i in range(1, 41):
+        assert (P.solve(b, hist_cap=100_000 * i)[1]["hist"] == first).all()
+    assert free - _free(torch) <= 64 * MB
+    P.close()
+
+
+def test_failed_block_solve_keeps_the_history(torch_cuda):
+    """A blocked solve that ends in an error half-way (here: a capture of its stream, which it
+    cannot run under) leaves the single-column solves as they were, also past the blocks' end."""
+    import ctypes as C
+
+    torch = torch_cuda
+    rt = C.CDLL(next(l.split()[-1] for l in open("/proc/self/maps") if "libcudart" in l))
+    P = _problem(2, 6)
+    b = P.rhs()
+    B = torch.stack([b, 2 * b, 3 * b], dim=1).contiguous()
+    P.setup()
+    x, st = P.solve(b, hist_cap=64)
+    X = P.solve(B)[0]
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    assert rt.cudaStreamBeginCapture(C.c_void_p(s.cuda_stream), 2) == 0  # relaxed: this stream alone
+    with pytest.raises(L.PkaspError):
+        P.solve(B, torch.zeros_like(B), stream=s)
+    g = C.c_void_p()
+    rt.cudaStreamEndCapture(C.c_void_p(s.cuda_stream), C.byref(g))
+    rt.cudaGetLastError()
+    assert torch.equal(P.solve(B)[0], X)
+    P.set_kappa(kappa_lognormal(P.nt, 1))  # the blocks' memory goes
+    P.setup()
+    x2, st2 = P.solve(b, hist_cap=64)
+    assert torch.equal(x2, x) and (st2["hist"] == st["hist"]).all()
+    P.close()
