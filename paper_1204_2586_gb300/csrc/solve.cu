@@ -553,7 +553,14 @@ void precondition(pkasp_problem *p, const double *r, double *z, cudaStream_t s, 
             to_pt<float>(r, p->w_rr32, p->nh, s);
             k_dense_mv<float, float, double><<<g, 128, 0, s>>>(p->nh, p->d_dense32, p->w_rr32, z);
         } else {
-            k_dense_mv<double, double, double><<<g, 128, 0, s>>>(p->nh, p->d_dense, r, z);
+            // every entry of z takes all of r, so z may not be written over r as it may in the
+            // other forms, which write z last
+            const double *in = r;
+            if (r < z + p->nh && z < r + p->nh) {
+                PK_CUDA(cudaMemcpyAsync(p->w_rr, r, sizeof(double) * p->nh, cudaMemcpyDeviceToDevice, s));
+                in = p->w_rr;
+            }
+            k_dense_mv<double, double, double><<<g, 128, 0, s>>>(p->nh, p->d_dense, in, z);
         }
         PK_LAUNCH();
         return;

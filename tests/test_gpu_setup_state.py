@@ -139,3 +139,24 @@ def test_failed_block_solve_keeps_the_history(torch_cuda):
     x2, st2 = P.solve(b, hist_cap=64)
     assert torch.equal(x2, x) and (st2["hist"] == st["hist"]).all()
     P.close()
+
+
+@pytest.mark.parametrize("k,n,prec,mode", [(2, 8, 0, 0), (2, 8, 1, 0), (2, 4, 0, 0), (2, 9, 0, 0), (2, 8, 0, 1), (2, 6, 0, 2)])
+def test_preconditioner_in_place(torch_cuda, k, n, prec, mode):
+    """z = B r with z on r, or overlapping it: the result of separate vectors, bit for bit,
+    whether B is one dense product, sweeps or a cycle."""
+    torch = torch_cuda
+    P = _problem(k, n)
+    P.setup(precond_precision=prec, mode=mode)
+    g = torch.Generator("cuda").manual_seed(n)
+    r = torch.randn(P.nh, dtype=torch.float64, device="cuda", generator=g)
+    z = P.apply_prec(r)
+    s = torch.cuda.current_stream().cuda_stream
+    for shift in (0, 1, P.nh // 2, P.nh - 1):
+        for first in (0, shift):  # r above z, and z above r
+            buf = torch.zeros(P.nh + shift, dtype=torch.float64, device="cuda")
+            rv, zv = buf[first:first + P.nh], buf[shift - first:shift - first + P.nh]
+            rv.copy_(r)
+            L.check(L.load().pkasp_apply_prec(P.h, rv.data_ptr(), zv.data_ptr(), s))
+            assert torch.equal(zv, z)
+    P.close()
