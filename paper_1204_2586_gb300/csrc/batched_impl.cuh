@@ -619,11 +619,7 @@ __global__ void __launch_bounds__(kBlock) kb_dense(int64_t n, const PT *__restri
     const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x % W, g = (threadIdx.x & 31) / W;
     if (row >= n) return;  // a whole warp
-    PT acc[U][CPL];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int k = 0; k < CPL; ++k) acc[u][k] = PT(0);
+    DenseSum<PT> acc[U][CPL];
     const PT *m = M + row * n;
 #pragma unroll 2
     for (int64_t j0 = g; j0 < n; j0 += U * E) {
@@ -633,17 +629,17 @@ __global__ void __launch_bounds__(kBlock) kb_dense(int64_t n, const PT *__restri
             if (j >= n) break;
             const PT a = ldg(&m[j]);
 #pragma unroll
-            for (int k = 0; k < CPL; ++k) acc[u][k] += a * B[j * NC + lane + k * W];
+            for (int k = 0; k < CPL; ++k) acc[u][k].add(a, B[j * NC + lane + k * W]);
         }
     }
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
-        PT t = acc[0][k];
+        DenseSum<PT> t = acc[0][k];
 #pragma unroll
-        for (int u = 1; u < U; ++u) t += acc[u][k];
+        for (int u = 1; u < U; ++u) t.merge(acc[u][k]);
 #pragma unroll
-        for (int o = W; o < 32; o <<= 1) t += __shfl_xor_sync(kFull, t, o);
-        if (g == 0) X[row * NC + lane + k * W] = t;
+        for (int o = W; o < 32; o <<= 1) t.merge(t.shfl_xor(o));
+        if (g == 0) X[row * NC + lane + k * W] = t.template value<PT>();
     }
 }
 

@@ -200,3 +200,52 @@ def test_colouring_in_one_block_and_in_rounds(oracle_mod, n):
     c, nc = G.colours(-1)
     assert np.array_equal(c, O.fine_colour()) and nc == c.max() + 1
     assert np.array_equal(G.colours(0)[0], O.level(0)["colour"])
+
+
+@pytest.mark.parametrize("k,n,level_smoother", [(2, 8, 0), (1, 16, 1), (2, 5, 0), (1, 9, 0), (3, 5, 1)])
+def test_dense_preconditioner_fp32_is_as_exact_as_sweeps(k, n, level_smoother):
+    """Each against FP64 on the same vectors: the one product of thousands of terms is no
+    further off than the sweeps whose place it takes."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, k, kappa_lognormal(t.shape[0], 1))
+    g = torch.Generator("cuda").manual_seed(n)
+    rs = [torch.randn(P.nh, dtype=torch.float64, device="cuda", generator=g) for _ in range(4)]
+    err = []
+    for layout in (4, 0):
+        z = []
+        for prec in (0, 1):
+            P.setup(smoother_layout=layout, precond_precision=prec, level_smoother=level_smoother)
+            z.append([P.apply_prec(r) for r in rs])
+        err.append(sum(((a - b).norm() / b.norm()).item() for a, b in zip(z[1], z[0])))
+    assert err[1] <= err[0]
+    P.close()
+
+
+@pytest.mark.parametrize("n", [7, 9, 12, 16])
+def test_dense_tail_fp32_rounds_three_times(n):
+    """A cycle that is one dense product (P1 meshes: the tail begins on the finest level) rounds
+    its matrix, its input and its result to FP32: each an independent relative error, uniform
+    within half a unit of the last place, 2^-24 / sqrt(3) / 1.5 in the mean square over a binade
+    (2.3e-8). For entries of random sign the three add up to 4e-8; the bound allows 1.5 times that
+    and nothing for the sums."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, 1, kappa_lognormal(t.shape[0], 1))
+    g = torch.Generator("cuda").manual_seed(n)
+    bs = [torch.randn(P.nH, dtype=torch.float64, device="cuda", generator=g) for _ in range(4)]
+    x = []
+    for prec in (0, 1):
+        P.setup(precond_precision=prec)
+        x.append([P.apply_vcycle(b) for b in bs])
+    e = max(((a - c).norm() / c.norm()).item() for a, c in zip(x[1], x[0]))
+    assert e <= 1.5 * 3 ** 0.5 * 2.3e-8
+    P.close()
