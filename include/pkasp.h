@@ -153,6 +153,14 @@ typedef struct {
     int64_t l2_persist_bytes; /* bytes of the fine smoother's vector kept in the L2
                                persisting set-aside after setup (options.l2_persist);
                                0: none */
+    int tail_level;         /* AMG level from which the V-cycle of one right-hand side is one
+                               dense product (levels - 1: the coarsest inverse alone); 0
+                               before setup */
+    int dense_prec;         /* 1: the whole additive preconditioner of one right-hand side is
+                               one dense product (a small problem with the default layouts)
+                               and a solve runs no sweep; 0: sweeps and a cycle */
+    int block_tail_level;   /* tail_level of the multi-RHS blocks of the last solve with
+                               ncols > 1; 0 before one */
 } pkasp_info;
 
 /* Per-solve statistics, filled by pkasp_solve (which synchronises the stream). */

@@ -44,7 +44,8 @@ class pkasp_info(C.Structure):
                 ("setup_ms", C.c_double), ("assemble_ms", C.c_double),
                 ("spmv_layout", C.c_int), ("smoother_layout", C.c_int),
                 ("block_width", C.c_int), ("block_group", C.c_int), ("block_lanes", C.c_int),
-                ("l2_persist_bytes", C.c_int64)]
+                ("l2_persist_bytes", C.c_int64), ("tail_level", C.c_int), ("dense_prec", C.c_int),
+                ("block_tail_level", C.c_int)]
 
 
 class pkasp_stats(C.Structure):

@@ -212,6 +212,9 @@ int pkasp_problem_info(const pkasp_problem *p, pkasp_info *info) {
         info->block_group = p->bgroup_cols;
         info->block_lanes = p->blanes;
         info->l2_persist_bytes = (int64_t)p->l2_win_bytes;
+        info->tail_level = p->tail;
+        info->dense_prec = p->d_dense || p->d_dense32;
+        info->block_tail_level = p->bwork_nc > 0 ? p->btail : 0;
     }
     return PKASP_OK;
 }

@@ -74,6 +74,7 @@ void ensure_batched(pkasp_problem *p, int NC, int hist_entries) {
     }
     p->bw_hist = w.get<double>(std::max(hist_entries, 1));
     p->bw_mask = w.get<int>(PKASP_MAX_COLS);
+    p->btail = block_tail_level(p, NC);
     p->bwork_nc = NC;
     p->bwork_hist = hist_entries;
 }

@@ -612,31 +612,42 @@ __global__ void kb_add_div(int64_t n, const PT *R, const PT *__restrict__ d, PT 
 }
 
 // X = M B for the dense tail of the V-cycle (tail.cu): one warp per row, 32 / W groups of
-// lanes share its entries, each with four partial sums per column
+// lanes share its entries. A group's entries are a chain of loads, so a step loads U of them
+// before it adds the first (198 rows: 48 columns FP32 28 us a row task of W lanes with plain
+// sums, 16 so; 64 columns FP32 15.7 and 22, 32 columns FP64 25 and 26 to 29).
 template <int NC, typename PT>
 __global__ void __launch_bounds__(kBlock) kb_dense(int64_t n, const PT *__restrict__ M, const PT *B, PT *X) {
-    constexpr int W = Tile<NC>::W, CPL = Tile<NC>::CPL, E = 32 / W, U = CPL > 1 ? 2 : 4;
+    constexpr int W = Tile<NC>::W, CPL = Tile<NC>::CPL, E = 32 / W, U = 8, S = 4;
     const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x % W, g = (threadIdx.x & 31) / W;
     if (row >= n) return;  // a whole warp
-    DenseSum<PT> acc[U][CPL];
+    DenseSum<PT> acc[S][CPL];
     const PT *m = M + row * n;
-#pragma unroll 2
-    for (int64_t j0 = g; j0 < n; j0 += U * E) {
+    int64_t j = g;
+    for (; j + (U - 1) * E < n; j += U * E) {
+        PT a[U], v[U][CPL];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t j = j0 + u * E;
-            if (j >= n) break;
-            const PT a = ldg(&m[j]);
+            a[u] = ldg(&m[j + u * E]);
 #pragma unroll
-            for (int k = 0; k < CPL; ++k) acc[u][k].add(a, B[j * NC + lane + k * W]);
+            for (int k = 0; k < CPL; ++k) v[u][k] = B[(j + u * E) * NC + lane + k * W];
         }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) acc[u % S][k].add(a[u], v[u][k]);
+    }
+#pragma unroll 4
+    for (; j < n; j += E) {
+        const PT a = ldg(&m[j]);
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) acc[0][k].add(a, B[j * NC + lane + k * W]);
     }
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
         DenseSum<PT> t = acc[0][k];
 #pragma unroll
-        for (int u = 1; u < U; ++u) t.merge(acc[u][k]);
+        for (int u = 1; u < S; ++u) t.merge(acc[u][k]);
 #pragma unroll
         for (int o = W; o < 32; o <<= 1) t.merge(t.shfl_xor(o));
         if (g == 0) X[row * NC + lane + k * W] = t.template value<PT>();
@@ -686,6 +697,7 @@ __global__ void __launch_bounds__(kBlock) kb_gs_full(int64_t pb, int64_t pe, con
     const int64_t p = pb + ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (W * E);
     const int lane = threadIdx.x % W, g = threadIdx.x % (W * E) / W;
     const bool ok = p < pe;
+    if (E == 1 && !ok) return;  // no shuffles then
     const int32_t i = ok ? perm[p] : 0;
     PT sl[CPL], su[CPL];
     bdote<W, E, CPL, PT>(ok ? lptr[p] : 0, ok ? lptr[p + 1] : 0, lcol, lval, (const PT *)X, NC, lane, g, sl);
@@ -809,12 +821,9 @@ struct Batched {
         PT *x = bpickw<PT>(p->bl_x[l], p->bl_x32[l]);
         PT *r = bpickw<PT>(p->bl_r[l], p->bl_r32[l]);
         const bool jac = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
-        // the dense tail takes NC times the FMAs of one column; with l1-Jacobi levels, whose
-        // few launches it replaces, only while those stay below 10^7
-        const bool tail = l == p->tail && (!jac || (double)n * n * NC <= 1e7);
-        if (tail || l == (int)p->lev.size() - 1) {
+        if (l == p->btail) {
             kb_dense<NC, PT><<<tasks_grid(n, 32), kBlock, 0, s>>>(
-                n, tail ? bpick<PT>(p->d_tail, p->d_tail32) : bpick<PT>(p->d_cinv, p->d_cinv32), b, x);
+                n, l == p->tail ? bpick<PT>(p->d_tail, p->d_tail32) : bpick<PT>(p->d_cinv, p->d_cinv32), b, x);
             PK_LAUNCH();
             return;
         }

@@ -257,6 +257,7 @@ struct pkasp_problem {
     // several right-hand sides: blocks [n][NC] (batched.cu), sized for one width NC
     pk::DevPool bwork_pool;
     int bwork_nc = -1, bwork_hist = 0;
+    int btail = 0;  // level from which the cycle of a block is one dense product (tail.cu)
     int bchunk = 0;  // 1 + the autotuned layout of the blocked fine smoother (0: not tuned yet)
     int bgroup_cols = 0, blanes = 0;  // that layout: columns per group, lanes per row
     double *bw_r = nullptr, *bw_z = nullptr, *bw_p = nullptr, *bw_q = nullptr, *bw_b = nullptr,
@@ -381,6 +382,7 @@ void build_slices(DevPool &pool, const DCSR &A, const DSplit &sp, int part, int 
 
 // the dense tail of the V-cycle (tail.cu); after the hierarchy and the coarsest inverse
 void build_tail(pkasp_problem *p, cudaStream_t s);
+int block_tail_level(const pkasp_problem *p, int NC);
 
 // SELL-32 builder (sell.cu)
 void build_sell_split(DevPool &pool, const DSplit &sp, int64_t n, bool upper, DSell &S, bool want32,

@@ -5,9 +5,10 @@
 // up) and the solve multiplies by that n x n matrix, as it always did with the coarsest
 // inverse: one launch that reads n^2 entries. The matrix is formed in FP64.
 //
-// One column block of a level is 256 threads wide; a thread carries one column through the
+// One column block of a level is kCols threads wide; a thread carries one column through the
 // row sums, so reads of the dense operand are coalesced and the matrix entry is a broadcast.
 #include <algorithm>
+#include <cmath>
 
 #include "internal.h"
 
@@ -122,8 +123,8 @@ double dense_us(double n, bool fp32) { return 2.5 + n * n / (fp32 ? 1.2e6 : 0.55
 }  // namespace
 
 // Level at which the cycle becomes one dense product: the highest where that is modelled
-// faster than the launches below it, within 5120 rows and 10^10 FMAs of setup work (about
-// 15 ms).
+// faster than the launches below it, within 5120 rows and n nnz <= 4 10^9 (the FMAs of one of the
+// level's own passes over the identity; the coarse product adds n_c^2 n of them).
 int tail_level(const pkasp_problem *p) {
     const bool jacobi = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
     const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
@@ -141,6 +142,55 @@ int tail_level(const pkasp_problem *p) {
         }
     }
     return best;
+}
+
+// The same for the cycle of a block of NC columns, which takes the dense matrix of p->tail or,
+// where that takes longer, the launches down to the coarsest inverse. In the additive form both
+// run beside the fine sweeps (S): launches wait most of their time and hide behind them, the
+// product wants the FP64 pipe and the L1 as they do and adds to them. So the times (us) compared
+// are  max(S, D) + share min(S, D)  for the product and  max(S, L)  for the launches; with no
+// sweep beside them D and L. w is NC / 64, `row` a level's mean row in units of 50 entries:
+//   D  chain n W / 32 for a group's entries one after another, or the n^2 NC FMAs (a warp a row,
+//      so whole rounds of eight rows on each of 152 SMs) at `rate` a us
+//   L  Gauss-Seidel: level + a phase a colour and sweep of c0 + c1 w + row (c2 + c3 w);
+//      l1-Jacobi: level + row (c2 + c3 w); and the product of the coarsest level
+// Fitted to graph solves with and without the product, P1 7^3 to 42^3, P2 9^3 to 32^3, P3 9^3
+// to 21^3, P4 8^3 to 16^3, constant and lognormal coefficients, widths 4 to 64, as is the estimate
+// of S. Of 864 pairs 14 come out more than 3% above the faster side, four more than 3% above the
+// launches (by 10% at most). Taking the product always had made wide blocks up to twice as slow:
+// an iteration of P2 17^3, 64 columns, FP64, Gauss-Seidel levels 1724 us as launches and 3321 with
+// 4096 rows dense; with l1-Jacobi levels and n^2 NC <= 10^7, P1 9^3, 32 columns 162 and 210.
+struct BlockCycle {
+    double chain, rate, share, level, c0, c1, c2, c3;
+};
+constexpr BlockCycle kBlockCycle[2][2] = {  // [FP32][l1-Jacobi]
+    {{0.20, 0.30e6, 0.95, 60, 1.1, 5.4, 8, 3}, {0.54, 0.41e6, 0.36, 71, 0, 0, 76, 14}},
+    {{0.025, 1.5e6, 0.45, 170, 0.64, 0, 3.7, 0}, {0.13, 0.52e6, 0.86, 55, 0, 0, 26, 4.1}}};
+
+int block_tail_level(const pkasp_problem *p, int NC) {
+    const bool jacobi = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
+    const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
+    const BlockCycle &c = kBlockCycle[fp32][jacobi];
+    const int last = (int)p->lev.size() - 1, W = NC % 32 == 0 ? 32 : NC % 16 == 0 ? 16 : NC % 8 == 0 ? 8 : 4;
+    const double w = NC / 64.0;
+    auto product = [&](int l) {
+        const double n = (double)p->lev[l].A.n;
+        return 3.0 + std::max(c.chain * n * W / 32, std::ceil(n / 1216) * 1216 * n * NC / c.rate);
+    };
+    double launches = product(last);
+    for (int l = p->tail; l < last; ++l) {
+        const Level &L = p->lev[l];
+        const double row = (double)L.A.nnz / (double)L.A.n / 50, each = c.c0 + c.c1 * w + row * (c.c2 + c.c3 * w);
+        launches += c.level + (jacobi ? 1 : 2 * L.sp.ncol) * each;
+    }
+    double sweeps = 0;
+    if (p->opt.mode == PKASP_MODE_ADDITIVE && p->opt.smoother == PKASP_SMOOTHER_SGS) {
+        const double row = (double)p->Ah.nnz / (double)p->nh / 50, ph = 2.0 * p->fine.ncol, m = 1e-6 * (double)p->Ah.nnz;
+        sweeps = fp32 ? ph * (1.5 + row * (1.5 + 3.2 * w)) + m * (0.42 * NC + 9.7)
+                      : ph * (1.3 + row * (2.4 + 6.1 * w)) + m * (2.4 * NC + 17.0);
+    }
+    const double d = product(p->tail);
+    return std::max(sweeps, d) + c.share * std::min(sweeps, d) < std::max(sweeps, launches) ? p->tail : last;
 }
 
 // Whether the whole additive preconditioner B = S_k + I_P V I_P^T of a small problem is

@@ -249,3 +249,30 @@ def test_dense_tail_fp32_rounds_three_times(n):
     e = max(((a - c).norm() / c.norm()).item() for a, c in zip(x[1], x[0]))
     assert e <= 1.5 * 3 ** 0.5 * 2.3e-8
     P.close()
+
+
+# blocks on both sides of the line between one dense product and the launches of the levels:
+# by width, by rows, by level smoother and precision
+@pytest.mark.parametrize("n,ncols,prec,level_smoother,dense", [(17, 3, 0, 0, True), (17, 64, 0, 0, False), (17, 64, 1, 0, False),
+                                                               (26, 64, 0, 0, True), (9, 32, 0, 1, False), (11, 3, 0, 1, True),
+                                                               (22, 16, 1, 1, False)])
+def test_block_cycle_with_and_without_dense_tail(n, ncols, prec, level_smoother, dense):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, 1, kappa_lognormal(t.shape[0], 1))
+    P.setup(precond_precision=prec, level_smoother=level_smoother)
+    b = torch.randn(P.nh, ncols, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    x, st = P.solve(b)
+    i = P.info
+    assert i.tail_level < i.levels - 1
+    assert i.block_tail_level == (i.tail_level if dense else i.levels - 1)
+    assert max(st["true_rel"]) <= 1e-8
+    for c in (0, ncols - 1):
+        xc, sc = P.solve(b[:, c].contiguous())
+        assert abs(sc["iters"][0] - st["iters"][c]) <= 1
+        assert (x[:, c] - xc).norm() <= 1e-8 * xc.norm()
+    P.close()
