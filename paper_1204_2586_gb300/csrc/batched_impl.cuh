@@ -194,9 +194,12 @@ __global__ void __launch_bounds__(kBlock) kb_init_residual(int64_t n, const int6
 }
 
 // Q = A P and alpha_c = rho_c / (p_c, q_c) for the columns still running; E entry groups
-// share a row (W * E = 32 lanes, or E = 1): with fewer rows than two passes of the grid the
-// longest row's chain is the kernel's time (P3 9^3, 5 columns: 76 -> 59 us; P4 6^3, 3 columns:
-// 115 -> 53)
+// share a row (W * E = 32 lanes, or E = 1): with few rows a lane the longest row's chain is the
+// kernel's time. us without -> with, by entries a row (rows times W):
+//   46 (P3) and 72 (P4)  P3 9^3, 8 columns (141,000) 74 -> 58, 13^3, 3 (219,000) 85 -> 76; P4 8^3, 8
+//                        (238,000) 125 -> 86; P4 12^3, 3 (415,000) 158 -> 172
+//   27 (P2)              13^3, 8 (125,000) 54 -> 50; 17^3, 3 (144,000) 54 -> 58; 13^3, 48 (250,000) 84 -> 86
+//   14 (P1)              17^3, 8 (33,000) 41 -> 39; 18^3, 16 (79,000) 41 -> 43; 42^3, 3 (276,000) 46 -> 68
 template <int NC, int E>
 __global__ void __launch_bounds__(kBlock) kb_spmv_pq(int64_t n, const int64_t *__restrict__ ptr,
                                                      const int32_t *__restrict__ col, const double *__restrict__ val,
@@ -933,8 +936,14 @@ struct Batched {
         PK_LAUNCH();
     }
 
+    // whole warps per row in the SpMM: the longer a row, the more rows per lane it takes before
+    // its chain hides (kb_spmv_pq)
+    static bool split_spmm(const pkasp_problem *p) {
+        const double row = (double)p->Ah.nnz / (double)p->nh;
+        return p->nh * W <= (row < 20 ? 40000 : row < 40 ? 140000 : 2 * (int64_t)kRedGrid * kBlock);
+    }
     static void spmm_pq(pkasp_problem *p, cudaStream_t s) {
-        auto kern = p->nh * W <= 2 * (int64_t)kRedGrid * kBlock ? kb_spmv_pq<NC, 32 / W> : kb_spmv_pq<NC, 1>;
+        auto kern = split_spmm(p) ? kb_spmv_pq<NC, 32 / W> : kb_spmv_pq<NC, 1>;
         kern<<<kRedGrid, kBlock, 0, s>>>(p->nh, p->Ah.ptr, p->Ah.col, p->Ah.val, p->bw_p, p->bw_q, p->d_state,
                                          p->d_partials, p->d_counter);
         PK_LAUNCH();

@@ -276,3 +276,25 @@ def test_block_cycle_with_and_without_dense_tail(n, ncols, prec, level_smoother,
         assert abs(sc["iters"][0] - st["iters"][c]) <= 1
         assert (x[:, c] - xc).norm() <= 1e-8 * xc.norm()
     P.close()
+
+
+# both sides of the line from which a row of the blocked product is a whole warp's, for rows of
+# 14 and 27 entries (P3 and P4: test_block_widths and the block tests against the oracle)
+@pytest.mark.parametrize("k,n,ncols", [(1, 17, 8), (1, 18, 16), (2, 13, 8), (2, 17, 3)])
+def test_block_product_of_short_rows(k, n, ncols):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, k, kappa_lognormal(t.shape[0], 1))
+    P.setup(level_smoother=1)
+    b = torch.randn(P.nh, ncols, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    x, st = P.solve(b)
+    assert max(st["true_rel"]) <= 1e-8
+    for c in (0, ncols - 1):
+        xc, sc = P.solve(b[:, c].contiguous())
+        assert abs(sc["iters"][0] - st["iters"][c]) <= 1
+        assert (x[:, c] - xc).norm() <= 1e-8 * xc.norm()
+    P.close()
