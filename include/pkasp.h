@@ -149,7 +149,8 @@ typedef struct {
                                or 64) of the last solve with ncols > 1; 0 before one */
     int block_group;        /* columns per group of the multi-RHS fine smoother phases,
                                autotuned at the first solve of a width (0 before) */
-    int block_lanes;        /* threads per row of those phases (autotuned with it) */
+    int block_lanes;        /* threads per row of those phases (32 where small phases take a
+                               warp per row, else autotuned with the group) */
     int64_t l2_persist_bytes; /* bytes of the fine smoother's vector kept in the L2
                                persisting set-aside after setup (options.l2_persist);
                                0: none */

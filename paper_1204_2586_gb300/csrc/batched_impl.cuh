@@ -951,8 +951,9 @@ struct Batched {
 
     // the autotuner of the fine smoother's layout (column group width, lanes per row):
     // times one symmetric sweep per candidate. Results are the same bits for every
-    // layout: each column's sums run over the same entries in the same order. Returns
-    // 1 + the index of the fastest layout.
+    // candidate: each column's sums run over the same entries in the same order (in whole
+    // warps, which small phases take without a choice, in another one). Returns 1 + the index
+    // of the fastest layout.
     static int tune_group(pkasp_problem *p, cudaStream_t s) {
         if (p->opt.smoother == PKASP_SMOOTHER_L1JACOBI || split_rows(p->fine)) return 1;
         int best = 0;
@@ -1120,7 +1121,9 @@ int solve_nc(pkasp_problem *p, const double *b, double *x, int ncols, int64_t ld
     if (p->bchunk == 0) {
         p->bchunk = Batched<NC>::tune_group(p, s);
         p->bgroup_cols = Batched<NC>::layout_ch(p->bchunk - 1);
-        p->blanes = Batched<NC>::layout_w(p->bchunk - 1);
+        // rows taken by whole warps: 32 / W groups of the block's W lanes (gs_sym)
+        const bool whole = p->opt.smoother == PKASP_SMOOTHER_SGS && Batched<NC>::split_rows(p->fine);
+        p->blanes = whole ? 32 : Batched<NC>::layout_w(p->bchunk - 1);
     }
     const int64_t n = p->nh, ne = n * NC;
     const unsigned eg = (unsigned)((ne + kBlock - 1) / kBlock);

@@ -298,3 +298,19 @@ def test_block_product_of_short_rows(k, n, ncols):
         assert abs(sc["iters"][0] - st["iters"][c]) <= 1
         assert (x[:, c] - xc).norm() <= 1e-8 * xc.norm()
     P.close()
+
+
+@pytest.mark.parametrize("n,ncols,lanes", [(6, 3, {32}), (6, 8, {32}), (6, 16, {32}), (32, 3, {2, 4}), (32, 8, {4, 8})])
+def test_block_lanes_are_those_that_run(n, ncols, lanes):
+    """P3: phases of 200 rows take a warp per row, phases of 34,000 the block's own lanes."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, 3)
+    P.setup(level_smoother=1, max_iter=2)
+    P.solve(torch.ones(P.nh, ncols, dtype=torch.float64, device="cuda"), raise_on_fail=False)
+    assert P.info.block_lanes in lanes
+    P.close()
