@@ -615,30 +615,63 @@ __global__ void kb_add_div(int64_t n, const PT *R, const PT *__restrict__ d, PT 
 }
 
 // X = M B for the dense tail of the V-cycle (tail.cu): one warp per row, 32 / W groups of
-// lanes share its entries. A group's entries are a chain of loads, so a step loads U of them
-// before it adds the first (198 rows: 48 columns FP32 28 us a row task of W lanes with plain
-// sums, 16 so; 64 columns FP32 15.7 and 22, 32 columns FP64 25 and 26 to 29).
-template <int NC, typename PT>
+// lanes share its entries.
+// AHEAD: a step loads eight entries before it adds the first (198 rows, 48 columns FP32: 28 us a
+// row task of W lanes, 12 so; 64 columns 15.7 and 22; 32 columns FP64 25 and 26). Without: four,
+// tested one by one. Alone that is no faster, but FP64 products of one column a lane that fill the
+// chip leave the sweeps beside them more of the FP64 pipe: the preconditioner of P2 17^3, 3
+// columns, 219 us against 282 (48 and 64 columns the other way: P2 24^3, 64, 4273 against 3400).
+// FP32 carries the rounding errors of its sums along as the single-column product does
+// (DenseSum), but every four terms: with one FMA a loaded value the 11 instructions a term would be
+// the kernel's time (4096 rows, 48 columns: an iteration 581 us, 380 so), and chains of four are no
+// further off than the launches (host count of the roundings, 1728 rows: 6.0e-8 against 8e-8;
+// 1.1e-7 with plain sums, 4.4e-8 with every term carried).
+template <int NC, typename PT, bool AHEAD>
 __global__ void __launch_bounds__(kBlock) kb_dense(int64_t n, const PT *__restrict__ M, const PT *B, PT *X) {
-    constexpr int W = Tile<NC>::W, CPL = Tile<NC>::CPL, E = 32 / W, U = 8, S = 4;
+    constexpr bool kF32 = std::is_same<PT, float>::value;
+    constexpr int W = Tile<NC>::W, CPL = Tile<NC>::CPL, E = 32 / W, U = AHEAD ? 8 : 4, S = kF32 ? 2 : 4;
     const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x % W, g = (threadIdx.x & 31) / W;
     if (row >= n) return;  // a whole warp
     DenseSum<PT> acc[S][CPL];
     const PT *m = M + row * n;
     int64_t j = g;
-    for (; j + (U - 1) * E < n; j += U * E) {
-        PT a[U], v[U][CPL];
+    if constexpr (AHEAD) {
+        for (; j + (U - 1) * E < n; j += U * E) {
+            PT a[U], v[U][CPL];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            a[u] = ldg(&m[j + u * E]);
+            for (int u = 0; u < U; ++u) {
+                a[u] = ldg(&m[j + u * E]);
 #pragma unroll
-            for (int k = 0; k < CPL; ++k) v[u][k] = B[(j + u * E) * NC + lane + k * W];
+                for (int k = 0; k < CPL; ++k) v[u][k] = B[(j + u * E) * NC + lane + k * W];
+            }
+#pragma unroll
+            for (int h = 0; h < U; h += 4)
+#pragma unroll
+                for (int k = 0; k < CPL; ++k) {
+                    if constexpr (kF32) {
+                        float t = a[h] * v[h][k];
+#pragma unroll
+                        for (int u = h + 1; u < h + 4; ++u) t = fmaf(a[u], v[u][k], t);
+                        acc[h / 4][k].two_sum(t, 0.0f);
+                    } else {
+#pragma unroll
+                        for (int u = h; u < h + 4; ++u) acc[u % S][k].add(a[u], v[u][k]);
+                    }
+                }
         }
+    } else {
+        static_assert(!kF32, "FP32 sums run in the other form");
+#pragma unroll 2
+        for (; j < n; j += U * E) {
 #pragma unroll
-        for (int u = 0; u < U; ++u)
+            for (int u = 0; u < U; ++u) {
+                if (j + u * E >= n) break;
+                const PT a = ldg(&m[j + u * E]);
 #pragma unroll
-            for (int k = 0; k < CPL; ++k) acc[u % S][k].add(a[u], v[u][k]);
+                for (int k = 0; k < CPL; ++k) acc[u][k].add(a, B[(j + u * E) * NC + lane + k * W]);
+            }
+        }
     }
 #pragma unroll 4
     for (; j < n; j += E) {
@@ -825,7 +858,11 @@ struct Batched {
         PT *r = bpickw<PT>(p->bl_r[l], p->bl_r32[l]);
         const bool jac = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
         if (l == p->btail) {
-            kb_dense<NC, PT><<<tasks_grid(n, 32), kBlock, 0, s>>>(
+            // below 1216 rows, one block of eight on each SM, the product leaves the pipe to others
+            auto kern = kb_dense<NC, PT, true>;
+            if constexpr (std::is_same<PT, double>::value && Tile<NC>::CPL == 1)
+                if (n > 1216) kern = kb_dense<NC, PT, false>;
+            kern<<<tasks_grid(n, 32), kBlock, 0, s>>>(
                 n, l == p->tail ? bpick<PT>(p->d_tail, p->d_tail32) : bpick<PT>(p->d_cinv, p->d_cinv32), b, x);
             PK_LAUNCH();
             return;

@@ -156,16 +156,17 @@ int tail_level(const pkasp_problem *p) {
 //      l1-Jacobi: level + row (c2 + c3 w); and the product of the coarsest level
 // Fitted to graph solves with and without the product, P1 7^3 to 42^3, P2 9^3 to 32^3, P3 9^3
 // to 21^3, P4 8^3 to 16^3, constant and lognormal coefficients, widths 4 to 64, as is the estimate
-// of S. Of 864 pairs 14 come out more than 3% above the faster side, four more than 3% above the
-// launches (by 10% at most). Taking the product always had made wide blocks up to twice as slow:
+// of S: the constants stand for the choice they make, not for a kernel alone. Of 864 pairs ten
+// come out more than 3% above the faster side (13% at most), none more than 2% above the launches.
+// Taking the product always had made wide blocks up to twice as slow:
 // an iteration of P2 17^3, 64 columns, FP64, Gauss-Seidel levels 1724 us as launches and 3321 with
 // 4096 rows dense; with l1-Jacobi levels and n^2 NC <= 10^7, P1 9^3, 32 columns 162 and 210.
 struct BlockCycle {
     double chain, rate, share, level, c0, c1, c2, c3;
 };
 constexpr BlockCycle kBlockCycle[2][2] = {  // [FP32][l1-Jacobi]
-    {{0.20, 0.30e6, 0.95, 60, 1.1, 5.4, 8, 3}, {0.54, 0.41e6, 0.36, 71, 0, 0, 76, 14}},
-    {{0.025, 1.5e6, 0.45, 170, 0.64, 0, 3.7, 0}, {0.13, 0.52e6, 0.86, 55, 0, 0, 26, 4.1}}};
+    {{0.078, 0.33e6, 1.1, 30, 3.3, 7.1, 2.3, 9.4}, {0.87, 0.67e6, 0.62, 24, 0, 0, 160, 19}},
+    {{0.018, 1.3e6, 0.45, 410, 0.73, 0, 6.8, 0}, {0.17, 0.90e6, 0.076, 33, 0, 0, 55, 0.54}}};
 
 int block_tail_level(const pkasp_problem *p, int NC) {
     const bool jacobi = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;

@@ -253,9 +253,10 @@ def test_dense_tail_fp32_rounds_three_times(n):
 
 # blocks on both sides of the line between one dense product and the launches of the levels:
 # by width, by rows, by level smoother and precision
-@pytest.mark.parametrize("n,ncols,prec,level_smoother,dense", [(17, 3, 0, 0, True), (17, 64, 0, 0, False), (17, 64, 1, 0, False),
+@pytest.mark.parametrize("n,ncols,prec,level_smoother,dense", [(17, 3, 0, 0, True), (17, 64, 0, 0, False), (17, 64, 1, 0, True),
                                                                (26, 64, 0, 0, True), (9, 32, 0, 1, False), (11, 3, 0, 1, True),
-                                                               (22, 16, 1, 1, False)])
+                                                               (22, 16, 1, 1, True),
+                                                               (13, 32, 1, 1, False), (17, 32, 1, 1, False)])
 def test_block_cycle_with_and_without_dense_tail(n, ncols, prec, level_smoother, dense):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
