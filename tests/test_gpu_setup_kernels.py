@@ -315,3 +315,83 @@ def test_block_lanes_are_those_that_run(n, ncols, lanes):
     P.solve(torch.ones(P.nh, ncols, dtype=torch.float64, device="cuda"), raise_on_fail=False)
     assert P.info.block_lanes in lanes
     P.close()
+
+
+def _phase_entries(P):
+    i = P.info
+    return (i.nnz_h - i.n_h) / 2 / i.fine_colours
+
+
+# phases that let the next one launch after their own wait (FP64, 80,000 to 750,000 entries a
+# phase, both forms of the preconditioner), and FP32 slices of 4 lanes, steps and batches
+@pytest.mark.parametrize("k,n,prec,mode,lo,hi,lanes", [(2, 28, 0, 0, 80e3, 750e3, 2), (3, 18, 0, 0, 80e3, 750e3, 2),
+                                                       (4, 14, 0, 0, 80e3, 750e3, 2), (2, 26, 0, 1, 80e3, 375e3, 2),
+                                                       (3, 17, 0, 1, 80e3, 375e3, 2), (2, 28, 1, 0, 110e3, 2e6, 4),
+                                                       (3, 32, 1, 0, 5e5, 2e6, 4)])
+def test_late_and_middling_slices_match_rows(k, n, prec, mode, lo, hi, lanes):
+    """As test_slices_match_rows, at the sizes of these two forms."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, k, kappa_lognormal(t.shape[0], 1))
+    r = torch.randn(P.nh, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    out = []
+    for layout in (4, 0):
+        P.setup(smoother_layout=layout, precond_precision=prec, mode=mode, level_smoother=1)
+        assert P.info.smoother_layout == (500 + lanes if layout == 0 else layout)
+        out.append(P.apply_prec(r) if mode else P.apply_smoother(r))
+    assert lo <= _phase_entries(P) < hi
+    longest = 400 if k == 4 else 200
+    u = 2.0 ** -24 if prec else 2.0 ** -53
+    assert (out[1] - out[0]).norm() <= 2 * P.info.fine_colours * longest * u * out[0].norm()
+    P.close()
+
+
+def test_stokes_components_share_late_sweeps():
+    """As test_stokes_components_share_sweeps, with phases of the late form."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(26, 0.2, 0)
+    P = Problem(xyz, t, 2)
+    out = []
+    for layout in (4, 0):
+        P.setup(smoother_layout=layout, level_smoother=1)
+        P.stokes_setup()
+        r = torch.randn(P.stokes_n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+        out.append(P.stokes_prec(r)[: 3 * P.nh])
+    assert 80e3 <= _phase_entries(P) < 750e3
+    assert (out[1] - out[0]).norm() <= _sweep_bound(P, 0) * out[0].norm()
+    P.close()
+
+
+# problems on both sides of the line from which the whole additive preconditioner is one dense
+# product: 3375 unknowns of P2 are, of P4 (too many entries) are not; 2744, 64; 4913, 4096 not
+@pytest.mark.parametrize("k,n,prec,kw,dense", [(2, 8, 0, {}, 1), (2, 8, 1, {}, 1), (3, 5, 1, {}, 1), (1, 5, 0, {}, 1),
+                                               (4, 3, 0, {}, 1), (4, 4, 0, {}, 0), (2, 9, 0, {}, 0), (1, 17, 1, {}, 0),
+                                               (2, 8, 0, dict(smoother_layout=4), 0), (2, 8, 0, dict(spmv_threads=8), 0),
+                                               (2, 8, 0, dict(mode=1), 0), (2, 8, 0, dict(smoother=1), 0)])
+def test_dense_preconditioner_runs_where_it_should(k, n, prec, kw, dense):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1204_2586_gb300 import Problem
+
+    xyz, t = kuhn_mesh(n, 0.2, 0)
+    P = Problem(xyz, t, k)
+    P.setup(precond_precision=prec, **kw)
+    assert P.info.dense_prec == dense
+    P.close()
+
+
+@pytest.mark.parametrize("n,level_smoother,tail", [(17, 0, 0), (19, 0, 1), (22, 1, 2), (32, 0, 2)])
+def test_cycle_with_dense_tail_at_each_level(oracle_mod, n, level_smoother, tail):
+    torch, G, O = _pair(oracle_mod, 1, n, level_smoother=level_smoother)
+    assert G.info.tail_level == tail < G.info.levels - 1
+    b = np.random.default_rng(n).standard_normal(G.nH)
+    _close(G.apply_vcycle(torch.tensor(b, device="cuda")).cpu().numpy(), O.vcycle(b), 1e-11)
