@@ -110,11 +110,21 @@ CONFIG_BATCHED = {
 # per clock per SM (2 FP64 FMA per clock per SM) = 1.259 TFLOP/s (nominal 1.25)
 FP64_PEAK_TFLOPS = 152 * 2.070e9 * 4 / 1e12
 ORACLE_SAMPLE_ITERS = 12
-# ncu dram__bytes_read.sum + dram__bytes_write.sum per launch (summed over the phases of
-# one S_k application), keyed by (workload, cubes per side, smoother layout); a kernel
-# changed since the capture has no entry (traffic null)
+# ncu dram__bytes_read.sum + dram__bytes_write.sum of one S_k application (its launches summed)
+# and of one SpMV launch, with the profile that holds them, keyed by (workload, cubes per side,
+# layout): a kernel that was not captured in the layout that runs has no entry. S_k has none: its
+# L2 window does not act under ncu.
 SMOOTHER_TRAFFIC = {}
-SPMV_TRAFFIC = {("p4_n48_lognormal", 48): (6843905536 + 82143744 + 6831242496 + 91436544 + 6832146176 + 91604224) / 3}
+SPMV_TRAFFIC = {("p4_n48_lognormal", 48, "interleaved slices, 1 lanes per ordinary row"):
+                ((19444004864 + 264799232) / 3, "ncu dram__bytes_read+write per launch (mean of 3), profiles/k_slices_p4_n48.md")}
+
+
+def measured_traffic(table, layout):
+    """The line's traffic and traffic_note for the layout code that runs (null: not captured)."""
+    got, note = table.get((WORKLOAD["name"], WORKLOAD["n"], smoother_layout_name(layout)), (None, None))
+    return {"traffic": got, "traffic_note": note}
+
+
 NOMINAL_HBM_GBS = 8000.0  # GB300's nominal HBM3e bandwidth, for the second fraction
 # AMG level smoother: l1-Jacobi (1), one kernel per smoothing step; multicolour GS on the
 # dense coarse levels needs one launch per colour and costs ~25x more per V-cycle here
@@ -525,9 +535,6 @@ def main():
     # nonzero + 20 B per row.
     spmv_ms = G.time_kernel(0, 50)
     smoother_ms = G.time_kernel(1, 20)
-    # the same loads without the colour dependencies (all rows at once): the memory work
-    # of one S_k application with no barrier between its phases
-    nodep_ms = G.time_kernel(7, 20)
     # the GPU's random 8-byte gather rate from a vector of n_h values (pkasp_time_kernel
     # mode 8 returns nanoseconds per gather): the colour phases gather one value per
     # off-diagonal entry, and their L2 sector traffic, not DRAM bytes, binds them
@@ -544,20 +551,15 @@ def main():
     s_tf = smoother_flops / (smoother_ms / 1e3) / 1e12
     roof = {"bound": "hbm", "kernel": "k_slice_phase (colour phases of the fine SGS S_k, FP64)",
             "achieved": s_ach, "peak": peak, "unit": "GB/s", "frac": s_ach / peak,
-            "traffic": SMOOTHER_TRAFFIC.get((WORKLOAD["name"], WORKLOAD["n"], smoother_layout_name(
-                info64.smoother_layout))),
-            "traffic_note": "ncu dram__bytes_read+write summed over the 81 launches of one application, "
-                            "profiles/k_gs_phase_p4_n48.md",
+            **measured_traffic(SMOOTHER_TRAFFIC, info64.smoother_layout),
             "frac_of_nominal_8000": s_ach / NOMINAL_HBM_GBS,
             "peak_source": src, "bytes_per_application": smoother_bytes, "ms_per_application": smoother_ms,
             "phases_per_application": 2 * int(info64.fine_colours) - 1,
-            "dependency_free_pass_ms": nodep_ms,
             "gather_roof": {"achieved_Ggathers_per_s": (nnz - nh) / (smoother_ms / 1e3) / 1e9,
                             "peak_Ggathers_per_s": 1.0 / gather_ns,
                             "frac": (nnz - nh) / (smoother_ms / 1e3) / 1e9 * gather_ns,
                             "peak_source": "measured live: random 8-byte gathers from an n_h vector "
                                            "(pkasp_time_kernel mode 8)"},
-            "dependency_free_pass_frac": (smoother_bytes / (nodep_ms / 1e3) / 1e9) / peak,
             "fp64_pipe": {"achieved_tflops": s_tf, "peak_tflops": FP64_PEAK_TFLOPS,
                           "frac": s_tf / FP64_PEAK_TFLOPS, "flops_per_application": smoother_flops,
                           "peak_source": "derived: 152 SMs x 2.07 GHz x 4 FP64 flop/clk/SM"}}
@@ -565,8 +567,7 @@ def main():
     roof_spmv = {"bound": "hbm", "kernel": "k_spmv_q / k_spmv_y (fine SpMV, interleaved slices, FP64)",
                  "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                  "frac_of_nominal_8000": achieved / NOMINAL_HBM_GBS,
-                 "traffic": SPMV_TRAFFIC.get((WORKLOAD["name"], WORKLOAD["n"])),
-                 "traffic_note": "ncu dram__bytes_read+write per launch (mean of 3), profiles/k_spmv_q_p4_n48.md",
+                 **measured_traffic(SPMV_TRAFFIC, info64.spmv_layout),
                  "peak_source": src, "bytes_per_launch": spmv_bytes, "ms_per_launch": spmv_ms}
 
     def leg(**kw):

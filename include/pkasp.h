@@ -440,9 +440,11 @@ int pkasp_reference_tensors(int k, double *S_out);
  * multi-RHS blocks of the last solve with ncols > 1 (ESTATE before one): 4 blocked SpMM
  * Q = A_h P with its per-column dot (P, Q), 5 blocked fine smoother, 6 blocked
  * preconditioner. The blocked timings overwrite the solve's work blocks and scalars.
- * which = 7: the fine smoother's loads without its colour dependencies (every row of the
- * colour split at once, lower parts then upper parts, the smoother's lanes per row):
- * the memory work of one S_k application with no barrier between colour phases.
+ * which = 7: the loads of one S_k application without its colour dependencies, in the row
+ * layout (every row of the colour split at once, lower parts then upper parts, 4 lanes per
+ * row, or the smoother's 8 or 16 with such a smoother_layout): what that layout's phases
+ * cost without a barrier between them. The default layout reads fewer lines and is faster
+ * with its barriers.
  * which = 8: a gather-rate probe, random 8-byte gathers from an n_h vector driven by a
  * streamed index array of min(64M, 8 n_h) entries (scratch allocated for the call);
  * *ms_out then receives NANOSECONDS PER GATHER, the inverse of the GPU's random gather
