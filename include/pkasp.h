@@ -207,7 +207,7 @@ int pkasp_last_error(char *buf, size_t n);
  *              pkasp_nodes_host gives n_all and the node coordinates before assembly).
  *              f is taken as its nodal interpolant f_h = sum_n f_n phi_n, so the load is
  *              b = M f_nodal exactly up to rounding (M the P_k mass matrix; the rule is
- *              exact for f_h phi_i). The library keeps a copy (pkasp_set_kappa reuses it).
+ *              exact for f_h phi_i). The library keeps a copy.
  * Dirichlet nodes (those on faces with one adjacent element) are removed (Eq. 1,
  * u = 0 on the boundary). The node numbering is: vertices, then edges sorted by vertex
  * pair (nodes from the lower vertex), then faces sorted by vertex triple (nodes in
@@ -235,16 +235,18 @@ int pkasp_get_dofmap(const pkasp_problem *p, int64_t *dof_all_host, double *dof_
 int pkasp_get_rhs(const pkasp_problem *p, double *b, pkasp_stream_t stream);
 
 /* Replaces the coefficient kappa of Eq. (1) [nt] (host or device, > 0) and re-assembles
- * A_h, A_H (Eq. 7) and f_h on the same sparsity pattern, with the source given to
- * pkasp_assemble. Invalidates the setup (call pkasp_setup again). Synchronises. */
+ * A_h and A_H (Eq. 7) on the same sparsity pattern; f_h, which does not depend on kappa,
+ * stays. Discards the setup (call pkasp_setup again): its memory goes back to the device but
+ * for at most 1 GB, kept for the setup that follows. Synchronises. */
 int pkasp_set_kappa(pkasp_problem *p, const double *kappa, pkasp_stream_t stream);
 
 /* Builds the preconditioner on the device: Jones-Plassmann colouring of A_h, strength
  * graph (Sec. 6.2), PMIS C/F splitting, extended+i interpolation, Galerkin RAP per level
  * (the relation A_H = I_R A_h I_P of Sec. 2 applied recursively), colourings of every
  * level, the coarsest inverse, and FP32 copies when requested. Synchronises the stream.
- * Errors: EINVAL (options), ENOMEM (coarsest level above 8192 rows), EBREAKDOWN
- * (coarsest matrix not positive definite), ECUDA. */
+ * Errors: EINVAL (options; the previous setup stays), ENOMEM (device memory, coarsest level
+ * above 8192 rows), EBREAKDOWN (coarsest matrix not positive definite), ECUDA: after these
+ * three the problem has no setup and what was built is freed. */
 int pkasp_setup(pkasp_problem *p, const pkasp_options *opt, pkasp_stream_t stream);
 
 /* ------------------------------------------------------------------------------------
@@ -298,7 +300,8 @@ int pkasp_spmv(const pkasp_problem *p, const double *x_dev, double *y_dev, pkasp
 
 /* z = B r with the preconditioner of the last pkasp_setup: additive B = S_k + Pi B_1
  * Pi^T (Sec. 2), multiplicative (Algorithm 2.1 with Remark 2.1) or plain AMG on A_h
- * (Sec. 6.2), in FP64 or FP32 arithmetic. Enqueued on stream; ESTATE before setup. */
+ * (Sec. 6.2), in FP64 or FP32 arithmetic. z may overlap r. Enqueued on stream; ESTATE before
+ * setup. */
 int pkasp_apply_prec(pkasp_problem *p, const double *r_dev, double *z_dev, pkasp_stream_t stream);
 
 /* z = S_k r from a zero guess: the P_k smoother of Sec. 2 alone (one forward and one

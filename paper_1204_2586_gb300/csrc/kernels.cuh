@@ -682,7 +682,8 @@ __global__ void __launch_bounds__(kBlock) k_prolong_inplace(int64_t n, const int
 // has up to 5120 terms where a colour phase's has tens, so plain FP32 sums are further off than
 // the sweeps they replace. Against FP64, B r at P2 8^3: 6.5e-8 as sweeps, 1.2e-7 with plain sums,
 // 3.4e-8 so; the V-cycle at P3 16^3: 8.6e-8, 1.3e-7, 4.6e-8. The FP32 pipe has room for it beside
-// the loads: P2 8^3's product takes 12 us instead of 10, its solve 0.855 ms instead of 0.830.
+// the loads: P2 8^3's product takes 12 us instead of 10, its solve 0.86 ms instead of 0.825. (Errors
+// carried every two products leave P1 9^3, 512 rows, 7% further off than its sweeps.)
 template <typename T>
 struct DenseSum {
     T s = T(0);
@@ -721,9 +722,9 @@ struct DenseSum<float> {
     __device__ __forceinline__ TX value() const { return (TX)s + (TX)c; }
 };
 
-// x = M b for the dense tail of the V-cycle or a small problem's whole preconditioner (one warp per row; small blocks, so that a few
-// hundred rows spread over the chip). Bound by reading M: eight loads in flight per lane
-// and four partial sums.
+// x = M b for the dense tail of the V-cycle or a small problem's whole preconditioner (one warp
+// per row; small blocks, so that a few hundred rows spread over the chip). Bound by reading M:
+// eight loads in flight per lane and four partial sums.
 template <typename PT, typename TB, typename TX>
 __global__ void __launch_bounds__(128) k_dense_mv(int64_t n, const PT *__restrict__ M, const TB *__restrict__ b,
                                                   TX *__restrict__ x) {

@@ -124,7 +124,8 @@ double dense_us(double n, bool fp32) { return 2.5 + n * n / (fp32 ? 1.2e6 : 0.55
 
 // Level at which the cycle becomes one dense product: the highest where that is modelled
 // faster than the launches below it, within 5120 rows and n nnz <= 4 10^9 (the FMAs of one of the
-// level's own passes over the identity; the coarse product adds n_c^2 n of them).
+// level's own passes over the identity; the coarse product adds n_c^2 n of them: a setup of P1 17^3,
+// 4096 rows over 1241, takes 19 ms).
 int tail_level(const pkasp_problem *p) {
     const bool jacobi = p->opt.level_smoother == PKASP_SMOOTHER_L1JACOBI;
     const bool fp32 = p->opt.precond_precision == PKASP_PREC_FP32;
@@ -195,9 +196,17 @@ int block_tail_level(const pkasp_problem *p, int NC) {
 }
 
 // Whether the whole additive preconditioner B = S_k + I_P V I_P^T of a small problem is
-// applied as one dense product: its sweeps cost 1.5 us a phase (P2 8^3, 3375 unknowns, FP64:
-// B 42 us as launches; FP32 33). Within 3400 rows (92 MB, read from L2) and 6 10^8 FMAs of
-// setup work (about 1 ms). An explicit layout of the smoother keeps its sweeps.
+// applied as one dense product: its sweeps cost 1.5 us a phase, whatever their size. An iteration
+// (us, Gauss-Seidel levels, kappa = 1; product, sweeps):
+//   3375 rows  P2 8^3 FP64 60.6, 70.7, FP32 44.4, 65.5; P1 16^3 62, 76 and 47, 61; P4 4^3 60, 148
+//              and 43, 129
+//   4096 rows  P1 17^3 80, 92 and 49, 63
+//   4913 rows  P2 9^3 94, 75 and 53, 69; P3 6^3 91, 102 and 54, 92
+// The order changes between 3400 and 4900 rows for FP64 and few colours. The bound of 3400 rows is
+// that line (92 MB of matrix in FP64), taken for all degrees and both precisions, and the one of
+// 6 10^8 entries times rows keeps the setup's work at 1 ms: FP32, P3 and P4 would gain beyond them
+// (P4 4^3 has 6.3 10^8; its setup takes 3.5 ms with the product and 1.4 without). An explicit
+// layout of the smoother keeps its sweeps.
 bool dense_prec(const pkasp_problem *p) {
     const pkasp_options &o = p->opt;
     if (o.mode != PKASP_MODE_ADDITIVE || o.smoother != PKASP_SMOOTHER_SGS || o.smoother_layout != 0 ||
